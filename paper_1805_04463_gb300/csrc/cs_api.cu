@@ -176,10 +176,7 @@ int cs_sprinkle(int kind, int64_t n, uint64_t seed, int32_t* coords_dev, void* w
         !aligned(workspace_dev, 256))
         return CS_EINVAL;
     if (workspace_bytes < sprinkle_workspace_bytes(n)) return CS_ENOMEM;
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    cudaError_t e = clear_status(workspace_dev, st);
-    if (e == cudaSuccess) e = launch_sprinkle(kind, n, seed, coords_dev, workspace_dev, st);
-    return from_cuda(e);
+    return from_cuda(launch_sprinkle(kind, n, seed, coords_dev, workspace_dev, static_cast<cudaStream_t>(stream)));
 }
 
 int cs_causal_matrix(int kind, int64_t n, const int32_t* coords_dev, uint64_t* bits_dev, int64_t row_words,

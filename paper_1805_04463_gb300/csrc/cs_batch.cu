@@ -57,8 +57,6 @@ struct BatchSet {
     int64_t tile_begin;    // first column tile of this set in the concatenated tile range
 };
 
-constexpr int kRankThreads = 1024;
-
 __device__ __forceinline__ int find_set_elem(const BatchSet* sets, int nsets, int64_t idx) {
     int lo = 0, hi = nsets - 1;
     while (lo < hi) {
@@ -96,72 +94,6 @@ __global__ void __launch_bounds__(256) k_batch_keys(const BatchSet* __restrict__
     }
 }
 
-// Exact ranks of a set's n keys (ties by index: the order "sorted by time,
-// ties by generation index") in shared memory, O(n): count the keys into P
-// buckets by their top log2(P) bits (P the power of two >= n; the keys are
-// a time coordinate in the top bits, or random, so a bucket holds about
-// one key and at most a few), an exclusive scan of the counts, fill the
-// buckets, then rank each key within its bucket by comparison.  After the
-// fill, cnt[b] is the end of bucket b and cnt[b - 1] its start.  (A bitonic
-// sort of the (key, index) pairs, O(n log^2 n), took 0.38 ms for the
-// 768-set ensemble.)  All kRankThreads threads; rank[e] receives the rank.
-__device__ void rank_keys_smem(const uint64_t* __restrict__ src, int n, int lgP, uint64_t* sk, uint32_t* cnt,
-                               uint32_t* slot, uint32_t* rank) {
-    const int P = 1 << lgP, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int shift = 64 - lgP;
-    for (int i = tid; i < n; i += kRankThreads) sk[i] = src[i];
-    for (int i = tid; i < P; i += kRankThreads) cnt[i] = 0u;
-    __syncthreads();
-    for (int i = tid; i < n; i += kRankThreads) atomicAdd(&cnt[sk[i] >> shift], 1u);
-    __syncthreads();
-    // exclusive scan: each thread a run of P / kRankThreads buckets (P >= 1024
-    // is ensured by the caller), warp and block offsets through shuffles
-    const int per = P / kRankThreads;
-    uint32_t run = 0;
-    for (int k = 0; k < per; ++k) run += cnt[tid * per + k];
-    uint32_t incl = run;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += y;
-    }
-    __shared__ uint32_t wsum[kRankThreads / 32];
-    if (lane == 31) wsum[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-        uint32_t w = lane < kRankThreads / 32 ? wsum[lane] : 0u, wi = w;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, wi, o);
-            if (lane >= o) wi += y;
-        }
-        if (lane < kRankThreads / 32) wsum[lane] = wi - w;  // exclusive warp offsets
-    }
-    __syncthreads();
-    uint32_t at = wsum[warp] + incl - run;
-    for (int k = 0; k < per; ++k) {
-        const uint32_t c = cnt[tid * per + k];
-        cnt[tid * per + k] = at;  // start of the bucket, then its fill cursor
-        at += c;
-    }
-    __syncthreads();
-    for (int i = tid; i < n; i += kRankThreads) slot[atomicAdd(&cnt[sk[i] >> shift], 1u)] = uint32_t(i);
-    __syncthreads();
-    for (int i = tid; i < n; i += kRankThreads) {
-        const uint64_t ke = sk[i];
-        const uint32_t bk = uint32_t(ke >> shift);
-        const uint32_t s0 = bk ? cnt[bk - 1] : 0u, s1 = cnt[bk];
-        uint32_t r = s0;
-        for (uint32_t q = s0; q < s1; ++q) {
-            const uint32_t f = slot[q];
-            const uint64_t kf = sk[f];
-            r += (kf < ke) || (kf == ke && f < uint32_t(i));
-        }
-        rank[i] = r;
-    }
-    __syncthreads();
-}
-
 // One CTA per set: exact rank of each element (ties by index), then the
 // time-sorted coordinates.  Shared memory: keys 8P, bucket cursors 4P,
 // bucket slots 4P, ranks 4P (and the u ranks 4P of a 2D order): 24P bytes.
@@ -177,11 +109,16 @@ __global__ void __launch_bounds__(kRankThreads) k_batch_rank(const BatchSet* __r
     uint32_t* slot = cnt + P;
     uint32_t* rank = slot + P;
     uint32_t* ru = rank + P;
-    rank_keys_smem(b.key0, n, lgP, sk, cnt, slot, rank);
+    auto load = [&](const uint64_t* key) {
+        for (int i = threadIdx.x; i < n; i += kRankThreads) sk[i] = key[i];
+    };
+    load(b.key0);
+    rank_keys_smem(n, lgP, sk, cnt, slot, rank);
     if (b.kind == CS_2D_ORDER) {
         for (int e = threadIdx.x; e < n; e += kRankThreads) ru[e] = rank[e];  // u rank of element e
         __syncthreads();
-        rank_keys_smem(b.key1, n, lgP, sk, cnt, slot, rank);
+        load(b.key1);
+        rank_keys_smem(n, lgP, sk, cnt, slot, rank);
         for (int e = threadIdx.x; e < n; e += kRankThreads) {
             b.coords[ru[e]] = int32_t(ru[e]);
             b.coords[n + ru[e]] = int32_t(rank[e]);

@@ -11,6 +11,7 @@ size_t sprinkle_workspace_bytes(int64_t n);
 // once per device, synchronously, on first use); nullptr on failure, and a
 // failed upload is tried again on the next call.
 const uint64_t* ds_table_device();
+// Clears the workspace's status word first.
 cudaError_t launch_sprinkle(int kind, int64_t n, uint64_t seed, int32_t* coords, void* workspace,
                             cudaStream_t st);
 

@@ -5,10 +5,13 @@
 // Coordinates are drawn independently per element from the counter-based
 // generator, then elements are sorted by time (Section "Pairwise
 // Relations").  The sort is an exact ranking: every element gets
-// rank = #{f : (key_f, f) < (key_e, e)}.  Keys are bucketed on their top 16
-// bits (a counting pass, a scan, a fill), and each element compares itself
-// only with its bucket -- O(n + 65536) work for the hashed / uniform keys used
-// here, and the same ranks for any bucket fill order.
+// rank = #{f : (key_f, f) < (key_e, e)}.  Keys are bucketed on their top 10
+// to 16 bits, about one bucket per element (counted while the keys are drawn,
+// a scan, a fill), and each element compares itself only with its bucket --
+// O(n) work for the hashed / uniform keys used here, and the same ranks for
+// any bucket fill order.  Four launches; the first form, with one launch per
+// step and key stream and a one-block scan, spent 125 us on a set of 16384
+// elements and 240 us on a 2D order of 1024.
 #include <atomic>
 #include <cmath>
 #include <mutex>
@@ -45,139 +48,215 @@ std::vector<uint64_t> ds_thresholds_host() {
     return t;
 }
 
-__global__ void k_keys_ds_slab(int64_t n, uint64_t seed, const uint64_t* __restrict__ thr,
-                               int32_t* __restrict__ raw, uint64_t* __restrict__ key) {
-    const uint64_t s = stream_key(seed, kStreamDeSitter);
-    for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < n; e += int64_t(gridDim.x) * blockDim.x)
-        key[e] = draw_ds_slab(s, e, thr, raw[e], raw[n + e]);
-}
-
-constexpr int kBucketBits = 16;
-constexpr int kBuckets = 1 << kBucketBits;
+constexpr int kMinBucketBits = 10, kMaxBucketBits = 16;
 constexpr int kThreads = 256;
+constexpr int kScanBuckets = 1024;  // buckets per block of the scan
+constexpr int64_t kSmallSet = 2048;  // largest set one CTA sprinkles alone
 
-__global__ void k_keys_2d_order(int64_t n, uint64_t seed, uint64_t* __restrict__ key_u,
-                                uint64_t* __restrict__ key_v) {
-    const uint64_t su = stream_key(seed, kStreamOrderU), sv = stream_key(seed, kStreamOrderV);
-    for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < n; e += int64_t(gridDim.x) * blockDim.x)
-        draw_2d_order(su, sv, e, key_u[e], key_v[e]);
+// About one bucket per element: the ranks stay O(n) and a small set does not
+// scan 65536 buckets.
+int bucket_bits(int64_t n) {
+    int b = kMinBucketBits;
+    while (b < kMaxBucketBits && (int64_t(1) << b) < n) ++b;
+    return b;
 }
 
-__global__ void k_keys_2d_diamond(int64_t n, uint64_t seed, int32_t* __restrict__ raw,
-                                  uint64_t* __restrict__ key) {
-    const uint64_t s = stream_key(seed, kStreamDiamond2);
-    for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < n; e += int64_t(gridDim.x) * blockDim.x)
-        key[e] = draw_2d_diamond(s, e, raw[e], raw[n + e]);
+// Scratch of a sprinkle.  A 2D order ranks two key streams (u and v), side by
+// side in the same launches; the other kinds rank one and keep the drawn
+// coordinates in raw.
+struct SprinkleScratch {
+    uint64_t* key[2];
+    int32_t* raw;        // [dim][n], not for a 2D order
+    uint32_t* arrival[2];  // position of an element within its bucket
+    uint32_t* slot[2];     // bucket by bucket, the elements
+    uint32_t* count[2];    // elements per bucket (zeroed before the keys)
+    uint32_t* start[2];    // first slot of a bucket; start[buckets] = n
+};
+
+// Draw element e of a set: its sort key (two for a 2D order) and, for the
+// other kinds, its coordinates.  false: no rejection attempt was accepted.
+template <int KIND>
+__device__ __forceinline__ bool draw_element(uint64_t seed, int64_t e, const uint64_t* __restrict__ thr,
+                                             int32_t (&c)[4], uint64_t (&key)[2]) {
+    if constexpr (KIND == CS_2D_ORDER)
+        draw_2d_order(stream_key(seed, kStreamOrderU), stream_key(seed, kStreamOrderV), e, key[0], key[1]);
+    else if constexpr (KIND == CS_2D_DIAMOND)
+        key[0] = draw_2d_diamond(stream_key(seed, kStreamDiamond2), e, c[0], c[1]);
+    else if constexpr (KIND == CS_2D_SQUARE)
+        key[0] = draw_2d_square(stream_key(seed, kStreamSquare), e, c[0], c[1]);
+    else if constexpr (KIND == CS_2D_CYLINDER)
+        key[0] = draw_2d_cylinder(stream_key(seed, kStreamCylinder), e, c[0], c[1]);
+    else if constexpr (KIND == CS_2D_DS_SLAB)
+        key[0] = draw_ds_slab(stream_key(seed, kStreamDeSitter), e, thr, c[0], c[1]);
+    else if constexpr (KIND == CS_3D_DIAMOND)
+        return draw_3d_diamond(stream_key(seed, kStreamDiamond3), e, c, key[0]);
+    else
+        return draw_4d_diamond(stream_key(seed, kStreamDiamond4), e, c, key[0]);
+    return true;
 }
 
-__global__ void k_keys_2d_square(int64_t n, uint64_t seed, int32_t* __restrict__ raw, uint64_t* __restrict__ key) {
-    const uint64_t s = stream_key(seed, kStreamSquare);
-    for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < n; e += int64_t(gridDim.x) * blockDim.x)
-        key[e] = draw_2d_square(s, e, raw[e], raw[n + e]);
-}
+constexpr int kind_dim(int kind) { return kind == CS_4D_DIAMOND ? 4 : kind == CS_3D_DIAMOND ? 3 : 2; }
 
-__global__ void k_keys_2d_cylinder(int64_t n, uint64_t seed, int32_t* __restrict__ raw,
-                                   uint64_t* __restrict__ key) {
-    const uint64_t s = stream_key(seed, kStreamCylinder);
-    for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < n; e += int64_t(gridDim.x) * blockDim.x)
-        key[e] = draw_2d_cylinder(s, e, raw[e], raw[n + e]);
-}
-
-template <int D>
-__global__ void k_keys_diamond(int64_t n, uint64_t seed, int32_t* __restrict__ raw, uint64_t* __restrict__ key,
-                               WsHeader* hdr) {
-    const uint64_t s = stream_key(seed, D == 4 ? kStreamDiamond4 : kStreamDiamond3);
+// Keys, raw coordinates and bucket counts in one pass; the count's old value
+// is the element's place in its bucket, so the fill needs no second atomic.
+template <int KIND>
+__global__ void __launch_bounds__(kThreads) k_keys(int64_t n, uint64_t seed, const uint64_t* __restrict__ thr,
+                                                   SprinkleScratch s, int bits, WsHeader* hdr) {
     for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < n; e += int64_t(gridDim.x) * blockDim.x) {
         int32_t c[4];
-        if (!draw_diamond<D>(s, e, c, key[e])) set_status(hdr, CS_ERANGE);
+        uint64_t key[2];
+        if (!draw_element<KIND>(seed, e, thr, c, key)) set_status(hdr, CS_ERANGE);
 #pragma unroll
-        for (int k = 0; k < D; ++k) raw[k * n + e] = c[k];
-    }
-}
-
-__global__ void k_bucket_count(int64_t n, const uint64_t* __restrict__ key, uint32_t* __restrict__ count) {
-    for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < n; e += int64_t(gridDim.x) * blockDim.x)
-        atomicAdd(&count[key[e] >> (64 - kBucketBits)], 1u);
-}
-
-// Exclusive scan of the bucket counts (one block of 1024 threads, 64 buckets
-// each); start[b] = first slot of bucket b, start[kBuckets] = n.  The counts
-// are turned into fill cursors (= start) for k_bucket_fill.
-__global__ void __launch_bounds__(1024) k_bucket_scan(uint32_t* __restrict__ count, uint32_t* __restrict__ start) {
-    constexpr int per = kBuckets / 1024;
-    __shared__ uint32_t part[1024];
-    const int t = threadIdx.x;
-    uint32_t local[per];
-    uint32_t sum = 0;
-#pragma unroll
-    for (int k = 0; k < per; ++k) {
-        local[k] = count[t * per + k];
-        sum += local[k];
-    }
-    part[t] = sum;
-    __syncthreads();
-    for (int off = 1; off < 1024; off <<= 1) {  // Hillis-Steele inclusive scan
-        uint32_t v = t >= off ? part[t - off] : 0;
-        __syncthreads();
-        part[t] += v;
-        __syncthreads();
-    }
-    uint32_t run = part[t] - sum;
-#pragma unroll
-    for (int k = 0; k < per; ++k) {
-        start[t * per + k] = run;
-        count[t * per + k] = run;  // becomes the fill cursor
-        run += local[k];
-    }
-    if (t == 1023) start[kBuckets] = run;
-}
-
-__global__ void k_bucket_fill(int64_t n, const uint64_t* __restrict__ key, uint32_t* __restrict__ cursor,
-                              uint32_t* __restrict__ slot) {
-    for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < n; e += int64_t(gridDim.x) * blockDim.x) {
-        const uint32_t pos = atomicAdd(&cursor[key[e] >> (64 - kBucketBits)], 1u);
-        slot[pos] = uint32_t(e);
-    }
-}
-
-__global__ void k_bucket_rank(int64_t n, const uint64_t* __restrict__ key, const uint32_t* __restrict__ start,
-                              const uint32_t* __restrict__ slot, uint32_t* __restrict__ rank) {
-    for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < n; e += int64_t(gridDim.x) * blockDim.x) {
-        const uint64_t ke = key[e];
-        const uint32_t b = uint32_t(ke >> (64 - kBucketBits));
-        uint32_t r = start[b];
-        for (uint32_t p = start[b]; p < start[b + 1]; ++p) {
-            const uint32_t f = slot[p];
-            const uint64_t kf = key[f];
-            r += (kf < ke) || (kf == ke && f < uint32_t(e));
+        for (int q = 0; q < (KIND == CS_2D_ORDER ? 2 : 1); ++q) {
+            s.key[q][e] = key[q];
+            s.arrival[q][e] = atomicAdd(&s.count[q][key[q] >> (64 - bits)], 1u);
         }
-        rank[e] = r;
+        if constexpr (KIND != CS_2D_ORDER) {
+#pragma unroll
+            for (int k = 0; k < kind_dim(KIND); ++k) s.raw[k * n + e] = c[k];
+        }
     }
 }
 
-__global__ void k_scatter_2d_order(int64_t n, const uint32_t* __restrict__ ru, const uint32_t* __restrict__ rv,
-                                   int32_t* __restrict__ coords) {
+// Exclusive scan of the bucket counts, grid (buckets / 1024, key streams).
+// Each block sums every count before its own 1024 (at most 256 KB, read from
+// L2 in 16-byte words) and scans its own, so the blocks need not wait on one
+// another.  One block that walked all 65536 buckets, each thread its own run
+// of 64, took 103-110 us whatever n was (16-byte sectors of 64 separate
+// lines per thread and store); this takes about 3.
+__global__ void __launch_bounds__(256) k_bucket_scan(SprinkleScratch s, int64_t n) {
+    const uint32_t* count = s.count[blockIdx.y];
+    uint32_t* start = s.start[blockIdx.y];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const uint4* c4 = reinterpret_cast<const uint4*>(count);
+    uint32_t before = 0;
+#pragma unroll 8
+    for (int g = t; g < int(blockIdx.x) * (kScanBuckets / 4); g += 256) {
+        const uint4 v = c4[g];
+        before += v.x + v.y + v.z + v.w;
+    }
+    const uint4 own = c4[blockIdx.x * (kScanBuckets / 4) + t];
+    const uint32_t sum = own.x + own.y + own.z + own.w;
+    uint32_t incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+        before += __shfl_xor_sync(0xffffffffu, before, o);
+    }
+    __shared__ uint32_t wsum[8], wbefore[8];
+    if (lane == 31) wsum[warp] = incl;
+    if (lane == 0) wbefore[warp] = before;
+    __syncthreads();
+    uint32_t at = incl - sum;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) at += wbefore[w] + (w < warp ? wsum[w] : 0u);
+    reinterpret_cast<uint4*>(start)[blockIdx.x * (kScanBuckets / 4) + t] =
+        make_uint4(at, at + own.x, at + own.x + own.y, at + own.x + own.y + own.z);
+    if (t == 255 && blockIdx.x == gridDim.x - 1) start[gridDim.x * kScanBuckets] = uint32_t(n);
+}
+
+__global__ void __launch_bounds__(kThreads) k_bucket_fill(int64_t n, SprinkleScratch s, int bits) {
+    const int q = blockIdx.y;
+    for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < n; e += int64_t(gridDim.x) * blockDim.x)
+        s.slot[q][s.start[q][s.key[q][e] >> (64 - bits)] + s.arrival[q][e]] = uint32_t(e);
+}
+
+// Rank of element e's key, ties by index.
+__device__ __forceinline__ uint32_t rank_of(const uint64_t* __restrict__ key, const uint32_t* __restrict__ start,
+                                            const uint32_t* __restrict__ slot, int bits, int64_t e) {
+    const uint64_t ke = key[e];
+    const uint32_t b = uint32_t(ke >> (64 - bits));
+    const uint32_t begin = start[b], end = start[b + 1];
+    uint32_t r = begin;
+    for (uint32_t p = begin; p < end; ++p) {
+        const uint32_t f = slot[p];
+        const uint64_t kf = key[f];
+        r += (kf < ke) || (kf == ke && f < uint32_t(e));
+    }
+    return r;
+}
+
+// Ranks and, with them, the time-sorted coordinates.
+__global__ void __launch_bounds__(kThreads) k_rank_scatter(int64_t n, int dim, bool order2d, SprinkleScratch s, int bits,
+                                                           int32_t* __restrict__ coords) {
     for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < n; e += int64_t(gridDim.x) * blockDim.x) {
-        const uint32_t r = ru[e];
-        coords[r] = int32_t(r);
-        coords[n + r] = int32_t(rv[e]);
+        const uint32_t r = rank_of(s.key[0], s.start[0], s.slot[0], bits, e);
+        if (order2d) {
+            coords[r] = int32_t(r);
+            coords[n + r] = int32_t(rank_of(s.key[1], s.start[1], s.slot[1], bits, e));
+        } else {
+            for (int c = 0; c < dim; ++c) coords[c * n + r] = s.raw[c * n + e];
+        }
     }
 }
 
-__global__ void k_scatter_raw(int64_t n, int dim, const uint32_t* __restrict__ rank, const int32_t* __restrict__ raw,
-                              int32_t* __restrict__ coords) {
-    for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < n; e += int64_t(gridDim.x) * blockDim.x) {
-        const uint32_t r = rank[e];
-        for (int c = 0; c < dim; ++c) coords[c * n + r] = raw[c * n + e];
+// A whole small set in one CTA: draws, ranks in shared memory, coordinates
+// out; no scratch in the workspace.  Five launches of a handful of blocks
+// are all latency there.
+template <int KIND>
+__global__ void __launch_bounds__(kRankThreads) k_sprinkle_small(int n, int lgP, uint64_t seed,
+                                                                 const uint64_t* __restrict__ thr,
+                                                                 int32_t* __restrict__ coords, WsHeader* hdr) {
+    extern __shared__ uint8_t smem_raw[];
+    constexpr int kPer = int(kSmallSet) / kRankThreads;
+    const int P = 1 << lgP;
+    uint64_t* sk = reinterpret_cast<uint64_t*>(smem_raw);
+    uint32_t* cnt = reinterpret_cast<uint32_t*>(sk + P);
+    uint32_t* slot = cnt + P;
+    uint32_t* rank = slot + P;
+    if (threadIdx.x == 0) hdr->status = 0;
+    __syncthreads();
+    int32_t c[kPer][4];
+    uint64_t key[kPer][2];
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+        const int e = int(threadIdx.x) + q * kRankThreads;
+        if (e >= n) continue;
+        if (!draw_element<KIND>(seed, e, thr, c[q], key[q])) set_status(hdr, CS_ERANGE);
+        sk[e] = key[q][0];
+    }
+    rank_keys_smem(n, lgP, sk, cnt, slot, rank);
+    if constexpr (KIND == CS_2D_ORDER) {
+        uint32_t ru[kPer];
+#pragma unroll
+        for (int q = 0; q < kPer; ++q) {
+            const int e = int(threadIdx.x) + q * kRankThreads;
+            if (e >= n) continue;
+            ru[q] = rank[e];
+            sk[e] = key[q][1];
+        }
+        __syncthreads();
+        rank_keys_smem(n, lgP, sk, cnt, slot, rank);
+#pragma unroll
+        for (int q = 0; q < kPer; ++q) {
+            const int e = int(threadIdx.x) + q * kRankThreads;
+            if (e >= n) continue;
+            coords[ru[q]] = int32_t(ru[q]);
+            coords[n + ru[q]] = int32_t(rank[e]);
+        }
+    } else {
+#pragma unroll
+        for (int q = 0; q < kPer; ++q) {
+            const int e = int(threadIdx.x) + q * kRankThreads;
+            if (e >= n) continue;
+#pragma unroll
+            for (int k = 0; k < kind_dim(KIND); ++k) coords[k * n + rank[e]] = c[q][k];
+        }
     }
 }
 
 struct SprinkleLayout {
-    size_t key0, key1, raw, rank0, rank1, slot, count, start, total;
+    size_t key0, key1, raw, arrival, slot0, slot1, count, start, total;
+    int bits;
 };
 
+// The bucket counts follow the header, so one memset clears both.  A 2D
+// order's arrivals take raw's place and its second slots the arrivals'.
 SprinkleLayout sprinkle_layout(int64_t n) {
     SprinkleLayout L;
+    L.bits = bucket_bits(n);
+    const size_t buckets = size_t(1) << L.bits;
     size_t off = sizeof(WsHeader);
     auto take = [&](size_t bytes) {
         size_t at = off;
@@ -185,14 +264,14 @@ SprinkleLayout sprinkle_layout(int64_t n) {
         return at;
     };
     const size_t un = size_t(n);
+    L.count = take(2 * buckets * 4);
+    L.start = take(2 * (buckets + 64) * 4);
     L.key0 = take(un * 8);
     L.key1 = take(un * 8);
     L.raw = take(un * 16);
-    L.rank0 = take(un * 4);
-    L.rank1 = take(un * 4);
-    L.slot = take(un * 4);
-    L.count = take(size_t(kBuckets) * 4);
-    L.start = take(size_t(kBuckets + 1) * 4);
+    L.slot0 = take(un * 4);
+    L.slot1 = take(un * 4);
+    L.arrival = L.slot1;
     L.total = off;
     return L;
 }
@@ -204,19 +283,41 @@ int grid_for(int64_t n) {
     return int(b);
 }
 
-// Exact rank of each key with ties broken by index.
-cudaError_t rank_keys(int64_t n, const uint64_t* key, uint32_t* rank, uint8_t* ws, const SprinkleLayout& L,
-                      cudaStream_t st) {
-    uint32_t* count = reinterpret_cast<uint32_t*>(ws + L.count);
-    uint32_t* start = reinterpret_cast<uint32_t*>(ws + L.start);
-    uint32_t* slot = reinterpret_cast<uint32_t*>(ws + L.slot);
-    cudaError_t err = cudaMemsetAsync(count, 0, size_t(kBuckets) * 4, st);
+template <int KIND>
+cudaError_t sprinkle_kind(int64_t n, uint64_t seed, const uint64_t* thr, int32_t* coords, uint8_t* ws,
+                          cudaStream_t st) {
+    WsHeader* hdr = reinterpret_cast<WsHeader*>(ws);
+    const SprinkleLayout L = sprinkle_layout(n);
+    if (n <= kSmallSet) {
+        // 20 bytes per bucket: at most 40 KB, below the 48 KB any launch may take
+        k_sprinkle_small<KIND><<<1, kRankThreads, (size_t(1) << L.bits) * 20, st>>>(int(n), L.bits, seed, thr, coords,
+                                                                                   hdr);
+        return cudaGetLastError();
+    }
+    constexpr bool kOrder = KIND == CS_2D_ORDER;
+    constexpr int kStreams = kOrder ? 2 : 1;
+    const size_t buckets = size_t(1) << L.bits;
+    auto u32 = [&](size_t at) { return reinterpret_cast<uint32_t*>(ws + at); };
+    SprinkleScratch s;
+    s.key[0] = reinterpret_cast<uint64_t*>(ws + L.key0);
+    s.key[1] = reinterpret_cast<uint64_t*>(ws + L.key1);
+    s.raw = kOrder ? nullptr : reinterpret_cast<int32_t*>(ws + L.raw);
+    s.arrival[0] = kOrder ? u32(L.raw) : u32(L.arrival);
+    s.arrival[1] = u32(L.raw) + n;
+    s.slot[0] = u32(L.slot0);
+    s.slot[1] = u32(L.slot1);
+    for (int q = 0; q < 2; ++q) {
+        s.count[q] = u32(L.count) + q * buckets;
+        s.start[q] = u32(L.start) + q * (buckets + 64);
+    }
+    // the status word and the counts of the streams in use
+    cudaError_t err = cudaMemsetAsync(ws, 0, L.count + kStreams * buckets * 4, st);
     if (err != cudaSuccess) return err;
-    const int g = grid_for(n);
-    k_bucket_count<<<g, kThreads, 0, st>>>(n, key, count);
-    k_bucket_scan<<<1, 1024, 0, st>>>(count, start);
-    k_bucket_fill<<<g, kThreads, 0, st>>>(n, key, count, slot);
-    k_bucket_rank<<<g, kThreads, 0, st>>>(n, key, start, slot, rank);
+    const unsigned g = unsigned(grid_for(n));
+    k_keys<KIND><<<g, kThreads, 0, st>>>(n, seed, thr, s, L.bits, hdr);
+    k_bucket_scan<<<dim3(unsigned(buckets / kScanBuckets), kStreams), 256, 0, st>>>(s, n);
+    k_bucket_fill<<<dim3(g, kStreams), kThreads, 0, st>>>(n, s, L.bits);
+    k_rank_scatter<<<g, kThreads, 0, st>>>(n, kind_dim(KIND), kOrder, s, L.bits, coords);
     return cudaGetLastError();
 }
 
@@ -247,41 +348,19 @@ size_t sprinkle_workspace_bytes(int64_t n) { return sprinkle_layout(n).total; }
 
 cudaError_t launch_sprinkle(int kind, int64_t n, uint64_t seed, int32_t* coords, void* workspace,
                             cudaStream_t st) {
-    const SprinkleLayout L = sprinkle_layout(n);
     uint8_t* ws = static_cast<uint8_t*>(workspace);
-    WsHeader* hdr = reinterpret_cast<WsHeader*>(ws);
-    uint64_t* key0 = reinterpret_cast<uint64_t*>(ws + L.key0);
-    uint64_t* key1 = reinterpret_cast<uint64_t*>(ws + L.key1);
-    int32_t* raw = reinterpret_cast<int32_t*>(ws + L.raw);
-    uint32_t* rank0 = reinterpret_cast<uint32_t*>(ws + L.rank0);
-    uint32_t* rank1 = reinterpret_cast<uint32_t*>(ws + L.rank1);
-    const int g = grid_for(n);
-    cudaError_t err;
-    if (kind == CS_2D_ORDER) {
-        k_keys_2d_order<<<g, kThreads, 0, st>>>(n, seed, key0, key1);
-        if ((err = rank_keys(n, key0, rank0, ws, L, st)) != cudaSuccess) return err;
-        if ((err = rank_keys(n, key1, rank1, ws, L, st)) != cudaSuccess) return err;
-        k_scatter_2d_order<<<g, kThreads, 0, st>>>(n, rank0, rank1, coords);
-        return cudaGetLastError();
+    switch (kind) {
+        case CS_2D_ORDER: return sprinkle_kind<CS_2D_ORDER>(n, seed, nullptr, coords, ws, st);
+        case CS_2D_DIAMOND: return sprinkle_kind<CS_2D_DIAMOND>(n, seed, nullptr, coords, ws, st);
+        case CS_2D_SQUARE: return sprinkle_kind<CS_2D_SQUARE>(n, seed, nullptr, coords, ws, st);
+        case CS_2D_CYLINDER: return sprinkle_kind<CS_2D_CYLINDER>(n, seed, nullptr, coords, ws, st);
+        case CS_3D_DIAMOND: return sprinkle_kind<CS_3D_DIAMOND>(n, seed, nullptr, coords, ws, st);
+        case CS_4D_DIAMOND: return sprinkle_kind<CS_4D_DIAMOND>(n, seed, nullptr, coords, ws, st);
+        default: {
+            const uint64_t* thr = ds_table_device();
+            return thr ? sprinkle_kind<CS_2D_DS_SLAB>(n, seed, thr, coords, ws, st) : cudaErrorInvalidValue;
+        }
     }
-    if (kind == CS_2D_DIAMOND) {
-        k_keys_2d_diamond<<<g, kThreads, 0, st>>>(n, seed, raw, key0);
-    } else if (kind == CS_2D_SQUARE) {
-        k_keys_2d_square<<<g, kThreads, 0, st>>>(n, seed, raw, key0);
-    } else if (kind == CS_2D_CYLINDER) {
-        k_keys_2d_cylinder<<<g, kThreads, 0, st>>>(n, seed, raw, key0);
-    } else if (kind == CS_2D_DS_SLAB) {
-        const uint64_t* thr = ds_table_device();
-        if (!thr) return cudaErrorInvalidValue;
-        k_keys_ds_slab<<<g, kThreads, 0, st>>>(n, seed, thr, raw, key0);
-    } else if (kind == CS_3D_DIAMOND) {
-        k_keys_diamond<3><<<g, kThreads, 0, st>>>(n, seed, raw, key0, hdr);
-    } else {
-        k_keys_diamond<4><<<g, kThreads, 0, st>>>(n, seed, raw, key0, hdr);
-    }
-    if ((err = rank_keys(n, key0, rank0, ws, L, st)) != cudaSuccess) return err;
-    k_scatter_raw<<<g, kThreads, 0, st>>>(n, cs_dim(kind), rank0, raw, coords);
-    return cudaGetLastError();
 }
 
 }  // namespace cs

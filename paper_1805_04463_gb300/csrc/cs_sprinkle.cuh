@@ -116,4 +116,72 @@ __device__ __forceinline__ uint64_t draw_2d_cylinder(uint64_t s, int64_t e, int3
     return uint64_t(uint32_t(t) ^ 0x80000000u) << 32;
 }
 
+// Exact ranks of a set's n keys (ties by index: the order "sorted by time,
+// ties by generation index") in shared memory, O(n): count the keys into P
+// buckets by their top log2(P) bits (P the power of two >= n; the keys are
+// a time coordinate in the top bits, or random, so a bucket holds about
+// one key and at most a few), an exclusive scan of the counts, fill the
+// buckets, then rank each key within its bucket by comparison.  After the
+// fill, cnt[b] is the end of bucket b and cnt[b - 1] its start.  (A bitonic
+// sort of the (key, index) pairs, O(n log^2 n), took 0.38 ms for the
+// 768-set ensemble.)  sk holds the keys on entry, written before a barrier or
+// by their own threads (key i by thread i % kRankThreads).  All kRankThreads
+// threads; rank[e] receives the rank.
+constexpr int kRankThreads = 1024;
+__device__ __forceinline__ void rank_keys_smem(int n, int lgP, const uint64_t* sk, uint32_t* cnt, uint32_t* slot,
+                                               uint32_t* rank) {
+    const int P = 1 << lgP, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int shift = 64 - lgP;
+    for (int i = tid; i < P; i += kRankThreads) cnt[i] = 0u;
+    __syncthreads();
+    for (int i = tid; i < n; i += kRankThreads) atomicAdd(&cnt[sk[i] >> shift], 1u);
+    __syncthreads();
+    // exclusive scan: each thread a run of P / kRankThreads buckets (P >= 1024
+    // is ensured by the caller), warp and block offsets through shuffles
+    const int per = P / kRankThreads;
+    uint32_t run = 0;
+    for (int k = 0; k < per; ++k) run += cnt[tid * per + k];
+    uint32_t incl = run;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    __shared__ uint32_t wsum[kRankThreads / 32];
+    if (lane == 31) wsum[warp] = incl;
+    __syncthreads();
+    if (warp == 0) {
+        uint32_t w = lane < kRankThreads / 32 ? wsum[lane] : 0u, wi = w;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, wi, o);
+            if (lane >= o) wi += y;
+        }
+        if (lane < kRankThreads / 32) wsum[lane] = wi - w;  // exclusive warp offsets
+    }
+    __syncthreads();
+    uint32_t at = wsum[warp] + incl - run;
+    for (int k = 0; k < per; ++k) {
+        const uint32_t c = cnt[tid * per + k];
+        cnt[tid * per + k] = at;  // start of the bucket, then its fill cursor
+        at += c;
+    }
+    __syncthreads();
+    for (int i = tid; i < n; i += kRankThreads) slot[atomicAdd(&cnt[sk[i] >> shift], 1u)] = uint32_t(i);
+    __syncthreads();
+    for (int i = tid; i < n; i += kRankThreads) {
+        const uint64_t ke = sk[i];
+        const uint32_t bk = uint32_t(ke >> shift);
+        const uint32_t s0 = bk ? cnt[bk - 1] : 0u, s1 = cnt[bk];
+        uint32_t r = s0;
+        for (uint32_t q = s0; q < s1; ++q) {
+            const uint32_t f = slot[q];
+            const uint64_t kf = sk[f];
+            r += (kf < ke) || (kf == ke && f < uint32_t(i));
+        }
+        rank[i] = r;
+    }
+    __syncthreads();
+}
+
 }  // namespace cs

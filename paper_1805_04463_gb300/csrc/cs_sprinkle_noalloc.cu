@@ -71,8 +71,7 @@ extern "C" int cs_sprinkle_noalloc(int kind, int64_t n, uint64_t seed, int32_t* 
     if (sprinkle_workspace_bytes(CS_SPRINKLE_NOALLOC_MAX_N) > kScratchBytes) return CS_ENOMEM;
     void* scratch = nullptr;
     if (scratch_for_current_device(&scratch) != cudaSuccess) return CS_ECUDA;
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    cudaError_t e = cudaMemsetAsync(&static_cast<WsHeader*>(scratch)->status, 0, sizeof(int32_t), st);
-    if (e == cudaSuccess) e = launch_sprinkle(kind, n, seed, coords_dev, scratch, st);
-    return e == cudaSuccess ? CS_OK : CS_ECUDA;
+    return launch_sprinkle(kind, n, seed, coords_dev, scratch, static_cast<cudaStream_t>(stream)) == cudaSuccess
+               ? CS_OK
+               : CS_ECUDA;
 }
