@@ -284,9 +284,12 @@ int64_t cs_mma4_band_panels(int64_t n, size_t workspace_bytes) {
 namespace {
 
 // The least workspace a count runs with: the planned one, except on the FP4
-// path, which takes narrower bands down to one panel.
+// path, which takes narrower bands down to one panel (a band buffer holds two
+// groups of panels, so for the smallest sets the whole operands are less).
 size_t min_count_workspace(int64_t n, int path) {
-    return resolve_path(n, path) == CS_PATH_MMA4 ? mma4_band_bytes(n, 1) : cs_interval_abundance_workspace(n, path);
+    if (resolve_path(n, path) != CS_PATH_MMA4) return cs_interval_abundance_workspace(n, path);
+    const size_t band = mma4_band_bytes(n, 1), whole = mma4_workspace_bytes(n);
+    return band < whole ? band : whole;
 }
 
 // The count kernels of a resolved path.
