@@ -17,53 +17,68 @@ namespace cs {
 
 namespace {
 
-__global__ void __launch_bounds__(kActThreads) k_action_partial(int dim, int64_t n, const int64_t* __restrict__ hist,
-                                                                int64_t len, EpsArgs eps, dd* __restrict__ partial) {
-    __shared__ dd red[kActThreads];
-    const int tid = threadIdx.x;
-    const int64_t stride = int64_t(gridDim.x) * kActThreads;
-    for (int e = 0; e < eps.n; ++e) {
-        const double ep = eps.v[e];
-        if (is_local(ep)) continue;  // uniform across the grid
-        const dd q = dd_two_sum(1.0, -ep);
-        const int64_t kend = eps.kend[e];
-        dd sum = dd_from(0.0);
-        for (int64_t k = blockIdx.x * int64_t(kActThreads) + tid; k < kend; k += stride) {
-            const int64_t hk = hist[k];
-            if (hk == 0) continue;
-            const dd f = dd_mul(dd_pow(q, smear_qexp(dim, k)), smear_poly(dim, k, q, ep));
-            sum = dd_add(sum, dd_mul(dd_from_i64(hk), f));
-        }
-        red[tid] = sum;
-        __syncthreads();
-        for (int s = kActThreads / 2; s > 0; s >>= 1) {
-            if (tid < s) red[tid] = dd_add(red[tid], red[tid + s]);
-            __syncthreads();
-        }
-        if (tid == 0) partial[blockIdx.x * kMaxEps + e] = red[0];
-        __syncthreads();
-    }
+// Blocks of the smeared sum of cutoff kend with T threads each: one term per
+// thread until kActBlocks blocks are full.
+__host__ __device__ inline int act_blocks(int64_t kend, int T) {
+    const int64_t b = (kend + T - 1) / T;
+    return int(b < kActBlocks ? b : kActBlocks);
 }
 
-__global__ void k_action_final(int dim, int64_t n, const int64_t* __restrict__ hist, int64_t len, EpsArgs eps,
-                               const dd* __restrict__ partial, int nblocks, double* __restrict__ out,
-                               int64_t* __restrict__ bracket) {
-    const int e = threadIdx.x;
+// Partial smeared sums, grid (blocks of the longest cutoff, eps).  A term is
+// about 300 dependent FP64 operations (the power by repeated squaring, the
+// polynomial, two products), and GB300 issues about two FP64 lanes per SM
+// and cycle: what bounds this is how few SMs the terms sit on.  So a block
+// is one warp while the cutoffs are below 4096 terms (wider beyond),
+// the eps values run side by side, and the sum is a shuffle tree.  256
+// threads per block walking the eps values one after another took 102 us
+// for n = 1024 .. 16384 and three smeared eps; this takes 8.
+__global__ void __launch_bounds__(kActThreads) k_action_partial(int dim, const int64_t* __restrict__ hist,
+                                                                EpsArgs eps, dd* __restrict__ partial) {
+    __shared__ dd red[kActThreads / 32];
+    const int e = blockIdx.y, T = blockDim.x, tid = threadIdx.x;
+    const int64_t kend = eps.kend[e];  // 0 for a local action
+    const int nb = act_blocks(kend, T);
+    if (int(blockIdx.x) >= nb) return;
+    const double ep = eps.v[e];
+    const dd q = dd_two_sum(1.0, -ep);
+    dd sum = dd_from(0.0);
+    for (int64_t k = int64_t(blockIdx.x) * T + tid; k < kend; k += int64_t(nb) * T) {
+        const int64_t hk = hist[k];
+        if (hk == 0) continue;
+        const dd f = dd_mul(dd_pow(q, smear_qexp(dim, k)), smear_poly(dim, k, q, ep));
+        sum = dd_add(sum, dd_mul(dd_from_i64(hk), f));
+    }
+    sum = warp_sum_dd(sum);
+    if (T > 32) {  // uniform
+        if ((tid & 31) == 0) red[tid >> 5] = sum;
+        __syncthreads();
+        if (tid < 32) sum = warp_sum_dd(tid < T / 32 ? red[tid] : dd_from(0.0));
+    }
+    if (tid == 0) partial[e * kActBlocks + blockIdx.x] = sum;
+}
+
+// One warp per eps: its partial sums, the action; warp 0 writes the bracket.
+__global__ void __launch_bounds__(32 * kMaxEps) k_action_final(int dim, int64_t n, const int64_t* __restrict__ hist,
+                                                               int64_t len, EpsArgs eps, int T,
+                                                               const dd* __restrict__ partial,
+                                                               double* __restrict__ out,
+                                                               int64_t* __restrict__ bracket) {
+    const int e = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int64_t h4[4] = {0, 0, 0, 0};
     for (int k = 0; k < 4 && k < len; ++k) h4[k] = hist[k];
     const int64_t b = bracket_of(dim, n, h4);
-    if (e == 0 && bracket) *bracket = b;
-    if (e >= eps.n) return;
+    if (threadIdx.x == 0 && bracket) *bracket = b;
     const double ep = eps.v[e];
     dd s;
     if (is_local(ep)) {
-        s = local_action(dim, b);
+        s = local_action(eps.factor[e], b);
     } else {
+        const int nb = act_blocks(eps.kend[e], T);
         dd sum = dd_from(0.0);
-        for (int blk = 0; blk < nblocks; ++blk) sum = dd_add(sum, partial[blk * kMaxEps + e]);
-        s = smeared_action(dim, n, ep, sum);
+        for (int k = lane; k < nb; k += 32) sum = dd_add(sum, partial[e * kActBlocks + k]);
+        s = smeared_action(dim, n, ep, eps.factor[e], warp_sum_dd(sum));
     }
-    out[e] = s.hi + s.lo;
+    if (lane == 0) out[e] = s.hi + s.lo;
 }
 
 // B phi(j) from the layer sums (Eqs. b2d_local, b3d_local, b4d_local), one
@@ -111,7 +126,7 @@ int action_host(int dim, int64_t n, const int64_t* hist, int64_t len, double eps
     if (bracket) *bracket = b;
     dd s;
     if (is_local(eps)) {
-        s = local_action(dim, b);
+        s = local_action(local_factor(dim), b);
     } else {
         const dd q = dd_two_sum(1.0, -eps);
         double R = 0.0;  // any histogram may come in here: bound by its own sum
@@ -123,7 +138,7 @@ int action_host(int dim, int64_t n, const int64_t* hist, int64_t len, double eps
             if (hist[k] != 0) sum = dd_add(sum, dd_mul(dd_from_i64(hist[k]), dd_mul(p, smear_poly(dim, k, q, eps))));
             if (k >= deg) p = dd_mul(p, q);
         }
-        s = smeared_action(dim, n, eps, sum);
+        s = smeared_action(dim, n, eps, smeared_factor(dim, eps), sum);
     }
     if (out) *out = s.hi + s.lo;
     return CS_OK;
@@ -133,23 +148,19 @@ cudaError_t launch_action_device(int dim, int64_t n, const int64_t* hist, int64_
                                  double* out, int64_t* bracket, void* workspace, cudaStream_t st) {
     EpsArgs a;
     a.n = n_eps;
-    bool any_smeared = false;
+    int64_t kmax = 0;
     for (int e = 0; e < kMaxEps; ++e) {
         a.v[e] = e < n_eps ? eps[e] : 0.0;
         a.kend[e] = is_local(a.v[e]) ? 0 : smear_cutoff(dim, a.v[e], 0.5 * double(n) * double(n), len);
-        if (e < n_eps && !is_local(a.v[e])) any_smeared = true;
+        a.factor[e] = e < n_eps ? action_factor(dim, a.v[e]) : dd_from(0.0);
+        kmax = a.kend[e] > kmax ? a.kend[e] : kmax;
     }
-    // Blocks that hold terms only: block b's threads take k = 256 b + t (one
-    // term each while the grid covers the longest cutoff), and the blocks
-    // past the last term would only add exact zeros (FP64 is scarce here:
-    // their reductions had made both kernels about 0.1 ms each).
-    int64_t kmax = 0;
-    for (int e = 0; e < n_eps; ++e) kmax = a.kend[e] > kmax ? a.kend[e] : kmax;
-    int64_t blocks = (kmax + kActThreads - 1) / kActThreads;
-    blocks = blocks < 1 ? 1 : (blocks > kActBlocks ? kActBlocks : blocks);
+    int T = 32;  // threads per block: the fewest that give each thread one term
+    while (T < kActThreads && kmax > int64_t(kActBlocks) * T) T *= 2;
     dd* partial = reinterpret_cast<dd*>(static_cast<uint8_t*>(workspace) + sizeof(WsHeader));
-    if (any_smeared) k_action_partial<<<unsigned(blocks), kActThreads, 0, st>>>(dim, n, hist, len, a, partial);
-    k_action_final<<<1, 32, 0, st>>>(dim, n, hist, len, a, partial, int(blocks), out, bracket);
+    if (kmax > 0)
+        k_action_partial<<<dim3(unsigned(act_blocks(kmax, T)), unsigned(n_eps)), T, 0, st>>>(dim, hist, a, partial);
+    k_action_final<<<1, 32 * n_eps, 0, st>>>(dim, n, hist, len, a, T, partial, out, bracket);
     return cudaGetLastError();
 }
 

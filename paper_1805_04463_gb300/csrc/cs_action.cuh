@@ -11,11 +11,12 @@ namespace cs {
 
 constexpr int kMaxEps = 16;  // eps values per call
 constexpr int kActThreads = 256;
-constexpr int kActBlocks = 128;
+constexpr int kActBlocks = 128;  // partial sums per eps
 
 struct EpsArgs {
     double v[kMaxEps];
     int64_t kend[kMaxEps];  // smeared-sum cutoffs (single-set kernels; set on the host)
+    dd factor[kMaxEps];     // action_factor (single-set kernels; the batch has one set per dimension)
     int n;
 };
 
@@ -54,31 +55,46 @@ __host__ __device__ inline double c3_const() {
 
 __host__ __device__ inline bool is_local(double eps) { return eps <= 0.0 || eps == 1.0; }
 
-// Local action: 2 * bracket (1+1), c3 * bracket / 8 (2+1) or
-// 4/sqrt(6) * bracket (3+1).
-__host__ __device__ inline dd local_action(int dim, int64_t bracket) {
-    const dd b = dd_from_i64(bracket);
-    if (dim == 2) return dd_mul_d(b, 2.0);
-    if (dim == 3) return dd_mul_d(b, c3_const() * 0.125);
-    return dd_mul(dd_div(dd_from(4.0), dd_sqrt(dd_from(6.0))), b);
+// Factors of the actions that depend on eps (and the dimension) alone, found
+// on the host: on the device the 2+1 and 3+1 ones are a cube root, a gamma
+// function and two double-double divisions, FP64 work in one thread.
+//   local:   2 * bracket (1+1), c3 * bracket / 8 (2+1), 4/sqrt(6) * bracket (3+1)
+//   smeared, from sum = sum_k N_k f(k, eps):
+//     1+1: 2 eps [N - 2 eps sum];  2+1: c3 eps^(2/3) [N - eps sum];
+//     3+1: 4 sqrt(eps/6) [N - eps sum].
+inline dd local_factor(int dim) {
+    if (dim == 2) return dd_from(2.0);
+    if (dim == 3) return dd_from(c3_const() * 0.125);
+    return dd_div(dd_from(4.0), dd_sqrt(dd_from(6.0)));
 }
 
-// Smeared action from sum = sum_k N_k f(k, eps):
-//   1+1: 2 eps [N - 2 eps sum];  2+1: c3 eps^(2/3) [N - eps sum];
-//   3+1: 4 sqrt(eps/6) [N - eps sum].
-__host__ __device__ inline dd smeared_action(int dim, int64_t n, double eps, dd sum) {
-    const dd e = dd_from(eps);
-    if (dim == 2) {
-        const dd inner = dd_sub(dd_from_i64(n), dd_mul(dd_mul_d(e, 2.0), sum));
-        return dd_mul(dd_mul_d(e, 2.0), inner);
-    }
-    const dd inner = dd_sub(dd_from_i64(n), dd_mul(e, sum));
+inline dd smeared_factor(int dim, double eps) {
+    if (dim == 2) return dd_mul_d(dd_from(eps), 2.0);
     if (dim == 3) {
         const double r = cbrt(eps);
-        return dd_mul_d(inner, c3_const() * (r * r));
+        return dd_from(c3_const() * (r * r));
     }
-    const dd pref = dd_mul_d(dd_sqrt(dd_div(e, dd_from(6.0))), 4.0);
-    return dd_mul(pref, inner);
+    return dd_mul_d(dd_sqrt(dd_div(dd_from(eps), dd_from(6.0))), 4.0);
+}
+
+// The factor of one eps value, local or smeared.
+inline dd action_factor(int dim, double eps) { return is_local(eps) ? local_factor(dim) : smeared_factor(dim, eps); }
+
+__host__ __device__ inline dd local_action(dd factor, int64_t bracket) { return dd_mul(factor, dd_from_i64(bracket)); }
+
+__host__ __device__ inline dd smeared_action(int dim, int64_t n, double eps, dd factor, dd sum) {
+    const dd e = dim == 2 ? dd_mul_d(dd_from(eps), 2.0) : dd_from(eps);
+    return dd_mul(factor, dd_sub(dd_from_i64(n), dd_mul(e, sum)));
+}
+
+// Sum of one double-double per lane, in every lane.
+__device__ __forceinline__ dd warp_sum_dd(dd v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const dd y{__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)};
+        v = dd_add(v, y);
+    }
+    return v;
 }
 
 // Terms k >= K of the smeared sum that can be dropped.  For k >= deg,

@@ -233,6 +233,7 @@ struct CoefArgs {
     int64_t stride[kDimSlots];            // entries per eps (the slot's largest n)
     int64_t kcap[kDimSlots][kMaxEps];     // entries computed per (slot, eps)
     int64_t seg[kDimSlots * kMaxEps + 1];  // prefix sums of kcap in (slot, eps) order
+    dd factor[kDimSlots][kMaxEps];         // action_factor per (slot, eps)
 };
 
 // The same launch finds each (set, eps) cutoff once (kends), after the
@@ -267,10 +268,9 @@ __global__ void __launch_bounds__(32) k_batch_coef(dd* __restrict__ coef, CoefAr
 
 // One CTA per (set, eps): the set's bracket (written by its eps-0 CTA) and
 // one local or smeared action; the smeared sums take their coefficients from
-// the shared table.  Each sum keeps the per-thread order and the reduction
-// tree of the single-set action, so both give the same bits; a CTA per set
-// walking its eps values one after another left the FP64 pipe waiting on
-// the sums' dependency chains (0.29 ms for 768 sets and three smeared eps).
+// the shared table.  A CTA per set walking its eps values one after another
+// left the FP64 pipe waiting on the sums' dependency chains (0.29 ms for 768
+// sets and three smeared eps).
 __global__ void __launch_bounds__(kActThreads) k_batch_action(const BatchSet* __restrict__ sets,
                                                               const int64_t* __restrict__ hist_base, EpsArgs eps,
                                                               const dd* __restrict__ coef, CoefArgs c,
@@ -293,7 +293,7 @@ __global__ void __launch_bounds__(kActThreads) k_batch_action(const BatchSet* __
     const double ep = eps.v[e];
     if (is_local(ep)) {  // uniform across the CTA
         if (tid == 0 && actions) {
-            const dd s = local_action(dim, br);
+            const dd s = local_action(c.factor[slot][e], br);
             actions[int64_t(set) * eps.n + e] = s.hi + s.lo;
         }
         return;
@@ -312,7 +312,7 @@ __global__ void __launch_bounds__(kActThreads) k_batch_action(const BatchSet* __
         __syncthreads();
     }
     if (tid == 0 && actions) {
-        const dd s = smeared_action(dim, n, ep, red[0]);
+        const dd s = smeared_action(dim, n, ep, c.factor[slot][e], red[0]);
         actions[int64_t(set) * eps.n + e] = s.hi + s.lo;
     }
 }
@@ -644,6 +644,7 @@ int cs_batch_launch(const cs_batch* b, const double* eps_host, int n_eps, int64_
     for (int e = 0; e < kMaxEps; ++e) {
         a.v[e] = e < n_eps ? eps_host[e] : 0.0;
         a.kend[e] = 0;  // per set, in the kernel
+        a.factor[e] = dd_from(0.0);  // per dimension, in CoefArgs
         if (e < n_eps && !(a.v[e] <= 1.0)) return CS_EINVAL;
     }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -723,6 +724,7 @@ int cs_batch_launch(const cs_batch* b, const double* eps_host, int n_eps, int64_
                                    : 0;
                 c.seg[d * kMaxEps + e] = at;
                 at += c.kcap[d][e];
+                c.factor[d][e] = nm > 0 && e < n_eps ? action_factor(d + 2, a.v[e]) : dd_from(0.0);
             }
         }
         c.seg[kDimSlots * kMaxEps] = at;
