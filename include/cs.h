@@ -274,6 +274,23 @@ int cs_interval_abundance(int64_t n, const uint64_t *bits_dev, int64_t row_words
                           void *workspace_dev, size_t workspace_bytes, void *stream);
 
 /*
+ * The same abundances from the coordinates of a set whose relation is the
+ * product order of two of them (CS_2D_ORDER, CS_2D_DIAMOND, CS_2D_SQUARE): with
+ * elements numbered by u, |A_ab| is a difference of four counts
+ * #{c < x : v_c < y}, looked up in a table of n^2 / 128 bytes, O(n^2) for the
+ * whole set.  coords_dev as for cs_causal_matrix (any order of labels for the
+ * diamond and the square).  hist_dev is zeroed and then filled by the
+ * callee, with the same values as cs_interval_abundance on the set's causal
+ * matrix.  cs_evaluate and cs_batch_* take this route where path is
+ * CS_PATH_AUTO.  The workspace query returns 0 where the route is not taken
+ * (another kind, or n outside its range) and the call then returns
+ * CS_EUNSUPPORTED.  Errors: CS_EINVAL, CS_ENOMEM, CS_EUNSUPPORTED, CS_ECUDA.
+ */
+size_t cs_coords_abundance_workspace(int kind, int64_t n);
+int cs_coords_abundance(int kind, int64_t n, const int32_t *coords_dev, int64_t *hist_dev,
+                        void *workspace_dev, size_t workspace_bytes, void *stream);
+
+/*
  * Interval abundances plus the layer sums of the discrete d'Alembertian
  * (Section "The Benincasa-Dowker Action", Eqs. b2d_local, b4d_local): in the
  * same pass as cs_interval_abundance, for every element j and m = 0..kmax,

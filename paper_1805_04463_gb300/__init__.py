@@ -22,7 +22,8 @@ __all__ = [
     "sprinkle_workspace_bytes", "interval_abundance_workspace", "resolved_path", "action_workspace_bytes",
     "set_auto_paths", "get_auto_paths", "set_auto_memory_limit", "get_auto_memory_limit",
     "set_auto_tiles", "get_auto_tiles", "set_batch_tuning", "get_batch_tuning",
-    "sprinkle", "sprinkle_noalloc", "causal_matrix", "layer_sums", "dalembertian", "interval_abundance", "workspace_status", "action", "action_device",
+    "sprinkle", "sprinkle_noalloc", "causal_matrix", "layer_sums", "dalembertian", "interval_abundance", "coords_abundance_workspace",
+    "coords_abundance", "workspace_status", "action", "action_device",
     "evaluate", "Buffers", "allocate", "run", "SetDesc", "Batch", "CountJob", "count_items",
     "operands_bytes", "prepare_operands", "peak_probe", "count_jobs", "degrees", "sparse_relations", "longest_chain", "greedy_antichain", "BATCH_MAX_N", "FAULT_ALLOC", "FAULT_LAUNCH", "selftest_wait",
     "inject_fault",
@@ -91,6 +92,8 @@ def lib() -> ctypes.CDLL:
             "cs_get_batch_tuning": ([ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int)], i32),
             "cs_get_auto_memory_limit": ([], sz),
             "cs_interval_abundance": ([i64, vp, i64, vp, i32, vp, sz, vp], i32),
+            "cs_coords_abundance_workspace": ([i32, i64], sz),
+            "cs_coords_abundance": ([i32, i64, vp, vp, vp, sz, vp], i32),
             "cs_workspace_status": ([vp, vp], i32),
             "cs_layer_sums": ([i64, vp, i64, vp, i32, vp, i32, vp, vp, sz, vp], i32),
             "cs_dalembertian": ([i32, i64, vp, vp, i32, ctypes.c_double, vp, vp], i32),
@@ -288,6 +291,17 @@ def interval_abundance(n, bits, hist, path=PATH_AUTO, workspace=None, stream=Non
                                        _nbytes(workspace), _stream(stream)), "cs_interval_abundance")
 
 
+def coords_abundance_workspace(kind: int, n: int) -> int:
+    """Workspace of coords_abundance(), 0 where it does not take (kind, n)."""
+    return lib().cs_coords_abundance_workspace(kind, n)
+
+
+def coords_abundance(kind, n, coords, hist, workspace, stream=None):
+    """cs_coords_abundance: the N_k of a 1+1 product order straight from its coordinates."""
+    _check(lib().cs_coords_abundance(kind, n, _ptr(coords), _ptr(hist), _ptr(workspace), _nbytes(workspace),
+                                     _stream(stream)), "cs_coords_abundance")
+
+
 def layer_sums(n, bits, hist, layer, kmax, phi=None, path=PATH_AUTO, workspace=None, stream=None):
     """cs_layer_sums: histogram plus d'Alembertian layer sums layer[(kmax+1), n] (float64)."""
     _check(lib().cs_layer_sums(n, _ptr(bits), bits.shape[-1], _ptr(hist), path, _ptr(phi), kmax, _ptr(layer),
@@ -359,7 +373,10 @@ class Buffers:
         self.coords = torch.empty((self.dim, n), dtype=torch.int32, device=device)
         self.bits = torch.empty((n, self.rw), dtype=torch.int64, device=device)
         self.hist = torch.empty(hist_len(n), dtype=torch.int64, device=device)
-        ws = max(sprinkle_workspace_bytes(kind, n), interval_abundance_workspace(n, path), action_workspace_bytes())
+        # AUTO counts a 1+1 product order from its coordinates
+        self.by_coords = path == PATH_AUTO and coords_abundance_workspace(kind, n) > 0
+        ws = max(sprinkle_workspace_bytes(kind, n), interval_abundance_workspace(n, path), action_workspace_bytes(),
+                 coords_abundance_workspace(kind, n) if self.by_coords else 0)
         self.workspace = torch.empty(ws, dtype=torch.uint8, device=device)
         self.actions = torch.empty(16, dtype=torch.float64, device=device)
         self.bracket = torch.empty(1, dtype=torch.int64, device=device)
@@ -374,7 +391,10 @@ def run(buf: Buffers, seed: int, eps=(0.0,), stream=None, sprinkle_=True):
     if sprinkle_:
         sprinkle(buf.kind, buf.n, seed, buf.coords, buf.workspace, stream)
     causal_matrix(buf.kind, buf.n, buf.coords, buf.bits, stream)
-    interval_abundance(buf.n, buf.bits, buf.hist, buf.path, buf.workspace, stream)
+    if buf.by_coords:
+        coords_abundance(buf.kind, buf.n, buf.coords, buf.hist, buf.workspace, stream)
+    else:
+        interval_abundance(buf.n, buf.bits, buf.hist, buf.path, buf.workspace, stream)
     if eps:
         action_device(buf.dim, buf.n, buf.hist, list(eps), buf.actions, buf.bracket, buf.workspace, stream)
 

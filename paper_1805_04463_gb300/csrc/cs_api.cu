@@ -320,6 +320,26 @@ int cs_interval_abundance(int64_t n, const uint64_t* bits_dev, int64_t row_words
     return from_cuda(e);
 }
 
+size_t cs_coords_abundance_workspace(int kind, int64_t n) {
+    if (cs_dim(kind) == 0 || !valid_n(n) || !order_count_fits(kind, n)) return 0;
+    return order_workspace_bytes(n);
+}
+
+int cs_coords_abundance(int kind, int64_t n, const int32_t* coords_dev, int64_t* hist_dev, void* workspace_dev,
+                        size_t workspace_bytes, void* stream) {
+    CS_TRACE("cs_coords_abundance");
+    if (cs_dim(kind) == 0 || !valid_n(n) || !coords_dev || !aligned(coords_dev, 4) || !hist_dev ||
+        !aligned(hist_dev, 8) || !workspace_dev || !aligned(workspace_dev, 256))
+        return CS_EINVAL;
+    if (!order_count_fits(kind, n)) return CS_EUNSUPPORTED;
+    if (workspace_bytes < order_workspace_bytes(n)) return CS_ENOMEM;
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (fault_injected(CS_FAULT_LAUNCH)) return CS_ECUDA;
+    cudaError_t e = clear_status(workspace_dev, st);
+    if (e == cudaSuccess) e = launch_count_order(kind, n, coords_dev, hist_dev, workspace_dev, st);
+    return from_cuda(e);
+}
+
 int cs_layer_sums(int64_t n, const uint64_t* bits_dev, int64_t row_words, int64_t* hist_dev, int path,
                   const double* phi_dev, int kmax, double* layer_dev, void* workspace_dev, size_t workspace_bytes,
                   void* stream) {
@@ -409,7 +429,10 @@ int cs_evaluate(int kind, int64_t n, uint64_t seed, const int32_t* coords_host, 
 
     const int64_t rw = cs_row_words(n);
     const int64_t hl = cs_hist_len(n);
-    size_t ws_bytes = cs_interval_abundance_workspace(n, path);
+    // AUTO counts a product order from its coordinates, without a causal matrix
+    const bool by_coords = path == CS_PATH_AUTO && order_count_fits(kind, n);
+    size_t ws_bytes = by_coords ? order_workspace_bytes(n) : cs_interval_abundance_workspace(n, path);
+    const size_t bits_bytes = by_coords ? 0 : cs_bitset_bytes(n);
     if (cs_sprinkle_workspace_bytes(kind, n) > ws_bytes) ws_bytes = cs_sprinkle_workspace_bytes(kind, n);
     if (action_workspace_bytes() > ws_bytes) ws_bytes = action_workspace_bytes();
 
@@ -424,7 +447,7 @@ int cs_evaluate(int kind, int64_t n, uint64_t seed, const int32_t* coords_host, 
             rc = CS_ENOMEM;
     };
     alloc(reinterpret_cast<void**>(&coords), cs_coords_bytes(kind, n));
-    alloc(reinterpret_cast<void**>(&bits), cs_bitset_bytes(n));
+    if (bits_bytes) alloc(reinterpret_cast<void**>(&bits), bits_bytes);
     alloc(reinterpret_cast<void**>(&hist), size_t(hl) * 8);
     alloc(&ws, ws_bytes);
     alloc(reinterpret_cast<void**>(&out), 17 * 8);
@@ -440,8 +463,12 @@ int cs_evaluate(int kind, int64_t n, uint64_t seed, const int32_t* coords_host, 
     if (rc == CS_OK && !coords_host)
         rc = from_cuda(cudaMemcpyAsync(&status_sprinkle, &static_cast<WsHeader*>(ws)->status, sizeof(int32_t),
                                        cudaMemcpyDeviceToHost, st));
-    if (rc == CS_OK) rc = cs_causal_matrix(kind, n, coords, bits, rw, st);
-    if (rc == CS_OK) rc = cs_interval_abundance(n, bits, rw, hist, path, ws, ws_bytes, st);
+    if (by_coords) {
+        if (rc == CS_OK) rc = cs_coords_abundance(kind, n, coords, hist, ws, ws_bytes, st);
+    } else {
+        if (rc == CS_OK) rc = cs_causal_matrix(kind, n, coords, bits, rw, st);
+        if (rc == CS_OK) rc = cs_interval_abundance(n, bits, rw, hist, path, ws, ws_bytes, st);
+    }
     int32_t status = 0;
     if (rc == CS_OK)
         rc = from_cuda(cudaMemcpyAsync(&status, &static_cast<WsHeader*>(ws)->status, sizeof(status),
@@ -467,7 +494,7 @@ int cs_evaluate(int kind, int64_t n, uint64_t seed, const int32_t* coords_host, 
     // Freed blocks stay in the pool for the next call, except after a call
     // that took more than a quarter of the device: those go back at once, so
     // one very large evaluation does not hold its memory for the process.
-    const size_t took = cs_coords_bytes(kind, n) + cs_bitset_bytes(n) + size_t(hl) * 8 + ws_bytes;
+    const size_t took = cs_coords_bytes(kind, n) + bits_bytes + size_t(hl) * 8 + ws_bytes;
     if (took > device_total_memory() / 4) {
         cudaMemPool_t pool;
         if (cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess) cudaMemPoolTrimTo(pool, 0);

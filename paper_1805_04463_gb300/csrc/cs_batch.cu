@@ -12,6 +12,10 @@
 //                   diagonal word) of every bitset, one launch per geometry;
 //   k_batch_mirror  the lower triangle of every bitset, the transpose of the
 //                   upper one (the past rows);
+//   order table, order count   on CS_PATH_AUTO, for the product orders (2D
+//                   orders, the 1+1 diamond and square): the table of prefix
+//                   ranks and the pair count from it (cs_order.cuh), in
+//                   place of relate, mirror and the count below;
 //   count           the multi-set POPC kernel, or expand + multi-set tcgen05
 //                   kernel: one persistent grid over the tiles of all sets,
 //                   largest sets first (longest-processing-time order);
@@ -29,6 +33,7 @@
 #include <atomic>
 
 #include "cs_kernels.cuh"
+#include "cs_order.cuh"
 #include "cs_relate.cuh"
 #include "cs_sprinkle.cuh"
 
@@ -55,7 +60,18 @@ struct BatchSet {
     int64_t hist_off;      // offset of this set's histogram in the batch histogram
     ConeTable* ctab;       // light-cone kinds: one column table per column tile (else null)
     int64_t tile_begin;    // first column tile of this set in the concatenated tile range
+    OrderSet order;        // counted as a product order (p not null): its arrays, and no bits
+    int64_t ord_block;     // first block of this set in the order table build
+    int64_t ord_task;      // first of its tasks in the order count
 };
+
+// A set counted from its prefix-rank table.
+__host__ __device__ __forceinline__ bool by_order(const BatchSet& b) { return b.order.p != nullptr; }
+
+// Bands per column chunk of the order count's tasks, and its threads: two
+// CTAs per SM, so that one counts while the other flushes.
+constexpr int kBatchOrderM = 2;
+constexpr int kBatchOrderThreads = 512;
 
 __device__ __forceinline__ int find_set_elem(const BatchSet* sets, int nsets, int64_t idx) {
     int lo = 0, hi = nsets - 1;
@@ -109,6 +125,12 @@ __global__ void __launch_bounds__(kRankThreads) k_batch_rank(const BatchSet* __r
     uint32_t* slot = cnt + P;
     uint32_t* rank = slot + P;
     uint32_t* ru = rank + P;
+    int32_t* op = const_cast<int32_t*>(b.order.p);
+    int32_t* oq = const_cast<int32_t*>(b.order.q);
+    if (by_order(b) && b.kind != CS_2D_ORDER) {  // the count needs the ranks of u and v, not the time order
+        order_ranks_smem(b.raw, b.raw + n, false, n, lgP, smem_raw, op, oq);
+        return;
+    }
     auto load = [&](const uint64_t* key) {
         for (int i = threadIdx.x; i < n; i += kRankThreads) sk[i] = key[i];
     };
@@ -120,8 +142,13 @@ __global__ void __launch_bounds__(kRankThreads) k_batch_rank(const BatchSet* __r
         load(b.key1);
         rank_keys_smem(n, lgP, sk, cnt, slot, rank);
         for (int e = threadIdx.x; e < n; e += kRankThreads) {
-            b.coords[ru[e]] = int32_t(ru[e]);
-            b.coords[n + ru[e]] = int32_t(rank[e]);
+            if (by_order(b)) {
+                op[ru[e]] = int32_t(rank[e]);
+                oq[rank[e]] = int32_t(ru[e]);
+            } else {
+                b.coords[ru[e]] = int32_t(ru[e]);
+                b.coords[n + ru[e]] = int32_t(rank[e]);
+            }
         }
     } else {
         for (int e = threadIdx.x; e < n; e += kRankThreads) {
@@ -140,6 +167,59 @@ __global__ void __launch_bounds__(256) k_batch_ctab(const BatchSet* __restrict__
     if (g >= tiles) return;
     const BatchSet& b = sets[tile_set[g]];
     if (b.ctab) build_cone_table(b.coords, b.n, g - b.tile_begin, b.kind == CS_2D_ORDER, b.ctab + (g - b.tile_begin));
+}
+
+// The prefix-rank tables of the sets counted as product orders, eight rows
+// per block, the set read from a table.
+__global__ void __launch_bounds__(kOrdBuildThreads) k_batch_order_table(const BatchSet* __restrict__ sets,
+                                                                        const int32_t* __restrict__ block_set) {
+    const BatchSet& b = sets[block_set[blockIdx.x]];
+    order_build_rows(b.order, int(int64_t(blockIdx.x) - b.ord_block));
+}
+
+// Their pair counts.  Each CTA takes an equal, contiguous share of the
+// concatenated task list (tasks cost alike), so it meets few sets: its warps
+// stride over the share's tasks of a set, then the CTA adds its shared
+// histogram to the set's and clears it.  order_sets: the sets in task order.
+__global__ void __launch_bounds__(kBatchOrderThreads, 2) k_batch_order_count(const BatchSet* __restrict__ sets,
+                                                                          const int32_t* __restrict__ order_sets,
+                                                                          int n_order, int64_t tasks,
+                                                                          int64_t* __restrict__ hist_base) {
+    constexpr int kWarps = kBatchOrderThreads / 32;
+    extern __shared__ __align__(16) uint8_t smem_ord[];
+    const int warp = threadIdx.x >> 5;
+    int2* stage = reinterpret_cast<int2*>(smem_ord) + 32 * warp;
+    uint32_t* shist = reinterpret_cast<uint32_t*>(smem_ord + kWarps * 32 * sizeof(int2));
+    const uint32_t hist_s = smem_u32(shist);
+    int64_t t = tasks * blockIdx.x / gridDim.x;
+    const int64_t end = tasks * (blockIdx.x + 1) / gridDim.x;
+    int r = 0;  // the last set whose tasks begin at or before t
+    for (int hi = n_order - 1; r < hi;) {
+        const int mid = (r + hi + 1) >> 1;
+        if (sets[order_sets[mid]].ord_task <= t) r = mid; else hi = mid - 1;
+    }
+    for (; t < end; ++r) {
+        const BatchSet& b = sets[order_sets[r]];
+        const OrderSet s = b.order;
+        const int bins = s.n > 1 ? s.n - 1 : 1;  // every count of the set
+        unsigned long long* hist = reinterpret_cast<unsigned long long*>(hist_base + b.hist_off);
+        for (int k = threadIdx.x; k < bins; k += kBatchOrderThreads) shist[k] = 0u;
+        __syncthreads();
+        const int64_t own = b.ord_task + order_tasks(s.n, kBatchOrderM);  // end of the set's tasks
+        const int64_t stop = own < end ? own : end;
+        for (int64_t q = t + warp; q < stop; q += kWarps) {
+            int A, C;
+            order_decode(q - b.ord_task, kBatchOrderM, A, C);
+            order_task(s, A, C, kOrdBand * kBatchOrderM, hist_s, bins, hist, stage);
+        }
+        __syncthreads();
+        for (int k = threadIdx.x; k < bins; k += kBatchOrderThreads) {
+            const uint32_t c = shist[k];
+            if (c) atomicAdd(hist + k, (unsigned long long)c);
+        }
+        t = stop;
+        __syncthreads();
+    }
 }
 
 // Relate chunks.  Row tile rb of a set with V valid words needs words
@@ -344,6 +424,12 @@ struct cs_batch {
     int64_t total_mblocks = 0;
     int64_t total_tiles = 0;  // column tiles of all sets (k_batch_ctab's warps)
     int32_t* ttab = nullptr;  // column tile -> set
+    int n_general = 0;  // sets counted from their causal matrix
+    int n_order = 0;    // sets counted as product orders
+    int32_t* otab = nullptr;   // order table block -> set
+    int32_t* osets = nullptr;  // the product orders, in task order
+    int64_t ord_blocks = 0, ord_tasks = 0;
+    int64_t ord_nmax = 0;      // the largest of them
     unsigned geoms = 0;  // bit G: some set relates with geometry G
     int max_pow2 = 1;
     const uint64_t* ds_thr = nullptr;  // de Sitter thresholds, when a set needs them
@@ -364,8 +450,9 @@ struct cs_batch {
 namespace {
 
 struct Layout {
-    size_t sets, entries, rtab, rorder, etab, mtab, ttab, coef, kends, total;
+    size_t sets, entries, rtab, rorder, etab, mtab, ttab, otab, osets, coef, kends, total;
     std::vector<size_t> coords, bits, key0, key1, raw, ctab, op0, op1;
+    std::vector<size_t> ord_p, ord_q, ord_r, ord_d;  // product orders
 };
 
 bool batch_valid(const cs_set_desc* sets, int n_sets) {
@@ -383,7 +470,11 @@ int batch_path(const cs_set_desc* sets, int n_sets, int path) {
 
 bool tensor_path(int path) { return path == CS_PATH_MMA || path == CS_PATH_MMA4; }
 
-Layout batch_layout(const cs_set_desc* sets, int n_sets, int path) {
+// On CS_PATH_AUTO a product order is counted from its coordinates.  (Every
+// size: in a batch the route's launches are shared by all sets.)
+bool set_by_order(const cs_set_desc& d, bool auto_path) { return auto_path && order_kind(d.kind) && d.n >= 2; }
+
+Layout batch_layout(const cs_set_desc* sets, int n_sets, int path, bool auto_path) {
     Layout L;
     size_t off = sizeof(WsHeader);
     auto take = [&](size_t bytes) {
@@ -394,9 +485,13 @@ Layout batch_layout(const cs_set_desc* sets, int n_sets, int path) {
     L.sets = take(sizeof(BatchSet) * size_t(n_sets));
     off = align_up(off, 128);
     L.entries = take((tensor_path(path) ? sizeof(MmaSetEntry) : sizeof(PopcSetEntry)) * size_t(n_sets));
-    int64_t rblocks = 0, chunks = 0, mblocks = 0, tiles = 0;
+    int64_t rblocks = 0, chunks = 0, mblocks = 0, tiles = 0, oblocks = 0;
     for (int s = 0; s < n_sets; ++s) {
         const int64_t n = sets[s].n;
+        if (set_by_order(sets[s], auto_path)) {
+            oblocks += order_build_blocks(n);
+            continue;
+        }
         rblocks += chunk_sum((n + 63) / 64);
         tiles += (n + 63) / 64;
         const int64_t side = ((n + 63) / 64 + kMirTiles - 1) / kMirTiles;
@@ -408,6 +503,8 @@ Layout batch_layout(const cs_set_desc* sets, int n_sets, int path) {
     L.etab = take(size_t(chunks) * 4);   // expansion chunk -> set
     L.mtab = take(size_t(mblocks) * 4);  // mirror block -> set
     L.ttab = take(size_t(tiles) * 4);    // column tile -> set
+    L.otab = take(size_t(oblocks) * 4);  // order table block -> set
+    L.osets = take(size_t(n_sets) * 4);  // the product orders
     int64_t nmax[kDimSlots] = {0, 0, 0};
     for (int s = 0; s < n_sets; ++s) {
         int64_t& m = nmax[cs_dim(sets[s].kind) - 2];
@@ -418,14 +515,23 @@ Layout batch_layout(const cs_set_desc* sets, int n_sets, int path) {
     for (int s = 0; s < n_sets; ++s) {
         const int64_t n = sets[s].n;
         const int dim = cs_dim(sets[s].kind);
-        L.coords.push_back(take(size_t(n) * dim * 4));
-        L.bits.push_back(take(size_t(n) * size_t(cs_row_words(n)) * 8));
+        const bool order = set_by_order(sets[s], auto_path);
+        L.ord_p.push_back(order ? take(size_t(n) * 4) : 0);
+        L.ord_q.push_back(order ? take(size_t(n) * 4) : 0);
+        L.ord_r.push_back(order ? take(size_t(n) * 4) : 0);
+        L.ord_d.push_back(order ? take(order_table_bytes(n)) : 0);
+        L.coords.push_back(order ? 0 : take(size_t(n) * dim * 4));
+        L.bits.push_back(order ? 0 : take(size_t(n) * size_t(cs_row_words(n)) * 8));
         L.key0.push_back(take(size_t(n) * 8));
         L.key1.push_back(take(size_t(n) * 8));
         L.raw.push_back(take(size_t(n) * 16));
-        L.ctab.push_back(batch_geom(sets[s].kind) == kGeomLightCone ? take(size_t((n + 63) / 64) * sizeof(ConeTable))
-                                                                    : 0);
-        if (tensor_path(path)) {
+        L.ctab.push_back(!order && batch_geom(sets[s].kind) == kGeomLightCone
+                             ? take(size_t((n + 63) / 64) * sizeof(ConeTable))
+                             : 0);
+        if (order) {
+            L.op0.push_back(0);
+            L.op1.push_back(0);
+        } else if (tensor_path(path)) {
             off = align_up(off, 1024);
             L.op0.push_back(take(mma_operand_bytes(n, path == CS_PATH_MMA4, 0)));
             off = align_up(off, 1024);
@@ -442,7 +548,7 @@ extern "C" {
 
 size_t cs_batch_workspace_bytes(const cs_set_desc* sets, int n_sets, int path) {
     if (!batch_valid(sets, n_sets) || path < CS_PATH_AUTO || path > CS_PATH_MMA4) return 0;
-    return batch_layout(sets, n_sets, batch_path(sets, n_sets, path)).total;
+    return batch_layout(sets, n_sets, batch_path(sets, n_sets, path), path == CS_PATH_AUTO).total;
 }
 
 int64_t cs_batch_hist_len(const cs_set_desc* sets, int n_sets) {
@@ -462,7 +568,8 @@ int cs_batch_create(const cs_set_desc* sets, int n_sets, int path, void* workspa
         return CS_EINVAL;
     const int p = batch_path(sets, n_sets, path);
     if (tensor_path(p) && !device_has_tcgen05()) return CS_EUNSUPPORTED;
-    const Layout L = batch_layout(sets, n_sets, p);
+    const bool auto_path = path == CS_PATH_AUTO;
+    const Layout L = batch_layout(sets, n_sets, p, auto_path);
     if (workspace_bytes < L.total) return CS_ENOMEM;
     const uint64_t* ds_thr = nullptr;
     for (int s = 0; s < n_sets && !ds_thr; ++s)
@@ -472,6 +579,8 @@ int cs_batch_create(const cs_set_desc* sets, int n_sets, int path, void* workspa
 
     std::vector<BatchSet> bs(static_cast<size_t>(n_sets));
     int64_t elem = 0, rblk = 0, mblk = 0, hoff = 0, tiles = 0;
+    int64_t ord_blocks = 0, ord_tasks = 0, ord_nmax = 0;
+    std::vector<int32_t> otab, osets;
     int max_pow2 = 1;
     for (int s = 0; s < n_sets; ++s) {
         BatchSet& b = bs[s];
@@ -479,8 +588,25 @@ int cs_batch_create(const cs_set_desc* sets, int n_sets, int path, void* workspa
         b.dim = cs_dim(b.kind);
         b.n = sets[s].n;
         b.seed = sets[s].seed;
-        b.coords = reinterpret_cast<int32_t*>(ws + L.coords[s]);
-        b.bits = reinterpret_cast<uint64_t*>(ws + L.bits[s]);
+        const bool order = set_by_order(sets[s], auto_path);
+        b.coords = order ? nullptr : reinterpret_cast<int32_t*>(ws + L.coords[s]);
+        b.bits = order ? nullptr : reinterpret_cast<uint64_t*>(ws + L.bits[s]);
+        b.order = OrderSet{};
+        if (order) {
+            b.order.p = reinterpret_cast<int32_t*>(ws + L.ord_p[s]);
+            b.order.q = reinterpret_cast<int32_t*>(ws + L.ord_q[s]);
+            b.order.R = reinterpret_cast<int32_t*>(ws + L.ord_r[s]);
+            b.order.D = reinterpret_cast<uint2*>(ws + L.ord_d[s]);
+            b.order.n = int32_t(b.n);
+            b.order.W = order_words(b.n);
+            b.ord_block = ord_blocks;
+            b.ord_task = ord_tasks;
+            ord_blocks += order_build_blocks(b.n);
+            ord_tasks += order_tasks(b.n, kBatchOrderM);
+            ord_nmax = b.n > ord_nmax ? b.n : ord_nmax;
+            otab.insert(otab.end(), size_t(order_build_blocks(b.n)), int32_t(s));
+            osets.push_back(int32_t(s));
+        }
         b.row_words = cs_row_words(b.n);
         b.key0 = reinterpret_cast<uint64_t*>(ws + L.key0[s]);
         b.key1 = reinterpret_cast<uint64_t*>(ws + L.key1[s]);
@@ -488,10 +614,10 @@ int cs_batch_create(const cs_set_desc* sets, int n_sets, int path, void* workspa
         b.ctab = L.ctab[s] ? reinterpret_cast<ConeTable*>(ws + L.ctab[s]) : nullptr;
         b.elem_begin = elem;
         elem += b.n;
-        b.vwords = (b.n + 63) / 64;
+        b.vwords = order ? 0 : (b.n + 63) / 64;  // a product order has no bitset: no tiles, no blocks
         b.rblock_begin = rblk;
         rblk += chunk_sum(b.vwords);
-        b.mir_side = ((b.n + 63) / 64 + kMirTiles - 1) / kMirTiles;
+        b.mir_side = (b.vwords + kMirTiles - 1) / kMirTiles;
         b.mblock_begin = mblk;
         b.tile_begin = tiles;
         tiles += b.vwords;
@@ -532,6 +658,7 @@ int cs_batch_create(const cs_set_desc* sets, int n_sets, int path, void* workspa
     std::vector<MmaSetEntry> me;
     for (int r = 0; r < n_sets; ++r) {
         const BatchSet& b = bs[order[r]];
+        if (by_order(b)) continue;
         if (tensor_path(p)) {
             // FP4 pairs count in supertiles, FP8 in 128-row tiles
             const bool fp4 = p == CS_PATH_MMA4;
@@ -546,7 +673,7 @@ int cs_batch_create(const cs_set_desc* sets, int n_sets, int path, void* workspa
             e.hist_off = b.hist_off * 8;
             e.chunk_begin = chunks;
             chunks += mma_expand_chunks(b.n);
-            etab.insert(etab.end(), size_t(mma_expand_chunks(b.n)), int32_t(r));  // entry r of the table
+            etab.insert(etab.end(), size_t(mma_expand_chunks(b.n)), int32_t(me.size()));  // its entry of the table
             me.push_back(e);
         } else {
             PopcSetEntry e;
@@ -576,7 +703,15 @@ int cs_batch_create(const cs_set_desc* sets, int n_sets, int path, void* workspa
     h->sets_dev = reinterpret_cast<BatchSet*>(ws + L.sets);
     h->total_elems = elem;
     h->total_rblocks = rblk;
-    for (int s = 0; s < n_sets; ++s) h->geoms |= 1u << batch_geom(sets[s].kind);
+    for (int s = 0; s < n_sets; ++s)
+        if (!by_order(bs[s])) h->geoms |= 1u << batch_geom(sets[s].kind);
+    h->n_order = int(osets.size());
+    h->n_general = n_sets - h->n_order;
+    h->otab = reinterpret_cast<int32_t*>(ws + L.otab);
+    h->osets = reinterpret_cast<int32_t*>(ws + L.osets);
+    h->ord_blocks = ord_blocks;
+    h->ord_tasks = ord_tasks;
+    h->ord_nmax = ord_nmax;
     h->total_items = items;
     h->total_chunks = chunks;
     h->rtab = reinterpret_cast<int32_t*>(ws + L.rtab);
@@ -613,15 +748,19 @@ int cs_batch_create(const cs_set_desc* sets, int n_sets, int path, void* workspa
         e = cudaMemcpyAsync(h->mtab, mtab.data(), mtab.size() * 4, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess && !ttab.empty())
         e = cudaMemcpyAsync(h->ttab, ttab.data(), ttab.size() * 4, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess && !otab.empty())
+        e = cudaMemcpyAsync(h->otab, otab.data(), otab.size() * 4, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess && !osets.empty())
+        e = cudaMemcpyAsync(h->osets, osets.data(), osets.size() * 4, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess && !etab.empty())
         e = cudaMemcpyAsync(h->etab, etab.data(), etab.size() * 4, cudaMemcpyHostToDevice, st);
     if (tensor_path(p)) {
         h->mma_dev = reinterpret_cast<MmaSetEntry*>(ws + L.entries);
-        if (e == cudaSuccess)
+        if (e == cudaSuccess && !me.empty())
             e = cudaMemcpyAsync(h->mma_dev, me.data(), sizeof(MmaSetEntry) * me.size(), cudaMemcpyHostToDevice, st);
     } else {
         h->popc_dev = reinterpret_cast<PopcSetEntry*>(ws + L.entries);
-        if (e == cudaSuccess)
+        if (e == cudaSuccess && !pe.empty())
             e = cudaMemcpyAsync(h->popc_dev, pe.data(), sizeof(PopcSetEntry) * pe.size(), cudaMemcpyHostToDevice, st);
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // the host tables go out of scope
@@ -673,6 +812,15 @@ int cs_batch_launch(const cs_batch* b, const double* eps_host, int n_eps, int64_
         g_cone_attr[dev] = true;
     }
     k_batch_rank<<<unsigned(b->nsets), kRankThreads, rank_smem, st>>>(b->sets_dev);
+    if (b->n_order > 0) {
+        k_batch_order_table<<<unsigned(b->ord_blocks), kOrdBuildThreads, 0, st>>>(b->sets_dev, b->otab);
+        // at most 16 x 256 bytes of stages and 8192 bins: below the 48 KB any launch may take
+        const int64_t grid = (b->ord_tasks + 15) / 16 < int64_t(sms) * 2 ? (b->ord_tasks + 15) / 16 : int64_t(sms) * 2;
+        k_batch_order_count<<<unsigned(grid), kBatchOrderThreads,
+                              kBatchOrderThreads * sizeof(int2) + size_t(b->ord_nmax) * 4, st>>>(
+            b->sets_dev, b->osets, b->n_order, b->ord_tasks, hist_dev);
+        if ((err = cudaGetLastError()) != cudaSuccess) return CS_ECUDA;
+    }
     if (b->geoms & (1u << kGeomLightCone))
         k_batch_ctab<<<unsigned((b->total_tiles * 32 + 255) / 256), 256, 0, st>>>(b->sets_dev, b->ttab,
                                                                                  b->total_tiles);
@@ -693,20 +841,23 @@ int cs_batch_launch(const cs_batch* b, const double* eps_host, int n_eps, int64_
         k_batch_relate<kGeomDeSitter><<<unsigned(b->geo_count[kGeomDeSitter]), kRelThreads, 0, st>>>(
             b->sets_dev, b->rtab, range(kGeomDeSitter));
     if (b->total_mblocks > int64_t(0x7fffffff)) return CS_EINVAL;
-    k_batch_mirror<<<unsigned(b->total_mblocks), kRelThreads, 0, st>>>(b->sets_dev, b->mtab);
+    if (b->total_mblocks > 0)
+        k_batch_mirror<<<unsigned(b->total_mblocks), kRelThreads, 0, st>>>(b->sets_dev, b->mtab);
     if ((err = cudaGetLastError()) != cudaSuccess) return CS_ECUDA;
 
-    if (b->path == CS_PATH_MMA) {
+    if (b->n_general == 0) {
+        err = cudaSuccess;
+    } else if (b->path == CS_PATH_MMA) {
         if ((err = launch_expand_multi(b->mma_dev, b->etab, b->total_chunks, st)) != cudaSuccess) return CS_ECUDA;
-        err = launch_count_mma_multi(b->mma_dev, b->nsets, b->total_items, reinterpret_cast<uintptr_t>(hist_dev),
+        err = launch_count_mma_multi(b->mma_dev, b->n_general, b->total_items, reinterpret_cast<uintptr_t>(hist_dev),
                                      b->hdr, 0, st);
     } else if (b->path == CS_PATH_MMA4) {
         if ((err = launch_expand_multi(b->mma_dev, b->etab, b->total_chunks, st, true)) != cudaSuccess)
             return CS_ECUDA;
-        err = launch_count_mma4_multi(b->mma_dev, b->nsets, b->total_items, reinterpret_cast<uintptr_t>(hist_dev),
+        err = launch_count_mma4_multi(b->mma_dev, b->n_general, b->total_items, reinterpret_cast<uintptr_t>(hist_dev),
                                       b->hdr, st);
     } else {
-        err = launch_count_popc_multi(b->popc_dev, b->nsets, b->total_items, reinterpret_cast<uintptr_t>(hist_dev),
+        err = launch_count_popc_multi(b->popc_dev, b->n_general, b->total_items, reinterpret_cast<uintptr_t>(hist_dev),
                                       b->hdr, 0, st);
     }
     if (err != cudaSuccess) return CS_ECUDA;

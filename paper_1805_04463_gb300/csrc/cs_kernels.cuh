@@ -143,6 +143,14 @@ cudaError_t launch_count_mma4(int64_t n, const uint64_t* bits, int64_t row_words
                               void* workspace, size_t ws_bytes, cudaStream_t st, const double* phi = nullptr,
                               double* layer = nullptr, int kmax = -1);
 
+// cs_order.cu: the count of product orders (2D orders, the 1+1 diamond and
+// square) from their coordinates.  order_workspace_bytes(n) of workspace.
+bool order_kind(int kind);
+bool order_count_fits(int kind, int64_t n);
+size_t order_workspace_bytes(int64_t n);
+cudaError_t launch_count_order(int kind, int64_t n, const int32_t* coords, int64_t* hist, void* workspace,
+                               cudaStream_t st);
+
 // CS_OK for cudaSuccess; otherwise CS_ECUDA, remembering the error for
 // cs_last_cuda_error (per host thread).
 int cuda_status(cudaError_t e);

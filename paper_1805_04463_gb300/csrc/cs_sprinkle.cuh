@@ -126,8 +126,10 @@ __device__ __forceinline__ uint64_t draw_2d_cylinder(uint64_t s, int64_t e, int3
 // sort of the (key, index) pairs, O(n log^2 n), took 0.38 ms for the
 // 768-set ensemble.)  sk holds the keys on entry, written before a barrier or
 // by their own threads (key i by thread i % kRankThreads).  All kRankThreads
-// threads; rank[e] receives the rank.
+// threads; rank[e] receives the rank.  kLastFirst: equal keys rank the later
+// element first.
 constexpr int kRankThreads = 1024;
+template <bool kLastFirst = false>
 __device__ __forceinline__ void rank_keys_smem(int n, int lgP, const uint64_t* sk, uint32_t* cnt, uint32_t* slot,
                                                uint32_t* rank) {
     const int P = 1 << lgP, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -177,7 +179,7 @@ __device__ __forceinline__ void rank_keys_smem(int n, int lgP, const uint64_t* s
         for (uint32_t q = s0; q < s1; ++q) {
             const uint32_t f = slot[q];
             const uint64_t kf = sk[f];
-            r += (kf < ke) || (kf == ke && f < uint32_t(i));
+            r += (kf < ke) || (kf == ke && (kLastFirst ? f > uint32_t(i) : f < uint32_t(i)));
         }
         rank[i] = r;
     }
