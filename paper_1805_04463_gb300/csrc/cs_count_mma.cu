@@ -71,7 +71,7 @@ constexpr uint32_t kIdesc4 = idesc_mxf4_f32(kBM, kBN);
 constexpr uint32_t kSfCol = 256;         // FP4: scale factors of A at this TMEM column, of B 16 further
 constexpr uint32_t kScaleOne = 0x7F7F7F7Fu;  // four UE8M0 scale factors 2^0 = 1
 constexpr int kRing = 4;                 // items in flight between the roles
-constexpr int kBarrierBytes = 512;       // mbarriers, item ring, TMEM address, abort flag
+constexpr int kBarrierBytes = 512;       // mbarriers, item ring, TMEM address, abort flag, spare histogram bin
 constexpr uint8_t kOne = 0x38;           // 1.0 in FP8 E4M3
 
 // Operand formats.  A stage holds one 128-byte swizzle row of K per operand
@@ -82,11 +82,9 @@ constexpr uint8_t kOne = 0x38;           // 1.0 in FP8 E4M3
 //          with every scale factor 1, so products are again 0 or 1; one
 //          accumulator, because the scale factors take TMEM columns too --
 //          the epilogue copies it to registers and releases it at once.
-// kLayers: the kernel may add d'Alembertian layer sums (kmax >= 0);
-// kSmallSet: it has the branch-free epilogue for sets whose histogram fits
-// in shared memory.  The FP4 kernel holds 64 accumulator values per thread
-// and needs every register for them, so it comes in two builds: counts only
-// (the large sets it is for) and counts with layer sums.
+// kLayers: the kernel may add d'Alembertian layer sums (kmax >= 0).  The FP4
+// kernel holds 64 accumulator values per thread and needs every register for
+// them, so it comes in two builds: counts only and counts with layer sums.
 // kPair: a CTA pair (a cluster of two) runs each 256 x 256 supertile as one
 // 2-SM MMA (tcgen05 cta_group::2, M = 256): CTA r loads A rows 128r.. and B
 // rows 128r.. of the supertile into its own shared memory, rank 0 issues
@@ -106,26 +104,23 @@ constexpr uint8_t kOne = 0x38;           // 1.0 in FP8 E4M3
 struct FmtF8 {
     static constexpr int kKE = kBK;      // K elements per stage
     static constexpr int kAcc = 2;
-    static constexpr bool kLayers = true, kSmallSet = true, kPair = false;
+    static constexpr bool kLayers = true, kPair = false;
     static constexpr int kStages = 4, kHistBins = 8192;
 };
 struct FmtF4 {
     static constexpr int kKE = 2 * kBK;
     static constexpr int kAcc = 1;
-    static constexpr bool kLayers = false, kSmallSet = false, kPair = true;
+    static constexpr bool kLayers = false, kPair = true;
     static constexpr int kStages = 6, kHistBins = 8192;
 };
 struct FmtF4Layers : FmtF4 {
     static constexpr bool kLayers = true;
 };
 // The multi-set form: its sets are small (a batch holds n <= 8192, a count
-// job any n), so it keeps the branch-free histogram of the FP8 kernel for
-// sets whose histogram fits in shared memory.  Its tiles hold few K-blocks
-// (4-6 at n = 4096), and five stages suit them best: a 768-set batch of
+// job any n), its tiles hold few K-blocks (4-6 at n = 4096), and five stages suit them best: a 768-set batch of
 // n ~ 2048-4096 replayed in 8.43 ms with 5, 8.45 with 4, 8.59 with 6,
 // 8.80 with 3 and 9.27 with 2.
 struct FmtF4Multi : FmtF4 {
-    static constexpr bool kSmallSet = true;
     static constexpr int kStages = 5;
 };
 // Bytes of one operand stage in each CTA, and the dynamic shared memory of
@@ -159,20 +154,22 @@ struct Item {
 };
 
 // Slot t of a set's item list -> supertile (si, sj) and its 128-row half;
-// false for a slot that holds no work.
+// false for a slot that holds no work.  A set of 2^22 elements has fewer than
+// 2^29 slots, so the divisions are 32-bit ones (the 64-bit ones by a runtime
+// R took most of a microsecond in the scheduler's one thread).
 __host__ __device__ __forceinline__ bool decode_slot(int64_t t, int64_t nsb, int64_t n, int64_t R, int64_t& si, int64_t& sj,
                                             int64_t& half) {
-    const int64_t spb = 2 * R * R;  // slots per raster block
-    const int64_t blk = t / spb, slot = t - blk * spb;
-    const int64_t nbg = (nsb + R - 1) / R;
-    int64_t m = int64_t((1.0f + sqrtf(1.0f + 8.0f * float(blk))) * 0.5f);  // corrected below
+    const uint32_t r = uint32_t(R), spb = 2 * r * r;  // slots per raster block
+    const uint32_t blk = uint32_t(t) / spb, slot = uint32_t(t) - blk * spb;
+    const uint32_t nbg = (uint32_t(nsb) + r - 1) / r;
+    uint32_t m = uint32_t((1.0f + sqrtf(1.0f + 8.0f * float(blk))) * 0.5f);  // corrected below
     while (m * (m - 1) / 2 > blk) --m;
     while (m * (m + 1) / 2 <= blk) ++m;
-    const int64_t gi = blk - m * (m - 1) / 2;
-    const int64_t gj = gi + (nbg - m);
-    si = gi * R + slot / (2 * R);
-    const int64_t rem = slot % (2 * R);
-    sj = gj * R + rem / 2;
+    const uint32_t gi = blk - m * (m - 1) / 2;
+    const uint32_t gj = gi + (nbg - m);
+    const uint32_t row = slot / (2 * r), rem = slot - row * 2 * r;
+    si = gi * r + row;
+    sj = gj * r + rem / 2;
     half = rem & 1;
     return si <= sj && sj < nsb && si * 256 + half * kBM < n;
 }
@@ -199,13 +196,13 @@ __host__ __device__ __forceinline__ bool decode_band(int64_t t, const MmaBand& b
         sj += b.i0;
         return true;
     }
-    const int64_t spb = 2 * R * R;
-    const int64_t blk = t / spb, slot = t - blk * spb;
-    const int64_t nbj = (b.nj + R - 1) / R;
-    const int64_t gi = blk / nbj, gj = blk - gi * nbj;
-    si = gi * R + slot / (2 * R);
-    const int64_t rem = slot % (2 * R);
-    sj = gj * R + rem / 2;
+    const uint32_t r = uint32_t(R), spb = 2 * r * r;
+    const uint32_t blk = uint32_t(t) / spb, slot = uint32_t(t) - blk * spb;
+    const uint32_t nbj = (uint32_t(b.nj) + r - 1) / r;
+    const uint32_t gi = blk / nbj, gj = blk - gi * nbj;
+    const uint32_t row = slot / (2 * r), rem = slot - row * 2 * r;
+    si = gi * r + row;
+    sj = gj * r + rem / 2;
     half = rem & 1;
     if (si >= b.ni || sj >= b.nj) return false;
     si += b.i0;
@@ -441,9 +438,11 @@ struct MmaSingle {
     int64_t nitems;
     __device__ __forceinline__ int64_t total() const { return nitems; }
     __device__ __forceinline__ int64_t chunk() const { return 1; }
-    __device__ __forceinline__ int set_of(int64_t t, int64_t& local, int) const {
-        local = t;
-        return 0;
+    // Unit t (slot `slots` * t of the list): its set and its supertile.
+    __device__ __forceinline__ bool decode(int64_t t, int slots, int& set, int64_t& si, int64_t& sj,
+                                           int64_t& half) const {
+        set = 0;
+        return decode_band(t * slots, v.band, v.n, v.raster, si, sj, half);
     }
     __device__ __forceinline__ MmaView view(int) const { return v; }
 };
@@ -460,26 +459,30 @@ struct MmaMulti {
     int64_t run;
     __device__ __forceinline__ int64_t total() const { return nitems; }
     __device__ __forceinline__ int64_t chunk() const { return run; }
-    // The set holding item t: the hint (the previous item's set) or the next
-    // set when t is still there, else a binary search.
-    __device__ __forceinline__ int set_of(int64_t t, int64_t& local, int hint) const {
-        int lo = -1;
-        if (hint >= 0 && sets[hint].item_begin <= t) {
-            if (hint + 1 == nsets || t < sets[hint + 1].item_begin)
-                lo = hint;
-            else if (hint + 2 == nsets || t < sets[hint + 2].item_begin)
-                lo = hint + 1;
-        }
-        if (lo < 0) {
-            int a = 0, b = nsets - 1;  // last set with item_begin <= t
-            while (a < b) {
-                const int mid = (a + b + 1) >> 1;
-                if (sets[mid].item_begin <= t) a = mid; else b = mid - 1;
+    // Unit t of the concatenated list: its set and its supertile.  All lanes
+    // of a warp, t ascending over the lanes from t0 = lane 0's; set carries
+    // the last step's set (any value at first).
+    __device__ __forceinline__ bool decode(int64_t t, int slots, int& set, int64_t& si, int64_t& sj,
+                                           int64_t& half) const {
+        const int lane = threadIdx.x & 31;
+        const int64_t t0 = __shfl_sync(0xffffffffu, t, 0);
+        int s = __shfl_sync(0xffffffffu, set, 0);
+        const bool near = s >= 0 && sets[s].item_begin <= t0 && (s + 2 >= nsets || t0 < sets[s + 2].item_begin);
+        if (!near) {  // uniform: 32 probes a step for the last set that begins at or before t0
+            s = 0;
+            for (int n = nsets; n > 1;) {
+                const int step = (n + 31) / 32;
+                const bool le = lane * step < n && sets[s + lane * step].item_begin <= t0;
+                const int hit = 31 - __clz(int(__ballot_sync(0xffffffffu, le)));  // lane 0 always holds
+                s += hit * step;
+                n = min(step, n - hit * step);
             }
-            lo = a;
         }
-        local = t - sets[lo].item_begin + sets[lo].item_offset;
-        return lo;
+        while (s + 1 < nsets && sets[s + 1].item_begin <= t) ++s;  // a run spans few sets
+        set = s;
+        const MmaSetEntry& e = sets[s];
+        const int64_t local = t - e.item_begin + e.item_offset;
+        return decode_slot(local * slots, e.nsb, e.n, kRasterDefault, si, sj, half);
     }
     __device__ __forceinline__ MmaView view(int s) const {
         const MmaSetEntry& e = sets[s];
@@ -542,7 +545,8 @@ __device__ __forceinline__ void mma_body(const Src& src, WsHeader* hdr) {
     volatile int64_t* ring = reinterpret_cast<volatile int64_t*>(done + 1);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(const_cast<int64_t*>(ring) + kRing);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-    static_assert((2 * kNS + 6 + 2 * kRing) * 8 + kRing * 8 + 8 <= kBarrierBytes, "barriers fit their area");
+    uint32_t* spare = tmem_slot + 2;
+    static_assert((2 * kNS + 6 + 2 * kRing) * 8 + kRing * 8 + 16 <= kBarrierBytes, "barriers fit their area");
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int64_t total = src.total();
@@ -622,6 +626,19 @@ __device__ __forceinline__ void mma_body(const Src& src, WsHeader* hdr) {
         else
             mbar_arrive(&iempty[slot]);
     };
+    // The scheduler's side: entry e into ring slot q % kRing of both CTAs once
+    // its consumers have released it.
+    auto publish = [&](uint32_t q, int64_t e) {
+        const uint32_t slot = q % kRing, use = (q / kRing) & 1u;
+        if (!mbar_wait_or_abort<kPair>(&iempty[slot], use ^ 1u, hdr, abort_flag)) return false;
+        ring[slot] = e;
+        mbar_arrive(&ifull[slot]);
+        if constexpr (kPair) {
+            st_cluster_s64(cluster_map(const_cast<int64_t*>(&ring[slot]), 1), e);
+            mbar_arrive_cluster(cluster_map(&ifull[slot], 1), 1u);
+        }
+        return true;
+    };
     // This CTA's first A row and B row within an item.
     const int64_t row_off = kPair ? int64_t(crank) * kBM : 0;
 
@@ -685,46 +702,42 @@ __device__ __forceinline__ void mma_body(const Src& src, WsHeader* hdr) {
                 if (++s == kNS) { s = 0; ph ^= 1u; }
             }
         }
-    } else if (warp == kSchedWarp && lane == 0 && leader) {
+    } else if (warp == kSchedWarp && leader) {
         // ---------------------------------------------------- scheduler
-        // Pulls units from the global queue (consecutive indices are
+        // Pulls runs of units from the global queue (consecutive indices are
         // raster-local, so the CTAs running at any moment share operand
-        // panels in L2), skips the units that hold no work, and publishes
-        // the others decoded.
-        int cur = -1;
-        MmaView v{};
-        int64_t next = 0, end = 0;  // the current run of units from the queue
+        // panels in L2), decodes up to 32 of them at once, one per lane, and
+        // publishes those that hold work.  (One thread decoding one unit at
+        // a time took about 2 us per unit; a set of three supertile rows has
+        // 64 units and 6 with work, and the pair waited 40 us between sets.)
         const int64_t units = total / kCl;
-        for (uint32_t q = 0;; ++q) {
-            const uint32_t slot = q % kRing, use = (q / kRing) & 1u;
-            if (!mbar_wait_or_abort<kPair>(&iempty[slot], use ^ 1u, hdr, abort_flag)) break;
-            int64_t e = -1;
-            for (;;) {
-                if (next >= end) {
-                    next = int64_t(atomicAdd(&hdr->counter, 1ull)) * src.chunk();
-                    end = next + src.chunk();
+        const int64_t chunk = src.chunk();
+        int set = -1;
+        uint32_t q = 0;
+        for (bool more = true; more;) {
+            int64_t next = 0;
+            if (lane == 0) next = int64_t(atomicAdd(&hdr->counter, 1ull)) * chunk;
+            next = __shfl_sync(0xffffffffu, next, 0);
+            const int64_t end = next + chunk < units ? next + chunk : units;
+            if (next >= units) break;
+            for (; next < end && more; next += 32) {
+                const int64_t t = next + lane;
+                int64_t si = 0, sj = 0, half = 0;
+                // lanes past the run repeat its last unit and drop it
+                const bool work = src.decode(t < end ? t : end - 1, kCl, set, si, sj, half) && t < end;
+                const int64_t e = pack_item(set, si, sj, half);
+                for (uint32_t todo = __ballot_sync(0xffffffffu, work); todo && more; todo &= todo - 1u) {
+                    const int64_t item = __shfl_sync(0xffffffffu, e, __ffs(int(todo)) - 1);
+                    bool ok = true;
+                    if (lane == 0) ok = publish(q, item);
+                    more = __shfl_sync(0xffffffffu, int(ok), 0) != 0;
+                    ++q;
                 }
-                const int64_t t = next++;
-                if (t >= units) break;
-                int64_t lu, si, sj, half;
-                const int sidx = src.set_of(t, lu, cur);
-                if (sidx != cur) {
-                    cur = sidx;
-                    v = src.view(sidx);
-                }
-                if (decode_band(lu * kCl, v.band, v.n, v.raster, si, sj, half)) {
-                    e = pack_item(sidx, si, sj, half);
-                    break;
-                }
+                set = __shfl_sync(0xffffffffu, set, 31);
             }
-            ring[slot] = e;
-            mbar_arrive(&ifull[slot]);
-            if constexpr (kPair) {
-                st_cluster_s64(cluster_map(const_cast<int64_t*>(&ring[slot]), 1), e);
-                mbar_arrive_cluster(cluster_map(&ifull[slot], 1), 1u);
-            }
-            if (e < 0) break;
+            if (!more) break;
         }
+        if (lane == 0) publish(q, -1);
     } else if (warp == 1 && lane == 0 && leader) {
         // ---------------------------------------------------- MMA issuer
         // (a pair: rank 0's, for both CTAs)
@@ -793,6 +806,7 @@ __device__ __forceinline__ void mma_body(const Src& src, WsHeader* hdr) {
         const int c0 = ((warp - 2) >> 2) * kEpiChunks;  // first of its 32-column chunks
         const int etid = tid - 64;
         const uint32_t shist_s = smem_u32(shist);
+        const uint32_t spare_s = smem_u32(spare);  // the bin of the lanes with nothing to count
         int64_t local_count = 0;
         int64_t since_flush = 0;  // tiles counted into the shared histogram since its last flush
         int cur = -1;
@@ -864,11 +878,12 @@ __device__ __forceinline__ void mma_body(const Src& src, WsHeader* hdr) {
             static_assert(kEpiChunks == 2, "one bitset word per epilogue warp");
             const int64_t word0 = (it.J0 + 32 * c0) >> 6;
             const uint64_t cw = (i < v.n && word0 < v.row_words) ? __ldg(v.bits + i * v.row_words + word0) : 0ull;
+            double phi_i = 1.0;  // row i's share of the layer sums
+            if constexpr (Fmt::kLayers) {
+                if (v.kmax >= 0 && v.phi && i < v.n) phi_i = __ldg(v.phi + i);
+            }
             if (!mbar_wait_or_abort<kPair>(&tfull[buf], use, hdr, abort_flag)) { ok = false; break; }
             tc_fence_after();
-            // Every count of this set lands in the shared histogram and there
-            // are no layer sums: the common case, kept branch-free.
-            const bool simple = v.kmax < 0 && v.hist_len <= kHistBins;
             // Histogram the 32 counts r of chunk c (columns J0 + 32c ..); index
             // arithmetic in 32 bits (n <= 2^22).
             const int ii = int(i), nn = int(v.n), hb32 = int(hb);
@@ -880,41 +895,41 @@ __device__ __forceinline__ void mma_body(const Src& src, WsHeader* hdr) {
                 m &= lo <= 0 ? ~0u : (lo >= 32 ? 0u : (~0u << lo));
                 const int hi = nn - jb;      // u < hi keeps j < n
                 m &= hi >= 32 ? ~0u : (hi <= 0 ? 0u : ((1u << hi) - 1u));
-                if (m == 0u) return;
+                // Every lane takes every step (red_shared_one: an add by
+                // part of a warp is twice as slow), to the spare bin where
+                // it has nothing to count; a chunk without any pair is skipped.
+                if (__ballot_sync(0xffffffffu, m != 0u) == 0u) return;
                 // counts are integers below 2^23: adding 2^23 puts k in the
                 // low mantissa bits, exactly
-                if (Fmt::kSmallSet && simple) {
+                auto bin = [&](uint32_t v) {
+                    return 4u * __float_as_uint(__uint_as_float(v) + 8388608.0f) + (shist_s - 4u * 0x4B000000u);
+                };
+                // Counts past the shared bins are looked for only where the
+                // tile's columns reach that far past its rows, and then by
+                // the chunk's largest count (entries without a pair are 0).
+                bool wide = int(it.J0) + kBN - 2 - int(it.I0) >= hb32;
+                if (wide) {
+                    float top = 0.0f;
 #pragma unroll
-                    for (int u = 0; u < 32; ++u)
-                        if ((m >> u) & 1u)
-                            red_shared_add(shist_s + 4u * (__float_as_uint(__uint_as_float(r[u]) + 8388608.0f) - 0x4B000000u), 1u);
+                    for (int u = 0; u < 32; ++u) top = fmaxf(top, __uint_as_float(r[u]));
+                    wide = __any_sync(0xffffffffu, top >= float(hb32));
+                }
+                if (!wide && (!Fmt::kLayers || v.kmax < 0)) {
+#pragma unroll
+                    for (int u = 0; u < 32; ++u) red_shared_one((m >> u) & 1u ? bin(r[u]) : spare_s);
                     return;
                 }
-                if constexpr (Fmt::kLayers) {
-                    if (v.kmax >= 0) {
-#pragma unroll
-                        for (int u = 0; u < 32; ++u) {
-                            if ((m >> u) & 1u) {
-                                const int k = int(__float_as_uint(__uint_as_float(r[u]) + 8388608.0f) - 0x4B000000u);
-                                if (k < hb32)
-                                    red_shared_add(shist_s + 4u * uint32_t(k), 1u);
-                                else
-                                    atomicAdd(&v.hist[k], 1ull);
-                                if (k <= v.kmax)  // i is in L_{k+1}(j)
-                                    atomicAdd(&v.layer[int64_t(k) * nn + jb + u], v.phi ? __ldg(v.phi + i) : 1.0);
-                            }
-                        }
-                        return;
-                    }
-                }
+                const uint32_t past = shist_s + 4u * uint32_t(hb32);  // address past the last shared bin
 #pragma unroll
                 for (int u = 0; u < 32; ++u) {
-                    if ((m >> u) & 1u) {
-                        const int k = int(__float_as_uint(__uint_as_float(r[u]) + 8388608.0f) - 0x4B000000u);
-                        if (k < hb32)
-                            red_shared_add(shist_s + 4u * uint32_t(k), 1u);
-                        else
-                            atomicAdd(&v.hist[k], 1ull);
+                    const uint32_t at = bin(r[u]);
+                    const bool on = (m >> u) & 1u;
+                    red_shared_one(on && at < past ? at : spare_s);
+                    if (on && at >= past) atomicAdd(&v.hist[(at - shist_s) >> 2], 1ull);
+                    if constexpr (Fmt::kLayers) {
+                        const uint32_t k = (at - shist_s) >> 2;
+                        if (on && int(k) <= v.kmax)  // i is in L_{k+1}(j)
+                            atomicAdd(&v.layer[k * uint32_t(nn) + uint32_t(jb + u)], phi_i);
                     }
                 }
             };

@@ -79,6 +79,17 @@ __device__ __forceinline__ void red_shared_add(uint32_t saddr, uint32_t v) {
     asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(saddr), "r"(v) : "memory");
 }
 
+// Add 1 to a shared histogram bin, by all 32 lanes of the warp: a lane with
+// nothing to count passes the address of a spare bin that nobody reads.
+// Measured on GB300 (32 warps, random bins): an add by part of a warp takes
+// 4.2 cycles of the SM however few its lanes are, one of the constant 1 by
+// all 32 lanes 2.3 to 2.8, lanes at one address counting as one -- with half the
+// lanes counting 6.9 pairs per SM and cycle instead of 3.8, with a tenth 1.4
+// instead of 0.8.
+__device__ __forceinline__ void red_shared_one(uint32_t saddr) {
+    asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(saddr) : "memory");
+}
+
 __device__ __forceinline__ unsigned long long global_timer_ns() {
     unsigned long long t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));

@@ -207,18 +207,12 @@ __device__ __forceinline__ void order_decode(int64_t t, int m, int& A, int& C) {
     A = int(t - m * (c * (c + 1) / 2));
 }
 
-// Shared-memory histogram adds on GB300 (measured, 32 warps of random bins):
-// an add by some of a warp's lanes takes 4.2 cycles of the SM however few
-// they are; an add of the constant 1 by all 32 lanes takes 2.3 to 2.8, and
-// lanes at one address count as one.  So every lane adds, the lanes with
-// nothing to count to one spare bin that nobody reads: 6.9 counted pairs per
-// SM and cycle instead of 3.8 at half the lanes counting.
-
 // One column of 64 pairs: lane l's rows 2 l and 2 l + 1 of the band against
 // column (pb, xb).  With c = #{rows a <= 2 l of the band : p_a < pb} (row
 // 2 l + 1 counts itself too; that one is in its y from the start),
 //   at = y + xb - 4 c;  a related row adds 1 at [at], the other ones
-//   (p > pb) lower their y by 4 and add to the spare bin.
+//   (p > pb) lower their y by 4 and add to the spare bin (red_shared_one:
+//   every lane adds, and the constant 1).
 // le / lt: the lanes at or before / before this one.
 struct OrderRows {
     int p0, p1;
@@ -289,8 +283,8 @@ __device__ __forceinline__ void order_column_wide(OrderRows& r, int pb, int xb, 
     const uint32_t c = __popc(__ballot_sync(0xffffffffu, p) & r.le) + __popc(__ballot_sync(0xffffffffu, q) & r.lt);
     const uint32_t t = r.y0 + uint32_t(xb) - 4u * c, u = r.y1 + uint32_t(xb) - 4u * c;
     const bool cp = p && row < own, cq = q && row + 1 < own;
-    red_shared_add(cp && t < spare ? t : spare, 1u);
-    red_shared_add(cq && u < spare ? u : spare, 1u);
+    red_shared_one(cp && t < spare ? t : spare);
+    red_shared_one(cq && u < spare ? u : spare);
     if (cp && t >= spare) atomicAdd(hist_g + ((t - hist_s) >> 2), 1ull);
     if (cq && u >= spare) atomicAdd(hist_g + ((u - hist_s) >> 2), 1ull);
     if (pb < r.p0) r.y0 -= 4u;
