@@ -223,14 +223,19 @@ __global__ void __launch_bounds__(kBatchOrderThreads, 2) k_batch_order_count(con
 }
 
 // Relate chunks.  Row tile rb of a set with V valid words needs words
-// [rb, V) (the words before it are mirrored); they are covered by
-// ceil((V - rb) / 32) chunks of 32 words starting at the diagonal word, so
-// no block holds words before its row tile or whole groups of padding.
-// chunk_sum(x) = sum_{m=1..x} ceil(m / 32); the chunks of row tiles < rb
-// number chunk_sum(V) - chunk_sum(V - rb).
-__host__ __device__ __forceinline__ int64_t chunk_sum(int64_t x) {
-    const int64_t a = x / kRelWordsPerBlock, b = x % kRelWordsPerBlock;
-    return kRelWordsPerBlock * a * (a + 1) / 2 + b * (a + 1);
+// [rb, V) (the words before it are mirrored); they are covered by chunks of
+// 32 words from word 4 floor(rb / 4) on (a warp's words are one 32-byte
+// sector of a row), so no block holds whole groups of padding.  In units of four words,
+// V4 = ceil(V / 4), row tile rb has ceil((V4 - rb / 4) / 8) chunks.
+// chunk_sum8(x) = sum_{m=1..x} ceil(m / 8).
+__host__ __device__ __forceinline__ int64_t chunk_sum8(int64_t x) {
+    const int64_t a = x / 8, b = x % 8;
+    return 8 * a * (a + 1) / 2 + b * (a + 1);
+}
+// Chunks of the row tiles before rb; of all of them for rb = V.
+__host__ __device__ __forceinline__ int64_t chunks_before(int64_t V, int64_t rb) {
+    const int64_t V4 = (V + 3) / 4, g = rb / 4, left = V4 - g;
+    return 4 * (chunk_sum8(V4) - chunk_sum8(left)) + (rb & 3) * ((left + 7) / 8);
 }
 
 // Relation geometry of a kind.
@@ -245,14 +250,14 @@ __host__ __device__ __forceinline__ int batch_geom(int kind) {
 // row tile's last chunk, the first padding word to zero (else -1).
 __device__ __forceinline__ void decode_rblock(const BatchSet& b, int64_t local, int64_t& rb, int64_t& w0,
                                               int64_t& zero_from) {
-    const int64_t V = b.vwords, total = chunk_sum(V);
+    const int64_t V = b.vwords;
     int64_t lo = 0, hi = V - 1;  // last row tile whose first chunk is at or before `local`
     while (lo < hi) {
         const int64_t mid = (lo + hi + 1) >> 1;
-        if (total - chunk_sum(V - mid) <= local) lo = mid; else hi = mid - 1;
+        if (chunks_before(V, mid) <= local) lo = mid; else hi = mid - 1;
     }
     rb = lo;
-    w0 = rb + (local - (total - chunk_sum(V - rb))) * kRelWordsPerBlock;
+    w0 = (rb & ~int64_t(3)) + (local - chunks_before(V, rb)) * kRelWordsPerBlock;
     zero_from = w0 + kRelWordsPerBlock >= V ? w0 + kRelWordsPerBlock : -1;
 }
 
@@ -264,17 +269,16 @@ __device__ __forceinline__ void decode_rblock(const BatchSet& b, int64_t local, 
 // the registers it needs for itself.  Block x of a geometry's launch: relate block order[x] (the launch's slice
 // of the blocks grouped by geometry), of set rblock_set[order[x]].
 template <int G>
-__global__ void __launch_bounds__(kRelThreads, 5) k_batch_relate(const BatchSet* __restrict__ sets,
+__global__ void __launch_bounds__(kRelThreads) k_batch_relate(const BatchSet* __restrict__ sets,
                                                               const int32_t* __restrict__ rblock_set,
                                                               const int32_t* __restrict__ order) {
-    __shared__ __align__(16) int32_t sc[kStageInts];
+    __shared__ __align__(16) uint8_t sm[relate_stage_bytes(G)];
     const int64_t blk = order[blockIdx.x];
     const BatchSet& b = sets[rblock_set[blk]];
     if (batch_geom(b.kind) != G) return;  // never, by the order's construction
     int64_t rb, w0, zero_from;
     decode_rblock(b, blk - b.rblock_begin, rb, w0, zero_from);
-    relate_block<G>(b.coords, b.n, b.bits, b.row_words, rb, w0, sc, G == kGeomLightCone && b.kind == CS_2D_ORDER,
-                    zero_from);
+    relate_block<G>(b.coords, b.n, b.bits, b.row_words, rb, w0, sm, zero_from);
 }
 
 // The light-cone kinds, from the column tables k_batch_rank built (one
@@ -492,7 +496,7 @@ Layout batch_layout(const cs_set_desc* sets, int n_sets, int path, bool auto_pat
             oblocks += order_build_blocks(n);
             continue;
         }
-        rblocks += chunk_sum((n + 63) / 64);
+        rblocks += chunks_before((n + 63) / 64, (n + 63) / 64);
         tiles += (n + 63) / 64;
         const int64_t side = ((n + 63) / 64 + kMirTiles - 1) / kMirTiles;
         mblocks += side * side;
@@ -616,7 +620,7 @@ int cs_batch_create(const cs_set_desc* sets, int n_sets, int path, void* workspa
         elem += b.n;
         b.vwords = order ? 0 : (b.n + 63) / 64;  // a product order has no bitset: no tiles, no blocks
         b.rblock_begin = rblk;
-        rblk += chunk_sum(b.vwords);
+        rblk += chunks_before(b.vwords, b.vwords);
         b.mir_side = (b.vwords + kMirTiles - 1) / kMirTiles;
         b.mblock_begin = mblk;
         b.tile_begin = tiles;
@@ -639,7 +643,7 @@ int cs_batch_create(const cs_set_desc* sets, int n_sets, int path, void* workspa
         std::fill(mtab.begin() + bs[s].mblock_begin, mtab.begin() + bs[s].mblock_begin + bs[s].mir_side * bs[s].mir_side,
                   int32_t(s));
     for (int s = 0; s < n_sets; ++s)
-        std::fill(rtab.begin() + bs[s].rblock_begin, rtab.begin() + bs[s].rblock_begin + chunk_sum(bs[s].vwords),
+        std::fill(rtab.begin() + bs[s].rblock_begin, rtab.begin() + bs[s].rblock_begin + chunks_before(bs[s].vwords, bs[s].vwords),
                   int32_t(s));
     // the relate blocks grouped by geometry, so that each geometry's launch
     // covers only its own blocks (blocks of the other geometries returning at
@@ -651,7 +655,7 @@ int cs_batch_create(const cs_set_desc* sets, int n_sets, int path, void* workspa
         geo_begin[g] = int64_t(rorder.size());
         for (int s = 0; s < n_sets; ++s)
             if (batch_geom(bs[s].kind) == g)
-                for (int64_t k = 0; k < chunk_sum(bs[s].vwords); ++k) rorder.push_back(int32_t(bs[s].rblock_begin + k));
+                for (int64_t k = 0; k < chunks_before(bs[s].vwords, bs[s].vwords); ++k) rorder.push_back(int32_t(bs[s].rblock_begin + k));
         geo_count[g] = int64_t(rorder.size()) - geo_begin[g];
     }
     std::vector<PopcSetEntry> pe;

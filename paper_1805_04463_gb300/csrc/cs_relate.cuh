@@ -10,139 +10,121 @@ constexpr int kRelColsPerBlock = 2048;
 constexpr int kRelWordsPerBlock = kRelColsPerBlock / 64;
 constexpr int kRelRowsPerBlock = 64;
 constexpr int kRelThreads = 256;
+constexpr int kRelWarpWords = kRelWordsPerBlock / (kRelThreads / 32);  // words of one warp: a 32-byte sector
+static_assert(kRelWarpWords == 4, "a warp's words of a row are one sector");
 
 // Geometries of the relation test; the number of coordinates is geom_dim(G).
-constexpr int kGeomLightCone = 2, kGeom3 = 3, kGeom4 = 4, kGeomDeSitter = 5;
-constexpr int geom_dim(int g) { return g == kGeomDeSitter ? 2 : g; }
+// kGeomOrder: a random 2D order labelled by u (u increases with the label).
+constexpr int kGeomLightCone = 2, kGeom3 = 3, kGeom4 = 4, kGeomDeSitter = 5, kGeomOrder = 6;
+constexpr int geom_dim(int g) { return g == kGeom3 || g == kGeom4 ? g : 2; }
 
-// Symmetric timelike test between row element ci and staged column `col`:
-// du * dv > 0 (1+1, light-cone coordinates), dt^2 - |dx|^2 > 0 (2+1, 3+1)
-// exact in int64, or, on a circle (the de Sitter slab's conformal grid, Eq.
-// ds_metric, and the 1+1 cylinder), the angular separation below the
-// (conformal-)time separation.
+// Symmetric timelike test between elements i and j (coordinates a, b): du * dv > 0 (1+1,
+// light-cone coordinates), dt^2 - |dx|^2 > 0 (2+1, 3+1) exact in int64, or,
+// on a circle (the de Sitter slab's conformal grid, Eq. ds_metric, and the
+// 1+1 cylinder), the angular separation below the (conformal-)time
+// separation.
 template <int G>
-__device__ __forceinline__ bool rel_related(const int32_t (&ci)[geom_dim(G)], const int32_t (*sc)[kRelColsPerBlock],
-                                            int col) {
+__device__ __forceinline__ bool rel_related(const int32_t (&a)[geom_dim(G)], const int32_t (&b)[geom_dim(G)],
+                                            int64_t i, int64_t j) {
     if constexpr (G == kGeomDeSitter) {
         // |eta| < 2^30 (slab: < 2^29, cylinder: < 2^31 / pi), so de fits
         // int32; theta differences wrap modulo 2^32, one full turn.
-        const int32_t de = sc[0][col] - ci[0];
-        const uint32_t d = uint32_t(sc[1][col]) - uint32_t(ci[1]);
+        const int32_t de = b[0] - a[0];
+        const uint32_t d = uint32_t(b[1]) - uint32_t(a[1]);
         const uint32_t circ = min(d, 0u - d);
         return circ < uint32_t(abs(de));
     } else if constexpr (G == kGeomLightCone) {
         // du * dv > 0 as a sign test (|du|, |dv| < 2^31 fit int32)
-        const int32_t du = sc[0][col] - ci[0];
-        const int32_t dv = sc[1][col] - ci[1];
+        const int32_t du = b[0] - a[0];
+        const int32_t dv = b[1] - a[1];
         return (du ^ dv) >= 0 && du != 0 && dv != 0;
+    } else if constexpr (G == kGeomOrder) {
+        return j > i ? b[1] > a[1] : (j < i && b[1] < a[1]);
     } else {
         // |coordinates| < 2^29: differences fit int32 and each square is one
         // widening multiply-add into the int64 sum (< 2^62, exact)
-        const int32_t dt = sc[0][col] - ci[0];
+        const int32_t dt = b[0] - a[0];
         int64_t s2 = int64_t(dt) * dt;
 #pragma unroll
         for (int d = 1; d < G; ++d) {
-            const int32_t dx = sc[d][col] - ci[d];
+            const int32_t dx = b[d] - a[d];
             s2 -= int64_t(dx) * dx;
         }
         return s2 > 0;
     }
 }
 
+// A word of the matrix, exactly, by a whole warp: lane l holds columns
+// 64 W + l and 64 W + l + 32, two ballots fold the tests of a row.  Columns
+// at or beyond n are 0.
+template <int G>
+struct ExactWord {
+    static constexpr int D = geom_dim(G);
+    int32_t b[2][D];
+    int64_t j0;
+    bool in[2];
+    __device__ __forceinline__ ExactWord(const int32_t* __restrict__ coords, int64_t n, int64_t W) {
+        j0 = 64 * W + (threadIdx.x & 31);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            in[k] = j0 + 32 * k < n;
+#pragma unroll
+            for (int d = 0; d < D; ++d) b[k][d] = in[k] ? __ldg(coords + d * n + j0 + 32 * k) : 0;
+        }
+    }
+    __device__ __forceinline__ uint64_t row(const int32_t* __restrict__ coords, int64_t n, int64_t i) const {
+        int32_t a[D];
+#pragma unroll
+        for (int d = 0; d < D; ++d) a[d] = __ldg(coords + d * n + i);
+        const uint32_t lo = __ballot_sync(0xffffffffu, in[0] && rel_related<G>(a, b[0], i, j0));
+        const uint32_t hi = __ballot_sync(0xffffffffu, in[1] && rel_related<G>(a, b[1], i, j0 + 32));
+        return (uint64_t(hi) << 32) | lo;
+    }
+};
+
 // FP32 filter for the 2+1 and 3+1 tests.  With every coordinate in
-// [-kFilterRange, kFilterRange] = [-2^20, 2^20] the coordinates and their
-// differences (|d| <= 2^21) are exact in FP32, every partial result of
-// dt^2 - dx^2 - ... is below 2^44 in magnitude, so each of the (at most
-// five) roundings is at most 2^20 and the FP32 value lies within
-// kFilterSlack = 2^23 of the exact one: above it the pair is related, below
-// its negative it is not, and only in between the exact int64 test runs.
+// [-kFilterRange, kFilterRange] = [-2^20, 2^20],
+//   s = 2^23 - (dt^2 - |dx|^2) = A_j + B_i + 2 t_i t_j - 2 x_i . x_j,
+//   B = |x|^2 - t^2, A = B + 2^23,
+// one add and D fused multiply-adds per pair.  A and B are off by less than
+// 2^18.6 each (every square is below 2^40, the sum below 2^42); A + B and the
+// partial sums stay below 2^43.8, so the add rounds by at most 2^18, the first
+// multiply-add by 2^18 and the others by 2^19: the value lies within 2^22 of
+// the exact one.  Negative means s2 > 2^23 - 2^22 > 0 (related), above 2^24
+// means s2 < 0, and only a value in [0, 2^24] needs the exact test (about one
+// word in a thousand holds one).
 constexpr int32_t kFilterRange = 1 << 20;
 constexpr float kFilterSlack = 8388608.0f;  // 2^23
-
-// s2 = dt^2 - dx^2 - dy^2 (- dz^2) in FP32 between a row (rc) and a staged
-// column x = (t, x, y, z), z = 0 in 2+1; the same chain of roundings
-// everywhere, so that every test of a pair decides alike.
-template <int DIM>
-__device__ __forceinline__ float filter_s2(const float (&rc)[4], float4 x) {
-    const float dt = x.x - rc[0];
-    float s2 = dt * dt;
-    const float dx = x.y - rc[1];
-    s2 = fmaf(-dx, dx, s2);
-    const float dy = x.z - rc[2];
-    s2 = fmaf(-dy, dy, s2);
-    if constexpr (DIM == 4) {
-        const float dz = x.w - rc[3];
-        s2 = fmaf(-dz, dz, s2);
-    }
-    return s2;
-}
-
-// The lane-per-word form's chain: 2^23 - s2 = 2^23 - dt^2 + dx^2 + dy^2
-// (+ dz^2), each square added by one fused multiply-add.  Every partial
-// result is below 2^44 in magnitude, so each of the (at most four) roundings
-// is at most 2^20 and the value lies within 2^22 of the exact one: negative
-// means s2 > 2^23 - 2^22 > 0 (related), above 2^24 means s2 < 0, and only
-// [0, 2^24] needs the exact test.
-template <int DIM>
-__device__ __forceinline__ float filter_offset(const float (&rc)[4], float4 x) {
-    const float dt = x.x - rc[0];
-    float s = fmaf(-dt, dt, kFilterSlack);
-    const float dx = x.y - rc[1];
-    s = fmaf(dx, dx, s);
-    const float dy = x.z - rc[2];
-    s = fmaf(dy, dy, s);
-    if constexpr (DIM == 4) {
-        const float dz = x.w - rc[3];
-        s = fmaf(dz, dz, s);
-    }
-    return s;
-}
 // Bits of the float 2^24: a value in [+0, 2^24] has bits at most this as an
 // unsigned integer, and every negative value (sign bit set) has more.
 constexpr uint32_t kBandBits = 0x4B800000u;
 
-// The exact int64 test on the same (integral) coordinates.
-template <int DIM>
-__device__ __forceinline__ bool exact_related(const float (&rc)[4], float4 x) {
-    const int32_t dt = int32_t(x.x) - int32_t(rc[0]), dx = int32_t(x.y) - int32_t(rc[1]),
-                  dy = int32_t(x.z) - int32_t(rc[2]), dz = int32_t(x.w) - int32_t(rc[3]);
-    int64_t e2 = int64_t(dt) * dt - int64_t(dx) * dx - int64_t(dy) * dy;
-    if constexpr (DIM == 4) e2 -= int64_t(dz) * dz;
-    return e2 > 0;
+// |x|^2 - t^2 in FP32.
+template <int D>
+__device__ __forceinline__ float filter_norm(const int32_t (&c)[D]) {
+    const float t = float(c[0]);
+    float s = -t * t;
+#pragma unroll
+    for (int d = 1; d < D; ++d) s = fmaf(float(c[d]), float(c[d]), s);
+    return s;
 }
 
-// The filtered test: the FP32 sign outside the band, the exact one inside.
-template <int DIM>
-__device__ __forceinline__ bool rel_filtered(const float (&rc)[4], float4 x) {
-    const float s2 = filter_s2<DIM>(rc, x);
-    if (s2 > kFilterSlack) return true;
-    if (s2 < -kFilterSlack) return false;
-    return exact_related<DIM>(rc, x);
+// Two FP32 values side by side, each operation rounded like the scalar one.
+__device__ __forceinline__ uint64_t f2_pack(float lo, float hi) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
 }
-
-// Light-cone kinds.  Labels are in time order, so in a word wholly after
-// the row tile only the future cone can hold (u_j > u_i and v_j > v_i); for
-// a random 2D order labelled by u the u test is implied by j > i and only v
-// is compared (USE_U = false).  Each lane owns one word (64 columns) of the
-// block and tests its columns one by one, for four rows at a time, with no
-// ballots.  Coordinates lie in [0, 2^31), so x_j - x_i - 1 fits int32 and is
-// non-negative iff x_j > x_i: a test is one or two integer multiply-adds
-// (x_j * 1 + ~x_i, on the FMA pipe, the multiplier a runtime 1 so that the
-// compiler keeps the multiply-add), an OR of the two with u, and a funnel
-// shift that appends the sign bit to the half-word's accumulator; the
-// accumulated sign bits are the complement of the relation bits.  The
-// compare-and-OR form it replaces kept the integer ALU pipe saturated.
-// The column coordinates are staged transposed, st[c][w] = column 64 w + c
-// (row pitch kConePitch: the lanes' reads of one offset c hit consecutive
-// banks); columns at or beyond n are staged as 0, which no cone test
-// passes.  The row tile's own word (lane ws) takes the full symmetric test
-// by ballots; words before the row tile are left to mirror_block.
-constexpr int kConePitch = kRelWordsPerBlock + 1;  // staged words per column offset
-constexpr int kConeRows = 4;                        // rows a lane tests together
-constexpr int kStageInts = 4 * kRelColsPerBlock;    // staging ints any geometry needs
-constexpr int kConeOne = 2 * 64 * kConePitch;       // after the (u, v) staging: a runtime 1 (the multiplier)
-constexpr int kConeInts = kConeOne + 1;             // staging ints of the light-cone kinds
-static_assert(kStageInts >= kConeInts, "the transposed (u, v) staging and the 1 fit");
+__device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
 
 // x * one + y as a multiply-add (one is 1 at run time).
 __device__ __forceinline__ int32_t cone_mad(int32_t x, int32_t one, int32_t y) {
@@ -151,337 +133,318 @@ __device__ __forceinline__ int32_t cone_mad(int32_t x, int32_t one, int32_t y) {
     return d;
 }
 
-// Lane `lane` stores word w0 + lane of row i (words before the row tile are
-// mirror_block's), and, when zero_from >= 0, zeroes word zero_from + lane
-// (padding words past the last chunk of a row, fewer than 32).
-__device__ __forceinline__ void store_row_words(uint64_t* __restrict__ bits, int64_t i, int64_t row_words, int64_t w0,
-                                                int lane, int wbeg, uint64_t word, int64_t zero_from) {
-    if (lane >= wbeg && w0 + lane < row_words) bits[i * row_words + w0 + lane] = word;
-    if (zero_from >= 0 && zero_from + lane < row_words) bits[i * row_words + zero_from + lane] = 0ull;
+// |d| - (ej - ei) modulo 2^32.
+__device__ __forceinline__ int32_t circle_gap(int32_t d, int32_t ei, int32_t ej) {
+    uint32_t a;
+    asm("abs.s32 %0, %1;" : "=r"(a) : "r"(d));  // 2^31 for d = -2^31
+    return int32_t(a + uint32_t(ei) - uint32_t(ej));
 }
 
-// The lane layout of the lane-per-word forms: W words from w0 (a power of
-// two, at most 32, the fewest covering the chunk's valid words), lane l
-// testing word l % W for the rows of row group l / W.  A chunk at the end of
-// a row with few valid words then keeps its lanes busy on more rows instead
-// of on words past the row's end.
-__device__ __forceinline__ int lane_words(int64_t valid) {
-    int W = 1;
-    while (W < valid && W < kRelWordsPerBlock) W <<= 1;
-    return W;
+// Staged bytes per column: u and v (light cone, circle), v alone (2D order),
+// the coordinates and A (filtered 2+1, 3+1).
+__host__ __device__ constexpr int relate_stage_bytes(int g) {
+    return kRelColsPerBlock * (g == kGeomOrder                              ? 4
+                               : g == kGeomLightCone || g == kGeomDeSitter ? 8
+                               : g == kGeom3                               ? 16
+                                                                           : 20) +
+           16;  // and a runtime 1 (the multiplier)
 }
 
-// Per row of the block, all lanes of a warp: the row tile's own word when
-// ws >= 0 (own(i, k): the relation of row i with column offset k of word ws,
-// folded by two ballots) and the zero padding words [z0, z1) of the row.
-template <class Own>
-__device__ __forceinline__ void own_words_and_padding(uint64_t* __restrict__ bits, int64_t row_words, int64_t w0,
-                                                      int64_t r0, int64_t r1, int ws, int64_t z0, int64_t z1,
-                                                      Own own) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    constexpr int kWarps = kRelThreads / 32;
-    if (ws < 0 && z0 >= z1) return;
-    for (int64_t i = r0 + warp; i < r1; i += kWarps) {
-        if (ws >= 0) {
-            const bool b0 = own(i, lane), b1 = own(i, lane + 32);
-            const uint64_t d = (uint64_t(__ballot_sync(0xffffffffu, b1)) << 32) | __ballot_sync(0xffffffffu, b0);
-            if (lane == 0) bits[i * row_words + w0 + ws] = d;
-        }
-        for (int64_t w = z0 + lane; w < z1; w += 32) bits[i * row_words + w] = 0ull;
-    }
+// A row as the tests see it: light cone ~u and ~v; circle eta and -theta;
+// filtered 2+1 and 3+1 the multipliers (2 t, -2 x, ..) and B, each twice.
+template <int G>
+struct RelRow {
+    int32_t nu, nv;
+};
+template <>
+struct RelRow<kGeom3> {
+    uint64_t k[3], b;
+};
+template <>
+struct RelRow<kGeom4> {
+    uint64_t k[4], b;
+};
+
+// acc shifted left by one, x's sign bit shifted in.
+__device__ __forceinline__ uint32_t push_sign(uint32_t x, uint32_t acc) {
+    uint32_t r;
+    asm("shf.l.wrap.b32 %0, %1, %2, 1;" : "=r"(r) : "r"(x), "r"(acc));
+    return r;
 }
 
-template <bool USE_U>
-__device__ __forceinline__ void relate_rows_cone(const int32_t* __restrict__ coords, int64_t n,
-                                                 uint64_t* __restrict__ bits, int64_t row_words, int64_t w0,
-                                                 int64_t c0, int64_t r0, int64_t r1, int ws,
-                                                 const int32_t* __restrict__ st, int64_t zero_from) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    constexpr int kWarps = kRelThreads / 32;
-    const int2* st2 = reinterpret_cast<const int2*>(st);  // USE_U: (u, v) pairs
-    const int wbeg = ws > 0 ? ws : 0;
-    const int32_t one = st[kConeOne];
-    for (int64_t ib = r0 + int64_t(warp) * kConeRows; ib < r1; ib += int64_t(kWarps) * kConeRows) {
-        int32_t ru[kConeRows], rv[kConeRows], nu[kConeRows], nv[kConeRows];
-        uint32_t lo[kConeRows], hi[kConeRows];
+// The sign bits of a lane's two rows against the 64 staged columns from pair
+// pbase on: acc[row][half], and (2+1, 3+1) the unsigned minimum of the
+// filter's bits.  kOwn: the row tile's own word, where column lane (+ 32 for
+// the second row) is the row itself, whose value lies in the band and is left
+// out of the minimum.
+template <int G, bool kOwn>
+__device__ __forceinline__ void relate_word(const uint8_t* __restrict__ smem, int pbase, const RelRow<G> (&row)[2],
+                                            int32_t one, uint32_t (&acc)[2][2], uint32_t (&band)[2]) {
+    constexpr bool kFilter = G == kGeom3 || G == kGeom4;
+    band[0] = band[1] = ~0u;
 #pragma unroll
-        for (int r = 0; r < kConeRows; ++r) {
-            const int64_t i = ib + r;
-            ru[r] = i < r1 ? coords[i] : INT32_MAX;  // a missing row passes no test
-            rv[r] = i < r1 ? coords[n + i] : INT32_MAX;
-            nu[r] = ~ru[r];  // -x_i - 1
-            nv[r] = ~rv[r];
-            lo[r] = hi[r] = 0u;
-        }
+    for (int h = 0; h < 2; ++h) {
+        uint32_t s0 = 0u, s1 = 0u;
+        // highest column first: after 32 shifts column 32 h is bit 0
+        if constexpr (kFilter) {
+            const ulonglong2* q0 = reinterpret_cast<const ulonglong2*>(smem) + pbase;
+            const ulonglong2* q1 = q0 + kRelColsPerBlock / 2;
+            const uint64_t* q2 = reinterpret_cast<const uint64_t*>(smem) + 2 * kRelColsPerBlock + pbase;
+#pragma unroll 4
+            for (int p = 16 * h + 15; p >= 16 * h; --p) {
+                const ulonglong2 tx = q0[p], yz = q1[p];
+                const uint64_t A = G == kGeom4 ? q2[p] : yz.y;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {  // the word's low and high halves
-            // highest column first: after 32 shifts column 32 h is bit 0
-#pragma unroll 8
-            for (int c = 32 * h + 31; c >= 32 * h; --c) {
-                int32_t xu = 0, xv;
-                if constexpr (USE_U) {
-                    const int2 x = st2[c * kConePitch + lane];
-                    xu = x.x;
-                    xv = x.y;
-                } else {
-                    xv = st[c * kConePitch + lane];
-                }
-#pragma unroll
-                for (int r = 0; r < kConeRows; ++r) {
-                    // sign bit set iff the column is not in the future cone
-                    const int32_t d = USE_U ? (cone_mad(xu, one, nu[r]) | cone_mad(xv, one, nv[r]))
-                                            : cone_mad(xv, one, nv[r]);
-                    if (h == 0) lo[r] = __funnelshift_l(uint32_t(d), lo[r], 1);
-                    else hi[r] = __funnelshift_l(uint32_t(d), hi[r], 1);
-                }
-            }
-        }
-#pragma unroll
-        for (int r = 0; r < kConeRows; ++r) {
-            const int64_t i = ib + r;
-            if (i >= r1) break;  // warp-uniform
-            uint64_t word = ~((uint64_t(hi[r]) << 32) | lo[r]);
-            if (ws >= 0) {  // the row tile's own word: full test (warp-uniform)
-                bool b[2];
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int k = lane + 32 * h;  // column offset in the word
-                    const int64_t j = c0 + int64_t(ws) * 64 + k;
-                    if constexpr (USE_U) {
-                        const int2 x = st2[k * kConePitch + ws];
-                        const int32_t du = x.x - ru[r], dv = x.y - rv[r];
-                        b[h] = j < n && (du ^ dv) >= 0 && du != 0 && dv != 0;
-                    } else {  // u increases with the label
-                        const int32_t xv = st[k * kConePitch + ws];
-                        b[h] = j < n && (j > i ? xv > rv[r] : (j < i && xv < rv[r]));
+                for (int r = 0; r < 2; ++r) {
+                    uint64_t s = f2_add(A, row[r].b);
+                    s = f2_fma(row[r].k[0], tx.x, s);
+                    s = f2_fma(row[r].k[1], tx.y, s);
+                    s = f2_fma(row[r].k[2], yz.x, s);
+                    if constexpr (G == kGeom4) s = f2_fma(row[r].k[geom_dim(G) - 1], yz.y, s);
+                    const uint32_t lo = uint32_t(s), hi = uint32_t(s >> 32);
+                    uint32_t& a = r == 0 ? s0 : s1;
+                    a = push_sign(hi, a);
+                    a = push_sign(lo, a);
+                    if constexpr (kOwn) {
+                        const int d = int(threadIdx.x & 31) + 32 * r - 2 * p;  // 0 or 1: this pair holds the row itself
+                        band[r] = min(band[r], min(d == 0 ? ~0u : lo, d == 1 ? ~0u : hi));
+                    } else {
+                        band[r] = min(band[r], min(lo, hi));
                     }
                 }
-                const uint64_t d = (uint64_t(__ballot_sync(0xffffffffu, b[1])) << 32) | __ballot_sync(0xffffffffu, b[0]);
-                if (lane == ws) word = d;
             }
-            store_row_words(bits, i, row_words, w0, lane, wbeg, word, zero_from);
-        }
-    }
-}
-
-// 2+1 and 3+1 with the FP32 filter, laid out like the light-cone kinds: each
-// lane owns one word and tests its 64 columns one by one against two rows
-// held in registers.  The columns are staged as float4 (t, x, y, z; z = 0 in
-// 2+1) at st4[c * 32 + (w ^ (c & 7))] for column 64 w + c of the block: one
-// 16-byte load per column and lane, conflict-free for the lanes' loads of
-// one offset c and for the staging stores of consecutive columns.  A test is
-// filter_offset's chain, a funnel shift of its sign (set: related) into the
-// half-word's accumulator and an unsigned minimum of its bits; a word whose
-// minimum shows a value in [0, 2^24] (near the light cone, about one word in
-// a thousand) is recomputed exactly by its lane.  Columns at or beyond n are
-// staged 10^9 units away in space (far outside the cone and the band) and
-// masked off.  The row tile's own word (lane ws, which holds the diagonal)
-// takes the filtered test by ballots; words before the row tile are left to
-// mirror_block.
-constexpr int kFiltRows = 2;  // rows a lane tests together (the 48-register budget of the batched kernel)
-
-template <int DIM>
-__device__ __forceinline__ void relate_rows_filtered(const int32_t* __restrict__ coords, int64_t n,
-                                                     uint64_t* __restrict__ bits, int64_t row_words, int64_t w0,
-                                                     int64_t c0, int64_t r0, int64_t r1, int ws, int W,
-                                                     const float4* __restrict__ st4) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    constexpr int kWarps = kRelThreads / 32;
-    const int wbeg = ws > 0 ? ws : 0;
-    const int wl = lane & (W - 1);                                   // this lane's word
-    const int64_t pass = int64_t(kFiltRows) * (kRelWordsPerBlock / W);  // rows of one warp pass
-    const int64_t g0 = int64_t(lane / W) * kFiltRows;                 // this lane's first row in a pass
-    // with W = 32 a pass's rows are the same in every lane, and the row
-    // tile's own word is folded by ballots right here; narrower layouts
-    // leave it to own_words_and_padding
-    const bool inline_own = W == kRelWordsPerBlock && ws >= 0;
-    const bool keep = wl >= wbeg && (wl != ws || inline_own) && w0 + wl < row_words;
-    const int64_t cw = c0 + 64 * int64_t(wl);  // this lane's first column
-    const uint64_t valid = cw >= n ? 0ull : (n - cw >= 64 ? ~0ull : (~0ull >> (64 - (n - cw))));
-    for (int64_t ib = r0 + int64_t(warp) * pass; ib < r1; ib += int64_t(kWarps) * pass) {
-        float rc[kFiltRows][4];
-        uint32_t lo[kFiltRows], hi[kFiltRows];
-        uint32_t band[kFiltRows];  // unsigned minimum of the chain's bits
+        } else if constexpr (G == kGeomOrder) {
+            const int4* q = reinterpret_cast<const int4*>(smem) + pbase / 2;  // four columns
 #pragma unroll
-        for (int r = 0; r < kFiltRows; ++r) {
-            const int64_t i = ib + g0 + r;
+            for (int p = 8 * h + 7; p >= 8 * h; --p) {
+                const int4 v = q[p];
 #pragma unroll
-            for (int d = 0; d < 4; ++d) rc[r][d] = (d < DIM && i < r1) ? float(coords[d * n + i]) : 0.0f;
-            lo[r] = hi[r] = 0u;
-            band[r] = ~0u;
-        }
+                for (int r = 0; r < 2; ++r) {
+                    uint32_t& a = r == 0 ? s0 : s1;
+                    a = push_sign(uint32_t(cone_mad(v.w, one, row[r].nv)), a);
+                    a = push_sign(uint32_t(cone_mad(v.z, one, row[r].nv)), a);
+                    a = push_sign(uint32_t(cone_mad(v.y, one, row[r].nv)), a);
+                    a = push_sign(uint32_t(cone_mad(v.x, one, row[r].nv)), a);
+                }
+            }
+        } else {
+            const int4* q = reinterpret_cast<const int4*>(smem) + pbase;  // two columns
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            // highest column first: after 32 shifts column 32 h is bit 0
-#pragma unroll 4
-            for (int c = 32 * h + 31; c >= 32 * h; --c) {
-                const float4 x = st4[c * 32 + (wl ^ (c & 7))];
+            for (int p = 16 * h + 15; p >= 16 * h; --p) {
+                const int4 x = q[p];
 #pragma unroll
-                for (int r = 0; r < kFiltRows; ++r) {
-                    const uint32_t sb = __float_as_uint(filter_offset<DIM>(rc[r], x));
-                    if (h == 0) lo[r] = __funnelshift_l(sb, lo[r], 1);
-                    else hi[r] = __funnelshift_l(sb, hi[r], 1);
-                    band[r] = min(band[r], sb);
+                for (int r = 0; r < 2; ++r) {
+                    int32_t d1 = cone_mad(x.w, one, row[r].nv), d0 = cone_mad(x.y, one, row[r].nv);
+                    if constexpr (G == kGeomDeSitter) {
+                        d1 = circle_gap(d1, row[r].nu, x.z);
+                        d0 = circle_gap(d0, row[r].nu, x.x);
+                    } else {
+                        d1 |= cone_mad(x.z, one, row[r].nu);
+                        d0 |= cone_mad(x.x, one, row[r].nu);
+                    }
+                    uint32_t& a = r == 0 ? s0 : s1;
+                    a = push_sign(uint32_t(d1), a);
+                    a = push_sign(uint32_t(d0), a);
                 }
             }
         }
-#pragma unroll
-        for (int r = 0; r < kFiltRows; ++r) {
-            const int64_t i = ib + g0 + r;
-            uint64_t word = ((uint64_t(hi[r]) << 32) | lo[r]) & valid;
-            if (keep && i < r1 && wl != ws && band[r] <= kBandBits) {  // near the light cone: the word exactly
-                word = 0ull;
-                for (int c = 0; c < 64 && cw + c < n; ++c)
-                    if (rel_filtered<DIM>(rc[r], st4[c * 32 + (wl ^ (c & 7))])) word |= 1ull << c;
-            }
-            if (inline_own) {
-                if (i >= r1) break;  // warp-uniform (g0 = 0)
-                bool b[2];
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int k = lane + 32 * h;  // column offset in the word
-                    b[h] = c0 + int64_t(ws) * 64 + k < n && rel_filtered<DIM>(rc[r], st4[k * 32 + (ws ^ (k & 7))]);
-                }
-                const uint64_t d = (uint64_t(__ballot_sync(0xffffffffu, b[1])) << 32) | __ballot_sync(0xffffffffu, b[0]);
-                if (lane == ws) word = d;
-            }
-            if (keep && i < r1) bits[i * row_words + w0 + wl] = word;
-        }
+        acc[0][h] = s0;
+        acc[1][h] = s1;
     }
 }
 
-// Rows [rb*64, rb*64+64) x words [w0, w0+32) of the bitset, less the
-// words wholly before the row tile (word < rb): the relation is symmetric,
-// so mirror_block fills those as transposes.  Column coordinates are staged
-// in shared memory `sc` (kStageInts ints, 16-byte aligned).  The light-cone
-// kinds test one cone per word (relate_rows_cone); order2d: the set is a
-// random 2D order whose coords[0] (u) increases strictly with the label,
-// which also drops the u test there.  The other geometries stage sc[d][col]
-// and each warp folds 64 tests per word into a uint64 with two
-// __ballot_sync, lane w keeps word w, and a row's words leave in one
-// coalesced store.  zero_from >= 0: the block also zeroes each row's words
-// [zero_from, row_words) (padding past a row's last chunk).  Must be called
-// by all 256 threads.
+// Rows [64 rb, 64 rb + 64) x words [w0, w0 + 32) of the bitset, less the words
+// before the row tile (word < rb): the relation is symmetric, so mirror_block
+// fills those as transposes.  w0 is a multiple of 4.  zero_from >= 0: the
+// block also zeroes each row's words [zero_from, row_words) (padding past a
+// row's last chunk).  smem: relate_stage_bytes(G), 16-byte aligned.  All 256
+// threads.
+//
+// A lane owns two rows (l and l + 32 of the tile) and a warp four words, so
+// that a row's words leave as one whole 32-byte sector, and every column's
+// values are read once by broadcast for 64 rows: with a lane per word instead
+// (32 lanes reading 32 different columns for two rows) the shared-memory
+// reads cost as much as the tests.  Labels are in time order, so a word after
+// the row tile needs only the future cone.  The words are built from sign
+// bits, funnel-shifted in one column at a time:
+//   light cone: x_j - x_i - 1 < 0 for u or v (coordinates in [0, 2^31): no
+//     overflow), one integer multiply-add each (x_j * 1 + ~x_i, the multiplier a runtime 1
+//     that keeps it on the FMA pipe; compares and ORs held the integer pipe);
+//   2D order: the same for v alone;
+//   circle: |dtheta| - deta < 0, dtheta modulo 2^32 in [-2^31, 2^31) and
+//     0 <= deta < 2^31: exact in 32 bits but where deta = 0 and |dtheta| = 2^31,
+//     so a word whose first column has the row's eta is found exactly;
+//   2+1, 3+1: the FP32 filter, two columns per packed operation, four
+//     instructions per test where differences and squares took ten; a word
+//     with a value near the cone is found exactly.
+// The integer tests' own word of the row tile (it holds the diagonal and both
+// cones) is found exactly; the filter is symmetric and takes it too.
 template <int G>
 __device__ __forceinline__ void relate_block(const int32_t* __restrict__ coords, int64_t n,
                                              uint64_t* __restrict__ bits, int64_t row_words, int64_t rb, int64_t w0,
-                                             int32_t* sc, bool order2d = false, int64_t zero_from = -1) {
-    constexpr int DIM = geom_dim(G);
-    const int64_t c0 = w0 * 64;
+                                             uint8_t* smem, int64_t zero_from = -1) {
+    constexpr int D = geom_dim(G);
+    constexpr bool kFilter = G == kGeom3 || G == kGeom4;
     if (w0 + kRelWordsPerBlock <= rb) return;  // wholly below the diagonal
-    // first word of the block at or after the row tile (< 0: all of them)
-    const int ws = rb - w0 < 0 ? -1 : int(rb - w0);
-    const int wbeg = ws > 0 ? ws : 0;
-    const int64_t r0 = rb * kRelRowsPerBlock;
-    const int64_t r1 = r0 + kRelRowsPerBlock < n ? r0 + kRelRowsPerBlock : n;
-    // The filtered 3+1 and 2+1 form tests W = lane_words(valid words) words
-    // from w0 and zeroes the row's words [w0 + W, z1) past them: the rest of
-    // the block's 32, and, at a row's last chunk (zero_from >= 0), the
-    // padding to row_words.  (The light-cone test, at a few instructions,
-    // gained less from narrow blocks than their fixed costs took, and keeps
-    // all 32 lanes on words.)
-    const int64_t z1 = zero_from >= 0 ? row_words : (w0 + kRelWordsPerBlock < row_words ? w0 + kRelWordsPerBlock
-                                                                                          : row_words);
-    auto pad_from = [&](int W) { return w0 + W < z1 ? w0 + W : z1; };
-    if constexpr (G == kGeomLightCone) {  // time order: one cone per word, see above
-        // transposed staging, word w of the block at row offset c: column 64 w + c
-        for (int t = threadIdx.x + 64 * wbeg; t < kRelColsPerBlock; t += kRelThreads) {
-            const int64_t col = c0 + t;
-            const int at = (t & 63) * kConePitch + (t >> 6);
-            if (order2d) {
-                sc[at] = col < n ? coords[n + col] : 0;
-            } else {
-                reinterpret_cast<int2*>(sc)[at] =
-                    col < n ? make_int2(coords[col], coords[n + col]) : make_int2(0, 0);
-            }
-        }
-        if (threadIdx.x == 0) sc[kConeOne] = 1;
-        __syncthreads();
-        if (order2d) relate_rows_cone<false>(coords, n, bits, row_words, w0, c0, r0, r1, ws, sc, zero_from);
-        else relate_rows_cone<true>(coords, n, bits, row_words, w0, c0, r0, r1, ws, sc, zero_from);
-    } else {
-        auto sd = reinterpret_cast<int32_t(*)[kRelColsPerBlock]>(sc);
-        // 2+1 and 3+1: when the block's columns and rows all lie within
-        // kFilterRange the columns are staged as floats for the FP32 filter.
-        constexpr bool kFilter = G == kGeom3 || G == kGeom4;
-        constexpr int kPer = kRelColsPerBlock / kRelThreads;  // staged columns per thread
-        int32_t v[kPer][DIM];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t V = (n + 63) >> 6;  // valid words
+    const int64_t c0 = w0 * 64, r0 = rb * kRelRowsPerBlock;
+    const int64_t wfirst = rb > w0 ? rb : w0;  // first word tested here
+    int32_t* one_s = reinterpret_cast<int32_t*>(smem + relate_stage_bytes(G) - 16);
+
+    // ---- stage the columns, two per thread and step
+    const int first = int(wfirst - w0) * 32;  // in column pairs
+    bool fast = true;
+    if constexpr (kFilter) {
         int out = 0;
+        ulonglong2* q0 = reinterpret_cast<ulonglong2*>(smem);      // (t, t), (x, x)
+        ulonglong2* q1 = q0 + kRelColsPerBlock / 2;                // (y, y), (z, z); 2+1: (y, y), (A, A)
+        uint64_t* q2 = reinterpret_cast<uint64_t*>(q1 + kRelColsPerBlock / 2);  // 3+1: (A, A)
+        for (int p = first + threadIdx.x; p < kRelColsPerBlock / 2; p += kRelThreads) {
+            int32_t c[2][D];
 #pragma unroll
-        for (int q = 0; q < kPer; ++q) {
-            const int t = threadIdx.x + q * kRelThreads;
-            const int64_t c = c0 + t;
+            for (int k = 0; k < 2; ++k)
 #pragma unroll
-            for (int d = 0; d < DIM; ++d) {
-                v[q][d] = (t >= 64 * wbeg && c < n) ? coords[d * n + c] : 0;
-                out |= v[q][d] < -kFilterRange || v[q][d] > kFilterRange;
+                for (int d = 0; d < D; ++d) {
+                    const int64_t j = c0 + 2 * p + k;
+                    c[k][d] = j < n ? __ldg(coords + d * n + j) : 0;
+                    out |= c[k][d] < -kFilterRange || c[k][d] > kFilterRange;
+                }
+            auto pair = [&](int d) { return f2_pack(float(c[0][d]), float(c[1][d])); };
+            const uint64_t A = f2_pack(filter_norm<D>(c[0]) + kFilterSlack, filter_norm<D>(c[1]) + kFilterSlack);
+            q0[p] = make_ulonglong2(pair(0), pair(1));
+            if constexpr (G == kGeom4) {
+                q1[p] = make_ulonglong2(pair(2), pair(3));
+                q2[p] = A;
+            } else {
+                q1[p] = make_ulonglong2(pair(2), A);
             }
         }
-        if (kFilter && threadIdx.x < r1 - r0) {
+        if (threadIdx.x < 64 && r0 + threadIdx.x < n) {
 #pragma unroll
-            for (int d = 0; d < DIM; ++d) {
-                const int32_t x = coords[d * n + r0 + threadIdx.x];
+            for (int d = 0; d < D; ++d) {
+                const int32_t x = __ldg(coords + d * n + r0 + threadIdx.x);
                 out |= x < -kFilterRange || x > kFilterRange;
             }
         }
-        const bool fast = kFilter && !__syncthreads_or(out);
-        if constexpr (kFilter) {
-            if (fast) {
-                float4* st4 = reinterpret_cast<float4*>(sc);
+        fast = !__syncthreads_or(out);
+    } else {
+        for (int p = first + threadIdx.x; p < kRelColsPerBlock / 2; p += kRelThreads) {
+            int32_t c[2][2];
 #pragma unroll
-                for (int q = 0; q < kPer; ++q) {
-                    const int t = threadIdx.x + q * kRelThreads;
-                    if (t < 64 * wbeg) continue;
-                    const int c = t & 63, w = t >> 6;
-                    float f[4] = {0.0f, 1e9f, 0.0f, 0.0f};  // a column at or beyond n: far away in space
-                    if (c0 + t < n) {
+            for (int k = 0; k < 2; ++k)
 #pragma unroll
-                        for (int d = 0; d < 4; ++d) f[d] = d < DIM ? float(v[q][d < DIM ? d : 0]) : 0.0f;
-                    }
-                    st4[c * 32 + (w ^ (c & 7))] = make_float4(f[0], f[1], f[2], f[3]);
+                for (int d = (G == kGeomOrder ? 1 : 0); d < 2; ++d) {
+                    const int64_t j = c0 + 2 * p + k;
+                    c[k][d] = j < n ? __ldg(coords + d * n + j) : 0;
                 }
-                __syncthreads();
-                // the row tile's own word (it holds the diagonal): the filtered test
-                auto own = [&](int64_t i, int k) {
-                    if (c0 + int64_t(ws) * 64 + k >= n) return false;
-                    float rc[4];
-#pragma unroll
-                    for (int d = 0; d < 4; ++d) rc[d] = d < DIM ? float(coords[d * n + i]) : 0.0f;
-                    return rel_filtered<DIM>(rc, st4[k * 32 + (ws ^ (k & 7))]);
-                };
-                const int W = lane_words((n + 63) / 64 - w0);
-                relate_rows_filtered<DIM>(coords, n, bits, row_words, w0, c0, r0, r1, ws, W, st4);
-                own_words_and_padding(bits, row_words, w0, r0, r1, W == kRelWordsPerBlock ? -1 : ws, pad_from(W), z1,
-                                      own);
-                return;
-            }
+            if constexpr (G == kGeomOrder)
+                reinterpret_cast<int2*>(smem)[p] = make_int2(c[0][1], c[1][1]);
+            else
+                reinterpret_cast<int4*>(smem)[p] = make_int4(c[0][0], c[0][1], c[1][0], c[1][1]);
         }
-#pragma unroll
-        for (int q = 0; q < kPer; ++q) {
-            const int t = threadIdx.x + q * kRelThreads;
-            if (t < 64 * wbeg) continue;
-#pragma unroll
-            for (int d = 0; d < DIM; ++d) sd[d][t] = v[q][d];
-        }
+        if (threadIdx.x == 0) *one_s = 1;
         __syncthreads();
-        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-        for (int64_t i = r0 + warp; i < r1; i += kRelThreads / 32) {
-            int32_t ci[DIM];
+    }
+
+    int32_t one = 1;
+    if constexpr (!kFilter) one = *one_s;
+    // ---- this lane's two rows
+    RelRow<G> row[2];
 #pragma unroll
-            for (int d = 0; d < DIM; ++d) ci[d] = coords[d * n + i];
-            uint64_t mine = 0;
-#pragma unroll 4
-            for (int w = wbeg; w < kRelWordsPerBlock; ++w) {
-                const int col = w * 64 + lane;
-                const bool b0 = c0 + col < n && rel_related<G>(ci, sd, col);
-                const bool b1 = c0 + col + 32 < n && rel_related<G>(ci, sd, col + 32);
-                const uint32_t lo = __ballot_sync(0xffffffffu, b0);
-                const uint32_t hi = __ballot_sync(0xffffffffu, b1);
-                if (lane == w) mine = (uint64_t(hi) << 32) | lo;
+    for (int r = 0; r < 2; ++r) {
+        const int64_t i = r0 + lane + 32 * r;
+        int32_t c[D];
+#pragma unroll
+        for (int d = 0; d < D; ++d) c[d] = i < n ? __ldg(coords + d * n + i) : 0;
+        if constexpr (kFilter) {
+#pragma unroll
+            for (int d = 0; d < D; ++d) {
+                const float k = (d == 0 ? 2.0f : -2.0f) * float(c[d]);
+                row[r].k[d] = f2_pack(k, k);
             }
-            store_row_words(bits, i, row_words, w0, lane, wbeg, mine, zero_from);
+            const float b = filter_norm<D>(c);
+            row[r].b = f2_pack(b, b);
+        } else if constexpr (G == kGeomDeSitter) {
+            row[r].nu = c[0];
+            row[r].nv = int32_t(0u - uint32_t(c[1]));
+        } else {
+            row[r].nu = ~c[0];
+            row[r].nv = ~c[1];
         }
     }
+    const int64_t wb = w0 + kRelWarpWords * warp;  // this warp's first word
+    if (wb + kRelWarpWords > rb && wb < row_words) {  // warp-uniform: some word at or after the row tile
+        // [word][row]; the words shift down as they are found, so that the loop
+        // is one copy of the tests (unrolled, the instruction cache missed)
+        uint64_t word[kRelWarpWords][2] = {};
+#pragma unroll 1
+        for (int k = 0; k < kRelWarpWords; ++k) {
+            const int64_t W = wb + k;
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+#pragma unroll
+                for (int x = 0; x + 1 < kRelWarpWords; ++x) word[x][r] = word[x + 1][r];
+                word[kRelWarpWords - 1][r] = 0ull;
+            }
+            uint64_t (&found)[2] = word[kRelWarpWords - 1];
+            if (W < rb || W >= V) continue;  // warp-uniform
+            // rows to find exactly: the own word of the integer tests, coordinates beyond the
+            // filter's range, and below the rows whose tests could not decide
+            bool exact[2] = {W == rb || !fast, W == rb || !fast};
+            if (kFilter ? fast : W != rb) {
+                const int pbase = int(W - w0) * 32;
+                uint32_t acc[2][2], band[2];
+                if (kFilter && W == rb)
+                    relate_word<G, true>(smem, pbase, row, one, acc, band);
+                else
+                    relate_word<G, false>(smem, pbase, row, one, acc, band);
+                const int64_t left = n - 64 * W;
+                const uint64_t valid = left >= 64 ? ~0ull : (1ull << left) - 1ull;
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    uint64_t x = (uint64_t(acc[r][1]) << 32) | acc[r][0];
+                    if constexpr (G == kGeomLightCone || G == kGeomOrder) x = ~x;  // sign set: not in the future cone
+                    found[r] = x & valid;
+                    if constexpr (kFilter) exact[r] = band[r] <= kBandBits;
+                    if constexpr (G == kGeomDeSitter) exact[r] = row[r].nu == __ldg(coords + 64 * W);
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                uint32_t todo = __ballot_sync(0xffffffffu, exact[r] && r0 + lane + 32 * r < n);
+                if (todo) {  // warp-uniform
+                    const ExactWord<G> ex(coords, n, W);
+#pragma unroll 2
+                    for (; todo; todo &= todo - 1u) {
+                        const int q = __ffs(int(todo)) - 1;
+                        const uint64_t y = ex.row(coords, n, r0 + 32 * r + q);
+                        if (lane == q) found[r] = y;
+                    }
+                }
+            }
+        }
+        // a row's four words as one 32-byte store; words before the row tile are mirror_block's
+        const bool whole = wb >= rb && (reinterpret_cast<uintptr_t>(bits) & 31) == 0;  // warp-uniform
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const int64_t i = r0 + lane + 32 * r;
+            if (i >= n) continue;
+            uint64_t* dst = bits + i * row_words + wb;
+            if (whole) {
+                asm volatile("st.global.v4.b64 [%0], {%1, %2, %3, %4};" ::"l"(dst), "l"(word[0][r]), "l"(word[1][r]),
+                             "l"(word[2][r]), "l"(word[3][r])
+                             : "memory");
+            } else {
+#pragma unroll
+                for (int k = 0; k < kRelWarpWords; ++k)
+                    if (wb + k >= rb) dst[k] = word[k][r];
+            }
+        }
+    }
+    if (zero_from >= 0 && zero_from < row_words)
+        for (int64_t i = r0 + warp; i < r0 + 64 && i < n; i += kRelThreads / 32)
+            for (int64_t w = zero_from + lane; w < row_words; w += 32) bits[i * row_words + w] = 0ull;
 }
 
 // ------------------------------------------------ light-cone column tables
@@ -581,8 +544,8 @@ __device__ __forceinline__ uint64_t cone_above(const int32_t* __restrict__ xs, c
 // tile's columns, the copy's mbarrier.
 constexpr int kConeTableSmem = kRelWordsPerBlock * int(sizeof(ConeTable)) + 128 * 4 + 16;
 
-// Rows [64 rb, 64 rb + 64) x words [w0, w0 + 32) (w0 >= rb) of a light-cone
-// set from its column tables (tables[C] for column tile C): the row tile's
+// Rows [64 rb, 64 rb + 64) x words [w0, w0 + 32) (less the words before rb) of
+// a light-cone set from its column tables (tables[C] for column tile C): the row tile's
 // own word rb by the exact symmetric test folded with ballots, every word
 // after it by the table look-ups, words at or past the last valid one zeroed
 // (and, with zero_from >= 0, the row's words [zero_from, row_words)).  The
@@ -604,7 +567,7 @@ __device__ __forceinline__ bool relate_block_tables(const int32_t* __restrict__ 
     const int64_t wt = w0 > rb ? w0 : rb + 1;                                      // first table word
     const int64_t we = w0 + kRelWordsPerBlock < V ? w0 + kRelWordsPerBlock : V;  // end of the valid words
     const int nt = wt < we ? int(we - wt) : 0;
-    const bool has_own = rb >= w0;  // then rb == w0: chunks start at the diagonal word
+    const bool has_own = rb >= w0;
     if (threadIdx.x == 0) {
         mbar_init(bar, 1);
         fence_mbar_init();
