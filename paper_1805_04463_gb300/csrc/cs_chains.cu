@@ -7,19 +7,22 @@
 // from peeling: the set S (A_ij for a pair, every element for the whole set)
 // loses all its minimal elements -- those with no predecessor left in S --
 // once per round; the number of rounds is the number of elements of the
-// longest chain in S.  A round is one warp per element of S testing
-// P_k & S over the words before k, then one block clearing the removed bits.
+// longest chain in S.  Each element remembers the word of its row that last
+// held a predecessor in S: S only shrinks, so the words nearer than it stay
+// empty, and over all rounds a row is scanned once.
 //
-// Greedy antichain.  Each round scores every candidate j by
-// c_j = |A - J(j)| (one warp per candidate, popcounts of A & ~row_j), keeps
-// the best with one 64-bit atomicMax on (c_j, -j) -- the largest c, the
-// smallest label on ties, as in the algorithm's scan -- and one block
-// removes J(k) from A and J(k) + {k} from the candidates.
+// Greedy antichain.  Each round takes the candidate j with the largest c_j =
+// |A - J(j)|, the smallest label on ties, as in the algorithm's scan, and
+// removes J(k) from A and J(k) + {k} from the candidates.  Maximising c_j is
+// minimising the overlap o_j = |A & J(j)|; the candidates removed in a round
+// are what every other overlap loses.
 //
-// Both run all their rounds in one cooperative launch, the rounds separated
-// by bounded grid barriers; where a cooperative launch is not available they
-// fall back to batches of kBatch launches between host checks of the number
-// of elements left (rounds after the last one find nothing to do).
+// Both run all their rounds in one cooperative launch, one CTA per SM, each
+// with its own copy of the set (S, or the candidates) in shared memory, so
+// that a round takes one bounded grid barrier; where a cooperative launch is
+// not available they fall back to batches of kBatch launches between host
+// checks of the number of elements left (rounds after the last one find
+// nothing to do).
 #include "cs_kernels.cuh"
 
 namespace cs {
@@ -32,17 +35,16 @@ struct ChainState {
     unsigned long long best;  // antichain: packed (c, ~label) of the best candidate
     int32_t found;            // chain: this round removed something
     int32_t related;          // chain: i precedes j
-    int64_t rounds;           // rounds that removed something
+    int64_t rounds;           // rounds that removed something; -1 until known
     int64_t left;             // elements left in S (chain) or candidates left (antichain)
-    // persistent (cooperative) kernels: grid barrier and per-round-parity counters
-    unsigned int bar_count, bar_gen;
-    unsigned long long left2[2];
-    unsigned long long best2[2];
-    unsigned int rcount[2];   // antichain: candidates removed this round (list length)
+    // persistent (cooperative) kernels
+    unsigned int arrived;         // grid barrier: blocks that arrived, all rounds together
+    int32_t status;               // the kernel's cs_status
+    unsigned long long best3[3];  // antichain: smallest (overlap, label) of a round, rounds in turn
 };
 
 struct ChainLayout {
-    size_t state, s, m, over, rlist, total;
+    size_t state, s, m, total;
 };
 
 ChainLayout chain_layout(int64_t row_words) {
@@ -52,14 +54,15 @@ ChainLayout chain_layout(int64_t row_words) {
     off = align_up(off + sizeof(ChainState), 256);
     L.s = off;
     off = align_up(off + size_t(row_words) * 8, 256);
-    L.m = off;
-    off = align_up(off + size_t(row_words) * 8, 256);
-    L.over = off;  // antichain: overlap |A & J(j)| of every candidate j
-    off = align_up(off + size_t(row_words) * 64 * 4, 256);
-    L.rlist = off;  // antichain: the candidates removed in a round
-    off = align_up(off + size_t(row_words) * 64 * 4, 256);
+    L.m = off;  // chain: the elements removed in a round, three rounds in turn
+    off = align_up(off + 3 * size_t(row_words) * 8, 256);
     L.total = off;
     return L;
+}
+
+// The workspace header stands before the state.
+__device__ __forceinline__ WsHeader* header_of(ChainState* st) {
+    return reinterpret_cast<WsHeader*>(reinterpret_cast<uint8_t*>(st) - sizeof(WsHeader));
 }
 
 __device__ __forceinline__ bool bit_of(const uint64_t* row, int64_t k) { return (row[k >> 6] >> (k & 63)) & 1ull; }
@@ -90,9 +93,14 @@ __global__ void k_chain_init(const uint64_t* __restrict__ bits, int64_t n, int64
         if (!whole) x &= __ldg(bits + i * row_words + w) & __ldg(bits + j * row_words + w);
         S[w] = x;
         M[w] = 0ull;
+        M[row_words + w] = 0ull;
+        M[2 * row_words + w] = 0ull;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         st->found = 0;
+        st->arrived = 0u;
+        st->status = 0;
+        header_of(st)->status = 0;
         st->rounds = 0;
         st->related = whole ? 1 : int(bit_of(bits + i * row_words, j));
         st->left = 1;
@@ -161,6 +169,11 @@ __global__ void k_anti_init(const uint64_t* __restrict__ bits, int64_t n, int64_
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         st->best = 0ull;
         st->left = 1;
+        st->arrived = 0u;
+        st->status = 0;
+        header_of(st)->status = 0;
+        st->rounds = -1;
+        for (int k = 0; k < 3; ++k) st->best3[k] = ~0ull;
     }
 }
 
@@ -236,178 +249,265 @@ __global__ void __launch_bounds__(1024) k_count_bits(const uint64_t* __restrict_
 // kernel returns (every later barrier of the other blocks then times out
 // too), so a fault cannot hang the GPU.
 
-__device__ bool grid_barrier(ChainState* st, unsigned int nblocks, WsHeader* hdr) {
-    __shared__ int ok_s;
+constexpr int kPersistThreads = 1024;
+constexpr int kPersistWarps = kPersistThreads / 32;
+
+// Barrier number r (from 0) of all blocks: the blocks' writes before it are
+// visible after it (read them with __ldcg).  One counter that only grows: no
+// reset to wait for.
+__device__ bool grid_barrier(ChainState* st, unsigned int r) {
     __syncthreads();
-    if (threadIdx.x == 0) {
-        int ok = 1;
-        volatile unsigned int* gen = &st->bar_gen;
-        const unsigned int g = *gen;
+    int ok = 1;
+    if (threadIdx.x == 0 && gridDim.x > 1) {
+        const unsigned int target = (r + 1) * gridDim.x;
         __threadfence();
-        if (atomicAdd(&st->bar_count, 1u) == nblocks - 1u) {
-            st->bar_count = 0u;
-            __threadfence();
-            atomicAdd(&st->bar_gen, 1u);
-        } else {
-            const unsigned long long t0 = global_timer_ns();
-            while (*gen == g) {
-                if (global_timer_ns() - t0 > kWaitLimitNs) {
-                    set_status(hdr, CS_ETIMEOUT);
-                    ok = 0;
-                    break;
-                }
-                __nanosleep(64);
+        atomicAdd(&st->arrived, 1u);
+        const unsigned long long t0 = global_timer_ns();
+        for (unsigned int spin = 1;; ++spin) {
+            unsigned int seen;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&st->arrived) : "memory");
+            if (int(seen - target) >= 0) break;
+            if ((spin & 63u) == 0u && global_timer_ns() - t0 > kWaitLimitNs) {
+                atomicCAS(&st->status, 0, int(CS_ETIMEOUT));
+                set_status(header_of(st), CS_ETIMEOUT);
+                ok = 0;
+                break;
             }
         }
         __threadfence();
-        ok_s = ok;
     }
-    __syncthreads();
-    return ok_s != 0;
+    return __syncthreads_and(ok) != 0;
 }
 
-__device__ __forceinline__ unsigned long long block_sum_to(unsigned long long v, unsigned long long* dst) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0 && v) atomicAdd(dst, v);
-    return v;
-}
-
-// All peeling rounds: peel (as k_chain_peel), barrier, S -= M with the count
-// of what is left, barrier, stop when nothing is left.  rounds = the number
-// of rounds run (S is not empty at the start).
-__global__ void __launch_bounds__(256) k_chain_persist(const uint64_t* __restrict__ bits, int64_t row_words,
-                                                       int64_t lo, int64_t hi, int64_t max_rounds, uint64_t* S,
-                                                       uint64_t* M, ChainState* st, WsHeader* hdr) {
+// All peeling rounds, one barrier each.  Element lo + 1 + e belongs to lane
+// (e / warps) % 32 of warp e % warps (neighbours, which lose their
+// predecessors together, to different SMs); slot t holds its 32 t-th on.
+// Per slot the lane keeps the word w of its row that last met S, and that
+// word's predecessor bits x.  A round: S minus the last round's removals in
+// every block's shared copy; an element whose x no longer meets S has its
+// row searched by the whole warp from w down, 64 words a step; one that finds
+// nothing is minimal and enters this round's removals.  rounds = the number
+// of rounds run until S is empty.
+//
+// Two barriers a round of 1216 small blocks, and every element's row scanned
+// from its label down each round, took 20 us a round at n = 32768 (7.2 ms
+// for the 362 of a 2D order).
+template <int kSlots>
+__global__ void __launch_bounds__(kPersistThreads) k_chain_persist(const uint64_t* __restrict__ bits,
+                                                                   int64_t row_words, int64_t lo, int64_t hi,
+                                                                   int64_t max_rounds, const uint64_t* __restrict__ S0,
+                                                                   uint64_t* M, ChainState* st) {
+    extern __shared__ __align__(16) uint64_t S[];  // [row_words]
+    if (!st->related) return;  // the same in every block
     const int lane = threadIdx.x & 31;
-    const int64_t warps = int64_t(gridDim.x) * (blockDim.x >> 5);
-    const int64_t gwarp = int64_t(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int64_t gthread = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    const int64_t nthreads = int64_t(gridDim.x) * blockDim.x;
-    const int64_t wlo = lo < 0 ? 0 : lo >> 6;
+    const int64_t warps = int64_t(gridDim.x) * kPersistWarps;
+    const int64_t gwarp = int64_t(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    const int64_t wlo = lo < 0 ? 0 : lo >> 6, whi = hi > 0 ? (hi - 1) >> 6 : 0;  // words S may touch
+    int any = 0;
+    for (int64_t w = threadIdx.x; w < row_words; w += kPersistThreads) {
+        S[w] = __ldg(S0 + w);
+        any |= S[w] != 0ull;
+    }
+    if (!__syncthreads_or(any)) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) st->rounds = 0;
+        return;
+    }
+    // Predecessors of element k in word w of its row.
+    auto preds = [&](int64_t k, int64_t w, uint64_t x) {
+        return w == (k >> 6) ? x & ((1ull << (k & 63)) - 1ull) : x;
+    };
+    int w[kSlots];        // -1: no element, or removed
+    uint64_t x[kSlots];
+#pragma unroll
+    for (int t = 0; t < kSlots; ++t) {
+        const int64_t k = lo + 1 + (int64_t(32 * t + lane)) * warps + gwarp;
+        const bool in = k < hi && ((S[k >> 6] >> (k & 63)) & 1ull);
+        w[t] = in ? int(k >> 6) : -1;
+        x[t] = in ? preds(k, k >> 6, __ldg(bits + k * row_words + (k >> 6))) : 0ull;
+    }
     for (int64_t r = 0; r < max_rounds; ++r) {
-        for (int64_t k = lo + 1 + gwarp; k < hi; k += warps) {
-            if (!bit_of(S, k)) continue;  // warp-uniform
-            const int64_t wk = k >> 6;
-            int any = 0;
-            for (int64_t w = wk - lane; w >= wlo && !any; w -= 32) {  // nearest predecessors first
-                uint64_t x = __ldg(bits + k * row_words + w) & S[w];
-                if (w == wk) x &= (k & 63) ? ((1ull << (k & 63)) - 1ull) : 0ull;
-                any = x != 0ull;
+        uint64_t* Mr = M + (r % 3) * row_words;
+#pragma unroll
+        for (int t = 0; t < kSlots; ++t) {
+            const bool lost = w[t] >= 0 && (x[t] & S[w[t]]) == 0ull;
+            for (uint32_t todo = __ballot_sync(0xffffffffu, lost); todo; todo &= todo - 1u) {
+                const int f = __ffs(int(todo)) - 1;
+                const int64_t k = lo + 1 + (int64_t(32 * t + f)) * warps + gwarp;
+                const uint64_t* row = bits + k * row_words;
+                int64_t w1 = __shfl_sync(0xffffffffu, w[t], f) - 1;  // the next word to look at
+                int64_t at = -1;
+                uint64_t found = 0ull;
+                while (w1 >= wlo) {
+                    // lane l: words w1 - l and w1 - 32 - l
+                    const int64_t wa = w1 - lane, wc = wa - 32;
+                    const uint64_t xa = wa >= wlo ? __ldg(row + wa) : 0ull, xc = wc >= wlo ? __ldg(row + wc) : 0ull;
+                    const uint32_t ma = __ballot_sync(0xffffffffu, wa >= wlo && (xa & S[wa]) != 0ull);
+                    const uint32_t mc = __ballot_sync(0xffffffffu, wc >= wlo && (xc & S[wc]) != 0ull);
+                    if (ma | mc) {  // the nearest one
+                        const int q = __ffs(int(ma ? ma : mc)) - 1;
+                        at = w1 - q - (ma ? 0 : 32);
+                        found = __shfl_sync(0xffffffffu, ma ? xa : xc, q);
+                        break;
+                    }
+                    w1 -= 64;
+                }
+                if (lane == f) {
+                    w[t] = int(at);
+                    x[t] = found;
+                    if (at < 0) atomicOr(reinterpret_cast<unsigned long long*>(Mr + (k >> 6)), 1ull << (k & 63));
+                }
             }
-            if (!warp_or(any) && lane == 0) atomicOr(reinterpret_cast<unsigned long long*>(M + wk), 1ull << (k & 63));
         }
-        if (!grid_barrier(st, gridDim.x, hdr)) return;
-        unsigned long long mine = 0;
-        for (int64_t w = gthread; w < row_words; w += nthreads) {
-            const uint64_t x = S[w] & ~M[w];
-            S[w] = x;
-            M[w] = 0ull;
-            mine += __popcll(x);
+        // clear the next round's removals (last read in the round before this one)
+        uint64_t* Mn = M + ((r + 1) % 3) * row_words;
+        for (int64_t q = int64_t(blockIdx.x) * kPersistThreads + threadIdx.x; q < row_words;
+             q += int64_t(gridDim.x) * kPersistThreads)
+            Mn[q] = 0ull;
+        if (!grid_barrier(st, unsigned(r))) return;
+        int left = 0;
+        for (int64_t q = wlo + threadIdx.x; q <= whi; q += kPersistThreads) {
+            const uint64_t y = S[q] & ~__ldcg(Mr + q);
+            S[q] = y;
+            left |= y != 0ull;
         }
-        block_sum_to(mine, &st->left2[r & 1]);
-        if (gthread == 0) st->left2[(r + 1) & 1] = 0ull;  // last read before the previous barrier
-        if (!grid_barrier(st, gridDim.x, hdr)) return;
-        if (*reinterpret_cast<volatile unsigned long long*>(&st->left2[r & 1]) == 0ull) {
-            if (gthread == 0) st->rounds = r + 1;
+        if (!__syncthreads_or(left)) {
+            if (blockIdx.x == 0 && threadIdx.x == 0) st->rounds = r + 1;
             return;
         }
     }
 }
 
-// All greedy rounds, with incremental scores.  Maximising c_j = |A - J(j)|
-// is minimising the overlap o_j = |A & J(j)|.  When k is taken, A loses
-// R = A & J(k), which are exactly the candidates related to k (the members
-// are unrelated to every candidate), so every remaining o_j drops by the
-// number of R's elements related to j.  Per round: the smallest (o_j, j) by
-// one 64-bit atomicMin, barrier; remove J(k) from A and J(k) + {k} from X
-// and list R, barrier; stop if X is empty; subtract R's contributions from
-// the o_j of the remaining candidates (a thread per column, the list read
-// in step), barrier.  The overlaps are computed in full once, at the start.
-__global__ void __launch_bounds__(256) k_anti_persist(const uint64_t* __restrict__ bits, int64_t n,
-                                                      int64_t row_words, int64_t max_rounds, uint64_t* A,
-                                                      uint64_t* X, int32_t* over, int32_t* rlist, ChainState* st,
-                                                      WsHeader* hdr) {
-    const int lane = threadIdx.x & 31;
+// All greedy rounds, one barrier each.  Block b owns the candidates of its
+// share of the 32-column groups and keeps their overlaps in shared memory;
+// every block keeps all candidates X.  A round: the block's smallest (o_j, j),
+// one 64-bit atomicMin, barrier; then every block for itself reads row k and
+// takes J(k) and k out of X, lists the candidates R that this removed (A loses
+// exactly these: the members are unrelated to every candidate), and lowers
+// its overlaps by the number of R's elements related to j, the warps of a
+// group taking R's rows in turn (a row's word serves 32 candidates).  The
+// overlaps are counted in full once, at the start.  Three barriers a round
+// and one thread per candidate walking R took 37 us a round at n = 32768.
+constexpr int kListCap = 4096;  // elements of R listed at a time
+__global__ void __launch_bounds__(kPersistThreads) k_anti_persist(const uint64_t* __restrict__ bits, int64_t n,
+                                                                  int64_t row_words, int64_t seed, int64_t max_rounds,
+                                                                  uint64_t* members,
+                                                                  const uint64_t* __restrict__ X0, int64_t groups_per_block,
+                                                                  ChainState* st) {
+    extern __shared__ __align__(16) uint64_t X[];  // [row_words], then the overlaps, the list
+    int32_t* over = reinterpret_cast<int32_t*>(X + row_words);
+    int32_t* list = over + 32 * groups_per_block;
+    __shared__ int listed, valid;  // elements offered to the list, and listed without a gap
+    __shared__ unsigned long long least;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t nw = (n + 63) >> 6;
-    const int64_t warps = int64_t(gridDim.x) * (blockDim.x >> 5);
-    const int64_t gwarp = int64_t(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int64_t gthread = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    const int64_t nthreads = int64_t(gridDim.x) * blockDim.x;
-    for (int64_t k = gwarp; k < n; k += warps) {  // o_j for every candidate, once
-        if (!bit_of(X, k)) continue;               // warp-uniform
-        int c = 0;
-        for (int64_t w = lane; w < nw; w += 32) c += __popcll(A[w] & __ldg(bits + k * row_words + w));
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-        if (lane == 0) over[k] = c;
+    const int64_t g0 = int64_t(blockIdx.x) * groups_per_block;
+    const int64_t groups = (n + 31) / 32;
+    const int ng = int(g0 >= groups ? 0 : (groups - g0 < groups_per_block ? groups - g0 : groups_per_block));
+    for (int64_t w = threadIdx.x; w < row_words; w += kPersistThreads) {
+        X[w] = __ldg(X0 + w);
+        if (blockIdx.x == 0) members[w] = w == (seed >> 6) ? 1ull << (seed & 63) : 0ull;
     }
-    if (!grid_barrier(st, gridDim.x, hdr)) return;
+    __syncthreads();
+    for (int c = warp; c < 32 * ng; c += kPersistWarps) {
+        const int64_t j = 32 * g0 + c;
+        int o = 0;
+        if (j < n && bit_of(X, j)) {  // warp-uniform
+#pragma unroll 4
+            for (int64_t w = lane; w < nw; w += 32) o += __popcll(X[w] & __ldg(bits + j * row_words + w));
+            o = int(__reduce_add_sync(0xffffffffu, unsigned(o)));
+        }
+        if (lane == 0) over[c] = o;
+    }
+    __syncthreads();
+    // warps per group (a group per warp, in turn, when there are more groups)
+    const int share = ng > 0 && ng < kPersistWarps ? kPersistWarps / ng : 1;
+    int64_t taken = 0;
     for (int64_t r = 0; r < max_rounds; ++r) {
-        // the candidate with the smallest overlap, the smallest label on ties
+        if (threadIdx.x == 0) least = ~0ull;
+        __syncthreads();
         unsigned long long mine = ~0ull;
-        for (int64_t j = gthread; j < n; j += nthreads)
-            if (bit_of(X, j)) {
-                const unsigned long long key = (static_cast<unsigned long long>(over[j]) << 32) | uint64_t(j);
+        for (int c = threadIdx.x; c < 32 * ng; c += kPersistThreads) {
+            const int64_t j = 32 * g0 + c;
+            if (j < n && bit_of(X, j)) {
+                const unsigned long long key = (static_cast<unsigned long long>(over[c]) << 32) | uint64_t(j);
                 mine = key < mine ? key : mine;
             }
+        }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             const unsigned long long y = __shfl_xor_sync(0xffffffffu, mine, o);
             mine = y < mine ? y : mine;
         }
-        if (lane == 0 && mine != ~0ull) atomicMin(&st->best2[r & 1], mine);
-        if (gthread == 0) {
-            st->best2[(r + 1) & 1] = ~0ull;  // last read before the previous round's second barrier
-            st->rcount[(r + 1) & 1] = 0u;
-            st->left2[(r + 1) & 1] = 0ull;
+        if (lane == 0 && mine != ~0ull) atomicMin(&least, mine);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            if (least != ~0ull) atomicMin(&st->best3[r % 3], least);
+            if (blockIdx.x == 0) st->best3[(r + 1) % 3] = ~0ull;  // last read in the round before last
         }
-        if (!grid_barrier(st, gridDim.x, hdr)) return;
-        const unsigned long long best = *reinterpret_cast<volatile unsigned long long*>(&st->best2[r & 1]);
-        if (best == ~0ull) return;  // no candidates (every block sees the same value)
+        if (!grid_barrier(st, unsigned(r))) return;
+        const unsigned long long best = __ldcg(&st->best3[r % 3]);
+        if (best == ~0ull) break;  // no candidates (every block sees the same value)
+        ++taken;
         const int64_t k = int64_t(best & 0xFFFFFFFFull);
-        unsigned long long left = 0;
-        for (int64_t w = gthread; w < row_words; w += nthreads) {
-            const uint64_t rk = __ldg(bits + k * row_words + w);
-            const uint64_t x = X[w];
-            uint64_t removed = x & rk;
-            uint64_t nx = x & ~rk;
-            if (w == (k >> 6)) nx &= ~(1ull << (k & 63));
-            X[w] = nx;
-            A[w] &= ~rk;
-            left += __popcll(nx);
-            if (removed) {
-                unsigned int pos = atomicAdd(&st->rcount[r & 1], unsigned(__popcll(removed)));
-                for (; removed; removed &= removed - 1ull)
-                    rlist[pos++] = int32_t(64 * w + __ffsll(static_cast<long long>(removed)) - 1);
+        if (threadIdx.x == 0) {
+            X[k >> 6] &= ~(1ull << (k & 63));
+            if (blockIdx.x == 0) members[k >> 6] |= 1ull << (k & 63);
+        }
+        for (bool more = true; more;) {
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                listed = 0;
+                valid = kListCap;
+            }
+            __syncthreads();
+            int rest = 0;
+            for (int64_t w = threadIdx.x; w < nw; w += kPersistThreads) {
+                uint64_t y = X[w] & __ldg(bits + k * row_words + w);
+                if (!y) continue;
+                const int c = __popcll(y), at = atomicAdd(&listed, c);
+                if (at + c > kListCap) {  // stays in X; its turn comes in the next pass
+                    atomicMin(&valid, at);
+                    rest = 1;
+                    continue;
+                }
+                X[w] &= ~y;
+                for (int q = at; y; y &= y - 1ull, ++q)
+                    list[q] = int32_t(64 * w + __ffsll(static_cast<long long>(y)) - 1);
+            }
+            more = __syncthreads_or(rest) != 0;
+            const int nr = listed < valid ? listed : valid;
+            for (int g = warp / share; g < ng; g += kPersistWarps / share) {
+                if (warp / share >= kPersistWarps / share) break;  // the warps left over
+                const uint32_t* col = reinterpret_cast<const uint32_t*>(bits) + (g0 + g);
+                int d = 0;
+#pragma unroll 8
+                for (int t = warp % share; t < nr; t += share) {
+                    d += int((__ldg(col + int64_t(list[t]) * row_words * 2) >> lane) & 1u);
+                }
+                if (d) atomicSub(&over[32 * g + lane], d);
             }
         }
-        block_sum_to(left, &st->left2[r & 1]);
-        if (!grid_barrier(st, gridDim.x, hdr)) return;
-        if (*reinterpret_cast<volatile unsigned long long*>(&st->left2[r & 1]) == 0ull) return;
-        const unsigned int nr = *reinterpret_cast<volatile unsigned int*>(&st->rcount[r & 1]);
-        for (int64_t j = gthread; j < n; j += nthreads) {
-            if (!bit_of(X, j)) continue;
-            int d = 0;
-            for (unsigned int t = 0; t < nr; ++t)
-                d += int((__ldg(bits + int64_t(rlist[t]) * row_words + (j >> 6)) >> (j & 63)) & 1ull);
-            over[j] -= d;
-        }
-        if (!grid_barrier(st, gridDim.x, hdr)) return;
+        __syncthreads();
     }
+    if (blockIdx.x == 0 && threadIdx.x == 0) st->rounds = taken + 1;  // and the seed
 }
 
-// Blocks of a cooperative launch of `kernel` (all resident), capped by the work.
-int coop_grid(const void* kernel, int64_t warps_of_work) {
-    int dev = 0, coop = 0, per_sm = 0;
+// Blocks of a cooperative launch of `kernel` with `smem` bytes, one per SM at
+// most and `need` of them at most; 0 where it is not possible.
+int coop_grid(const void* kernel, int smem, int64_t need) {
+    int dev = 0, coop = 0, per_sm = 0, most = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 256, 0) != cudaSuccess || per_sm < 1)
+        cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess || smem > most - 1024)
         return 0;
-    int64_t g = int64_t(per_sm) * device_sm_count();
-    const int64_t need = (warps_of_work + 7) / 8;
-    if (g > need) g = need;
-    return int(g < 1 ? 1 : g);
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kPersistThreads, smem) != cudaSuccess ||
+        per_sm < 1) {
+        cudaGetLastError();
+        return 0;
+    }
+    const int64_t sms = device_sm_count();
+    return int(need < 1 ? 1 : need < sms ? need : sms);
 }
 
 int warp_grid(int64_t rows) {
@@ -458,37 +558,32 @@ extern "C" int cs_longest_chain(int64_t n, const uint64_t* bits_dev, int64_t row
     int64_t g = (row_words + 255) / 256;
     k_chain_init<<<unsigned(g < 1 ? 1 : g), 256, 0, st>>>(bits_dev, n, row_words, whole ? -1 : i, j, S, M, sd);
     ChainState h{};
-    // one cooperative launch for all rounds when the device allows it
-    const int cg = coop_grid(reinterpret_cast<const void*>(k_chain_persist), hi - lo - 1);
+    // one cooperative launch for all rounds when the device allows it: about
+    // four elements per warp where the set does not fill the SMs
+    const int64_t count = hi - lo - 1;
+    const int smem = int(row_words * 8);
+    const int64_t per_slot = int64_t(device_sm_count()) * kPersistThreads;
+    const auto kernel = count <= per_slot       ? k_chain_persist<1>
+                        : count <= 4 * per_slot ? k_chain_persist<4>
+                                                : k_chain_persist<12>;
+    const int64_t blocks = (count + 4 * kPersistWarps - 1) / (4 * kPersistWarps);
+    const int cg = count <= 12 * per_slot ? coop_grid(reinterpret_cast<const void*>(kernel), smem, blocks) : 0;
     if (cg > 0) {
-        k_count_bits<<<1, 1024, 0, st>>>(S, row_words, sd);  // |S| at the start into rounds
-        if (cudaGetLastError() != cudaSuccess || read_state(sd, &h, st) != cudaSuccess) return CS_ECUDA;
-        if (!h.related) {
-            *length = -1;
-            return CS_OK;
-        }
-        if (h.rounds == 0) {  // empty interval: a link, or an empty set
-            *length = whole ? 0 : 1;
-            return CS_OK;
-        }
-        WsHeader* hdr = reinterpret_cast<WsHeader*>(ws);
-        if (cudaMemsetAsync(&sd->bar_count, 0, sizeof(unsigned int) * 2 + sizeof(unsigned long long) * 4, st) !=
-                cudaSuccess ||
-            cudaMemsetAsync(&sd->rounds, 0xFF, sizeof(int64_t), st) != cudaSuccess ||  // -1 until the last round
-            cudaMemsetAsync(&hdr->status, 0, sizeof(int32_t), st) != cudaSuccess)
-            return CS_ECUDA;
         int64_t max_rounds = n + 1;
+        const uint64_t* S0 = S;
         void* args[] = {const_cast<uint64_t**>(&bits_dev), &row_words, const_cast<int64_t*>(&lo),
-                        const_cast<int64_t*>(&hi), &max_rounds, &S, &M, &sd, &hdr};
-        if (cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_chain_persist), dim3(unsigned(cg)), dim3(256),
-                                        args, 0, st) == cudaSuccess) {
-            int32_t status = 0;
-            if (read_state(sd, &h, st) != cudaSuccess ||
-                cudaMemcpy(&status, &hdr->status, sizeof(status), cudaMemcpyDeviceToHost) != cudaSuccess)
-                return CS_ECUDA;
-            if (status != 0) return status;
+                        const_cast<int64_t*>(&hi), &max_rounds, &S0, &M, &sd};
+        if (cudaMemsetAsync(&sd->rounds, 0xFF, sizeof(int64_t), st) != cudaSuccess) return CS_ECUDA;  // -1 until the last round
+        if (cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(kernel), dim3(unsigned(cg)),
+                                        dim3(kPersistThreads), args, size_t(smem), st) == cudaSuccess) {
+            if (read_state(sd, &h, st) != cudaSuccess) return CS_ECUDA;
+            if (h.status != 0) return h.status;
+            if (!h.related) {
+                *length = -1;
+                return CS_OK;
+            }
             if (h.rounds < 0) return CS_ERANGE;  // cannot happen for a transitive relation
-            *length = whole ? h.rounds : h.rounds + 1;
+            *length = whole ? h.rounds : h.rounds + 1;  // no round: a link, or an empty set
             return CS_OK;
         }
         cudaGetLastError();  // not launched: clear and take the multi-launch path
@@ -523,34 +618,30 @@ extern "C" int cs_greedy_antichain(int64_t n, const uint64_t* bits_dev, int64_t 
     int64_t g = (row_words + 255) / 256;
     k_anti_init<<<unsigned(g < 1 ? 1 : g), 256, 0, st>>>(bits_dev, n, row_words, seed, members_dev, X, sd);
     ChainState h{};
-    const int cg = coop_grid(reinterpret_cast<const void*>(k_anti_persist), n);
-    bool done = false;
-    if (cg > 0) {
-        WsHeader* hdr = reinterpret_cast<WsHeader*>(ws);
-        int32_t* over = reinterpret_cast<int32_t*>(ws + L.over);
-        int32_t* rlist = reinterpret_cast<int32_t*>(ws + L.rlist);
-        if (cudaMemsetAsync(&sd->bar_count, 0, sizeof(unsigned int) * 2 + sizeof(unsigned long long) * 2, st) !=
-                cudaSuccess ||
-            cudaMemsetAsync(&sd->best2[0], 0xFF, sizeof(unsigned long long), st) != cudaSuccess ||  // no best yet
-            cudaMemsetAsync(&sd->rcount[0], 0, sizeof(unsigned int) * 2, st) != cudaSuccess ||
-            cudaMemsetAsync(&hdr->status, 0, sizeof(int32_t), st) != cudaSuccess)
-            return CS_ECUDA;
+    const int64_t groups = (n + 31) / 32;
+    const int64_t sms = device_sm_count();
+    // at least four groups of 32 candidates per block, at most the SMs' share
+    int64_t per = (groups + sms - 1) / sms;
+    if (per < 4) per = 4;
+    const int64_t blocks = (groups + per - 1) / per;
+    const int smem = int(row_words * 8 + 32 * per * 4 + kListCap * 4);
+    const int cg = coop_grid(reinterpret_cast<const void*>(k_anti_persist), smem, blocks);
+    if (cg == blocks) {
         int64_t max_rounds = n + 1;
-        void* args[] = {const_cast<uint64_t**>(&bits_dev), &n, &row_words, &max_rounds, &members_dev, &X,
-                        &over, &rlist, &sd, &hdr};
-        if (cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_anti_persist), dim3(unsigned(cg)), dim3(256),
-                                        args, 0, st) == cudaSuccess) {
-            int32_t status = 0;
-            if (cudaStreamSynchronize(st) != cudaSuccess ||
-                cudaMemcpy(&status, &hdr->status, sizeof(status), cudaMemcpyDeviceToHost) != cudaSuccess)
-                return CS_ECUDA;
-            if (status != 0) return status;
-            done = true;
-        } else {
-            cudaGetLastError();
-            k_anti_init<<<unsigned(g < 1 ? 1 : g), 256, 0, st>>>(bits_dev, n, row_words, seed, members_dev, X, sd);
+        const uint64_t* X0 = X;
+        void* args[] = {const_cast<uint64_t**>(&bits_dev), &n, &row_words, &seed, &max_rounds, &members_dev, &X0, &per, &sd};
+        if (cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_anti_persist), dim3(unsigned(cg)),
+                                        dim3(kPersistThreads), args, size_t(smem), st) == cudaSuccess) {
+            if (read_state(sd, &h, st) != cudaSuccess) return CS_ECUDA;
+            if (h.status != 0) return h.status;
+            if (h.rounds < 0) return CS_ERANGE;
+            *size = h.rounds;
+            return CS_OK;
         }
+        cudaGetLastError();
+        k_anti_init<<<unsigned(g < 1 ? 1 : g), 256, 0, st>>>(bits_dev, n, row_words, seed, members_dev, X, sd);
     }
+    bool done = false;
     for (int64_t rounds = 0; !done && rounds <= n; rounds += kBatch) {  // multi-launch path
         for (int r = 0; r < kBatch; ++r) {
             k_anti_score<<<warp_grid(n), 256, 0, st>>>(bits_dev, n, row_words, members_dev, X, sd);
