@@ -166,14 +166,23 @@ __global__ void k_scan_add(int64_t* __restrict__ out, int64_t n, const int64_t* 
 // at cols[offsets[i] ..).  A row whose list would end past cols_capacity is
 // skipped and CS_ENOMEM recorded.  The warp walks its row 32 words at a
 // time, lane l owning word l: an inclusive warp scan of the words'
-// popcounts gives each word's first place in the step's run, each lane
-// writes its word's set columns (lowest bit first) into the warp's shared
-// buffer there, and the warp copies the run out in coalesced stores.  (One
-// lane per bit of each half-word in turn, with a popcount, a rank and a
-// predicated store per half-word, held the integer pipe at three times the
-// instructions per relation: 0.42 of the HBM rate at N = 2^17.)
+// popcounts gives each word's first place in the step's run, the set columns
+// go to the warp's shared buffer there, and the warp copies the run out in
+// coalesced stores.  What bounds it is the shared-memory pipe, so the columns
+// are placed in one of two ways, by the step's relations:
+//   few: every lane writes its own word's columns, lowest bit first -- as
+//     many passes as the fullest word has bits, the lanes' places on random
+//     banks (3 to 4 passes of the pipe per store: 510 per step of a 1+1 set,
+//     where half of the bits are set);
+//   many: word after word (read by broadcast), lane l placing bits l and l + 32 by
+//     their rank within the word: consecutive places, one pass per store and
+//     the same cost whatever is set, about that of the first way at 640
+//     relations a step (with a limit of 320 the lists of a de Sitter slab,
+//     whose steps hold up to 650, took 341 us instead of 308).
+// Future list of a 1+1 diamond, n = 30011: 398 -> 205 us (4.4 TB/s).
 constexpr int kColsWarps = 4;                      // warps per block
 constexpr int kColsRun = 32 * 64 + 4;              // the most columns one step emits, and an alignment shift
+constexpr int kManyColumns = 640;                  // columns of a step from which they are placed word after word
 __global__ void __launch_bounds__(kColsWarps * 32) k_side_columns(const uint64_t* __restrict__ bits, int64_t n,
                                                                    int64_t row_words, bool future,
                                                                    const int64_t* __restrict__ offsets,
@@ -181,6 +190,7 @@ __global__ void __launch_bounds__(kColsWarps * 32) k_side_columns(const uint64_t
                                                                    int64_t cols_capacity, WsHeader* hdr) {
     __shared__ __align__(16) int32_t stage[kColsWarps][kColsRun];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    __shared__ __align__(16) int4 words[kColsWarps][32];  // a step's words and the places of their halves
     int32_t* run = stage[warp];
     const int64_t warps = int64_t(gridDim.x) * kColsWarps;
     for (int64_t i = int64_t(blockIdx.x) * kColsWarps + warp; i < n; i += warps) {
@@ -211,11 +221,25 @@ __global__ void __launch_bounds__(kColsWarps * 32) k_side_columns(const uint64_t
             // run's 16-byte groups are the output's
             const int s0 = int((reinterpret_cast<uintptr_t>(cols + pos) >> 2) & 3);
             int at = s0 + incl - c;
-            const int32_t base = int32_t(64 * w);  // n <= 2^22
-            // lowest bit first, one 32-bit half at a time (cheaper steps than
-            // 64-bit find-first and clear-lowest)
-            for (uint32_t h = uint32_t(x); h; h &= h - 1u) run[at++] = base + (__ffs(int(h)) - 1);
-            for (uint32_t h = uint32_t(x >> 32); h; h &= h - 1u) run[at++] = base + 31 + __ffs(int(h));
+            if (total >= kManyColumns) {  // warp-uniform
+                words[warp][lane] =
+                    make_int4(int(uint32_t(x)), int(uint32_t(x >> 32)), at, at + __popc(uint32_t(x)));
+                __syncwarp();
+                const uint32_t bit = 1u << lane, before = bit - 1u;
+                int32_t column = int32_t(64 * w0) + lane;
+#pragma unroll 8
+                for (int q = 0; q < 32; ++q, column += 64) {
+                    const int4 v = words[warp][q];
+                    if (uint32_t(v.x) & bit) run[v.z + __popc(uint32_t(v.x) & before)] = column;
+                    if (uint32_t(v.y) & bit) run[v.w + __popc(uint32_t(v.y) & before)] = column + 32;
+                }
+            } else {
+                const int32_t base = int32_t(64 * w);  // n <= 2^22
+                // lowest bit first, one 32-bit half at a time (cheaper steps than
+                // 64-bit find-first and clear-lowest)
+                for (uint32_t h = uint32_t(x); h; h &= h - 1u) run[at++] = base + (__ffs(int(h)) - 1);
+                for (uint32_t h = uint32_t(x >> 32); h; h &= h - 1u) run[at++] = base + 31 + __ffs(int(h));
+            }
             __syncwarp();
             // a head up to the first 16-byte boundary, whole groups as
             // 16-byte stores, then a tail; positions at or past `end` are
