@@ -25,15 +25,20 @@ __host__ __device__ inline int act_blocks(int64_t kend, int T) {
 }
 
 // Partial smeared sums, grid (blocks of the longest cutoff, eps).  A term is
-// about 300 dependent FP64 operations (the power by repeated squaring, the
-// polynomial, two products), and GB300 issues about two FP64 lanes per SM
+// about 150 dependent FP64 operations (the power, the polynomial, two
+// products), and GB300 issues about two FP64 lanes per SM
 // and cycle: what bounds this is how few SMs the terms sit on.  So a block
 // is one warp while the cutoffs are below 4096 terms (wider beyond),
 // the eps values run side by side, and the sum is a shuffle tree.  256
 // threads per block walking the eps values one after another took 102 us
-// for n = 1024 .. 16384 and three smeared eps; this takes 8.
+// for n = 1024 .. 16384 and three smeared eps; this takes 12 (19 while every
+// thread squared its own powers).
+struct ActPowers {
+    EpsPowers e[kMaxEps];
+};
 __global__ void __launch_bounds__(kActThreads) k_action_partial(int dim, const int64_t* __restrict__ hist,
-                                                                EpsArgs eps, dd* __restrict__ partial) {
+                                                                EpsArgs eps, const __grid_constant__ ActPowers powers,
+                                                                dd* __restrict__ partial) {
     __shared__ dd red[kActThreads / 32];
     const int e = blockIdx.y, T = blockDim.x, tid = threadIdx.x;
     const int64_t kend = eps.kend[e];  // 0 for a local action
@@ -45,8 +50,8 @@ __global__ void __launch_bounds__(kActThreads) k_action_partial(int dim, const i
     for (int64_t k = int64_t(blockIdx.x) * T + tid; k < kend; k += int64_t(nb) * T) {
         const int64_t hk = hist[k];
         if (hk == 0) continue;
-        const dd f = dd_mul(dd_pow(q, smear_qexp(dim, k)), smear_poly(dim, k, q, ep));
-        sum = dd_add(sum, dd_mul(dd_from_i64(hk), f));
+        const dd f = dd_mul(power_of(powers.e[e], smear_qexp(dim, k)), smear_poly(dim, k, q, ep));
+        sum = dd_accumulate(sum, hk, f);
     }
     sum = warp_sum_dd(sum);
     if (T > 32) {  // uniform
@@ -158,8 +163,13 @@ cudaError_t launch_action_device(int dim, int64_t n, const int64_t* hist, int64_
     int T = 32;  // threads per block: the fewest that give each thread one term
     while (T < kActThreads && kmax > int64_t(kActBlocks) * T) T *= 2;
     dd* partial = reinterpret_cast<dd*>(static_cast<uint8_t*>(workspace) + sizeof(WsHeader));
-    if (kmax > 0)
-        k_action_partial<<<dim3(unsigned(act_blocks(kmax, T)), unsigned(n_eps)), T, 0, st>>>(dim, hist, a, partial);
+    if (kmax > 0) {
+        ActPowers powers;
+        for (int e = 0; e < kMaxEps; ++e)
+            if (e < n_eps && !is_local(a.v[e])) powers.e[e] = eps_powers(a.v[e]);
+        k_action_partial<<<dim3(unsigned(act_blocks(kmax, T)), unsigned(n_eps)), T, 0, st>>>(dim, hist, a, powers,
+                                                                                          partial);
+    }
     k_action_final<<<1, 32 * n_eps, 0, st>>>(dim, n, hist, len, a, T, partial, out, bracket);
     return cudaGetLastError();
 }

@@ -13,6 +13,39 @@ constexpr int kMaxEps = 16;  // eps values per call
 constexpr int kActThreads = 256;
 constexpr int kActBlocks = 128;  // partial sums per eps
 
+// Powers q^(2^b), q = 1 - eps, of one eps: found on the host, so that a power
+// on the device is a product of the few that its exponent's bits ask for (the
+// repeated squaring took as many dependent double-double products again).
+constexpr int kPowBits = 22;  // every exponent of a set (at most 2^22 elements)
+struct EpsPowers {
+    dd p[kPowBits];
+};
+inline EpsPowers eps_powers(double eps) {
+    EpsPowers t;
+    t.p[0] = dd_two_sum(1.0, -eps);
+    for (int b = 1; b < kPowBits; ++b) t.p[b] = dd_mul(t.p[b - 1], t.p[b - 1]);
+    return t;
+}
+__device__ __forceinline__ dd power_of(const EpsPowers& t, int64_t k) {
+    dd r = dd_from(1.0);
+    if (k >> kPowBits) r = dd_pow(dd_mul(t.p[kPowBits - 1], t.p[kPowBits - 1]), k >> kPowBits);  // a longer histogram
+    for (uint32_t m = uint32_t(k) & ((1u << kPowBits) - 1u); m; m &= m - 1u) r = dd_mul(r, t.p[__ffs(int(m)) - 1]);
+    return r;
+}
+
+// sum + c * f for a count c < 2^53 (exact as a double): the product to double-double,
+// its high part added with its rounding error kept, the low parts in plain
+// FP64.  The low sums stay below 2^-53 of the high ones, so what is lost is
+// below 2^-105 of the largest partial sum per term, at 15 FP64 operations
+// where the full double-double product and sum take 34.
+__device__ __forceinline__ dd dd_accumulate(dd sum, int64_t c, dd f) {
+    const double x = static_cast<double>(c);
+    const double p = x * f.hi;
+    const double e = fma(x, f.lo, fma(x, f.hi, -p));
+    const dd s = dd_two_sum(sum.hi, p);
+    return {s.hi, sum.lo + (s.lo + e)};
+}
+
 struct EpsArgs {
     double v[kMaxEps];
     int64_t kend[kMaxEps];  // smeared-sum cutoffs (single-set kernels; set on the host)

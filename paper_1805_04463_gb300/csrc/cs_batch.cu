@@ -323,7 +323,11 @@ struct CoefArgs {
 // The same launch finds each (set, eps) cutoff once (kends), after the
 // table entries: a fixed-point iteration of about 1500 FP64 operations, too
 // costly to repeat in every thread of the action kernel.
+struct BatchPowers {
+    EpsPowers e[kMaxEps];
+};
 __global__ void __launch_bounds__(32) k_batch_coef(dd* __restrict__ coef, CoefArgs c, EpsArgs eps,
+                                                    const __grid_constant__ BatchPowers powers,
                                                     const BatchSet* __restrict__ sets, int nsets,
                                                     int64_t* __restrict__ kends) {
     const int64_t total = c.seg[kDimSlots * kMaxEps];
@@ -346,7 +350,7 @@ __global__ void __launch_bounds__(32) k_batch_coef(dd* __restrict__ coef, CoefAr
         const double ep = eps.v[e];
         const dd q = dd_two_sum(1.0, -ep);
         coef[c.base[slot] + e * c.stride[slot] + k] =
-            dd_mul(dd_pow(q, smear_qexp(dim, k)), smear_poly(dim, k, q, ep));
+            dd_mul(power_of(powers.e[e], smear_qexp(dim, k)), smear_poly(dim, k, q, ep));
     }
 }
 
@@ -387,7 +391,7 @@ __global__ void __launch_bounds__(kActThreads) k_batch_action(const BatchSet* __
     dd sum = dd_from(0.0);
     for (int64_t k = tid; k < kend; k += kActThreads) {
         const int64_t hk = hist[k];
-        if (hk != 0) sum = dd_add(sum, dd_mul(dd_from_i64(hk), f[k]));
+        if (hk != 0) sum = dd_accumulate(sum, hk, f[k]);
     }
     red[tid] = sum;
     __syncthreads();
@@ -888,7 +892,10 @@ int cs_batch_launch(const cs_batch* b, const double* eps_host, int n_eps, int64_
             // cutoffs) spreads over every SM's FP64 pipe
             int64_t g = (at + int64_t(b->nsets) * a.n + 31) / 32;
             if (g > int64_t(sms) * 16) g = int64_t(sms) * 16;
-            k_batch_coef<<<unsigned(g), 32, 0, st>>>(b->coef, c, a, b->sets_dev, b->nsets, b->kends);
+            BatchPowers powers;
+            for (int e = 0; e < kMaxEps; ++e)
+                if (e < n_eps && !is_local(a.v[e])) powers.e[e] = eps_powers(a.v[e]);
+            k_batch_coef<<<unsigned(g), 32, 0, st>>>(b->coef, c, a, powers, b->sets_dev, b->nsets, b->kends);
         }
         k_batch_action<<<unsigned(b->nsets * (a.n > 0 ? a.n : 1)), kActThreads, 0, st>>>(
             b->sets_dev, hist_dev, a, b->coef, c, b->kends, actions_dev, brackets_dev);
