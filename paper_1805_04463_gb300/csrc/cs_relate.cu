@@ -20,7 +20,7 @@ namespace {
 
 // Relate kernel alone, before (a lane per word, or 64 tests per two ballots
 // for the circle) / now: 3+1 n = 16384 102 / 45 us, 2+1 n = 20011 150 / 57 us,
-// de Sitter slab n = 50021 632 / 268 us, 1+1 diamond n = 30011 79 / 81 us, 2D
+// de Sitter slab n = 50021 632 / 253 us, 1+1 diamond n = 30011 79 / 79 us, 2D
 // order n = 131072 789 / 802 us.  What bounds it now is the integer pipe (the
 // circle 83%, the light cone 70%), in 3+1 the FMA pipe (53%) with it (44%).
 template <int G>

@@ -410,17 +410,28 @@ __device__ __forceinline__ void relate_block(const int32_t* __restrict__ coords,
                     if constexpr (G == kGeomDeSitter) exact[r] = row[r].nu == __ldg(coords + 64 * W);
                 }
             }
-#pragma unroll
-            for (int r = 0; r < 2; ++r) {
-                uint32_t todo = __ballot_sync(0xffffffffu, exact[r] && r0 + lane + 32 * r < n);
-                if (todo) {  // warp-uniform
-                    const ExactWord<G> ex(coords, n, W);
-#pragma unroll 2
-                    for (; todo; todo &= todo - 1u) {
-                        const int q = __ffs(int(todo)) - 1;
-                        const uint64_t y = ex.row(coords, n, r0 + 32 * r + q);
-                        if (lane == q) found[r] = y;
+            const uint32_t todo0 = __ballot_sync(0xffffffffu, exact[0] && r0 + lane < n);
+            const uint32_t todo1 = __ballot_sync(0xffffffffu, exact[1] && r0 + lane + 32 < n);
+            if (todo0 | todo1) {  // warp-uniform
+                const ExactWord<G> ex(coords, n, W);
+                if ((!kFilter && W == rb) || !fast) {  // every row: their loads overlap
+#pragma unroll 4
+                    for (int q = 0; q < 32; ++q) {
+                        const uint64_t y0 = ex.row(coords, n, r0 + q < n ? r0 + q : n - 1);
+                        const uint64_t y1 = ex.row(coords, n, r0 + 32 + q < n ? r0 + 32 + q : n - 1);
+                        if (lane == q) {
+                            found[0] = y0;
+                            found[1] = y1;
+                        }
                     }
+                } else {
+#pragma unroll
+                    for (int r = 0; r < 2; ++r)
+                        for (uint32_t todo = r == 0 ? todo0 : todo1; todo; todo &= todo - 1u) {
+                            const int q = __ffs(int(todo)) - 1;
+                            const uint64_t y = ex.row(coords, n, r0 + 32 * r + q);
+                            if (lane == q) found[r] = y;
+                        }
                 }
             }
         }
