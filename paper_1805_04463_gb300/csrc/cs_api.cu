@@ -436,71 +436,80 @@ int cs_evaluate(int kind, int64_t n, uint64_t seed, const int32_t* coords_host, 
     if (cs_sprinkle_workspace_bytes(kind, n) > ws_bytes) ws_bytes = cs_sprinkle_workspace_bytes(kind, n);
     if (action_workspace_bytes() > ws_bytes) ws_bytes = action_workspace_bytes();
 
-    int32_t* coords = nullptr;
-    uint64_t* bits = nullptr;
-    int64_t* hist = nullptr;
-    void* ws = nullptr;
-    double* out = nullptr;  // [16] actions, then the bracket as int64
-    int rc = CS_OK;
-    auto alloc = [&](void** p, size_t b) {
-        if (rc == CS_OK && (fault_injected(CS_FAULT_ALLOC) || cudaMallocAsync(p, b, st) != cudaSuccess))
-            rc = CS_ENOMEM;
+    // One block for everything: coordinates, bitset, histogram, workspace, and
+    // the results: [16] actions, the bracket as int64, the status words of the
+    // sprinkle and the count.
+    size_t total = 0;
+    auto take = [&](size_t b) {
+        const size_t at = total;
+        total = align_up(total + b, 1024);
+        return at;
     };
-    alloc(reinterpret_cast<void**>(&coords), cs_coords_bytes(kind, n));
-    if (bits_bytes) alloc(reinterpret_cast<void**>(&bits), bits_bytes);
-    alloc(reinterpret_cast<void**>(&hist), size_t(hl) * 8);
-    alloc(&ws, ws_bytes);
-    alloc(reinterpret_cast<void**>(&out), 17 * 8);
+    const size_t at_coords = take(cs_coords_bytes(kind, n)), at_bits = take(bits_bytes), at_hist = take(size_t(hl) * 8),
+                 at_ws = take(ws_bytes), at_out = take(18 * 8);
+    uint8_t* mem = nullptr;
+    int rc = CS_OK;
+    if (fault_injected(CS_FAULT_ALLOC) || cudaMallocAsync(reinterpret_cast<void**>(&mem), total, st) != cudaSuccess)
+        rc = CS_ENOMEM;
+    int32_t* coords = reinterpret_cast<int32_t*>(mem + at_coords);
+    uint64_t* bits = reinterpret_cast<uint64_t*>(mem + at_bits);
+    int64_t* hist = reinterpret_cast<int64_t*>(mem + at_hist);
+    void* ws = mem + at_ws;
+    double* out = reinterpret_cast<double*>(mem + at_out);
     int64_t* bracket = reinterpret_cast<int64_t*>(out + 16);
+    int32_t* words = reinterpret_cast<int32_t*>(out + 17);
+    // The status word of the step just queued, kept beside the results: each
+    // copy to pageable host memory drains the stream, so there is one, at the
+    // end (five of them, one before the causal matrix was even queued, cost
+    // 40 us of a small set's call).
+    auto keep_status = [&](int which) {
+        return from_cuda(cudaMemcpyAsync(words + which, &static_cast<WsHeader*>(ws)->status, sizeof(int32_t),
+                                         cudaMemcpyDeviceToDevice, st));
+    };
 
+    if (rc == CS_OK) rc = from_cuda(cudaMemsetAsync(out, 0, 18 * 8, st));
     if (rc == CS_OK) {
         if (coords_host)
             rc = from_cuda(cudaMemcpyAsync(coords, coords_host, cs_coords_bytes(kind, n), cudaMemcpyHostToDevice, st));
         else
             rc = cs_sprinkle(kind, n, seed, coords, ws, ws_bytes, st);
     }
-    int32_t status_sprinkle = 0;
-    if (rc == CS_OK && !coords_host)
-        rc = from_cuda(cudaMemcpyAsync(&status_sprinkle, &static_cast<WsHeader*>(ws)->status, sizeof(int32_t),
-                                       cudaMemcpyDeviceToHost, st));
+    if (rc == CS_OK && !coords_host && dim > 2) rc = keep_status(0);  // only rejection sampling can fail
     if (by_coords) {
         if (rc == CS_OK) rc = cs_coords_abundance(kind, n, coords, hist, ws, ws_bytes, st);
     } else {
         if (rc == CS_OK) rc = cs_causal_matrix(kind, n, coords, bits, rw, st);
         if (rc == CS_OK) rc = cs_interval_abundance(n, bits, rw, hist, path, ws, ws_bytes, st);
+        if (rc == CS_OK) rc = keep_status(1);
     }
-    int32_t status = 0;
-    if (rc == CS_OK)
-        rc = from_cuda(cudaMemcpyAsync(&status, &static_cast<WsHeader*>(ws)->status, sizeof(status),
-                                       cudaMemcpyDeviceToHost, st));
-    if (rc == CS_OK && n_eps > 0) {
+    if (rc == CS_OK && n_eps > 0)
         rc = cs_action_device(dim, n, hist, hl, eps_host, n_eps, out, bracket, ws, ws_bytes, st);
-        if (rc == CS_OK)
-            rc = from_cuda(cudaMemcpyAsync(actions_host, out, size_t(n_eps) * 8, cudaMemcpyDeviceToHost, st));
-    }
-    if (rc == CS_OK && bracket_host) {
-        if (n_eps == 0) rc = cs_action_device(dim, n, hist, hl, eps_host ? eps_host : &kZero, 1, out, bracket, ws,
-                                              ws_bytes, st);
-        if (rc == CS_OK) rc = from_cuda(cudaMemcpyAsync(bracket_host, bracket, 8, cudaMemcpyDeviceToHost, st));
-    }
+    else if (rc == CS_OK && bracket_host)
+        rc = cs_action_device(dim, n, hist, hl, eps_host ? eps_host : &kZero, 1, out, bracket, ws, ws_bytes, st);
     if (rc == CS_OK && hist_host)
         rc = from_cuda(cudaMemcpyAsync(hist_host, hist, size_t(hl) * 8, cudaMemcpyDeviceToHost, st));
-    if (coords) cudaFreeAsync(coords, st);
-    if (bits) cudaFreeAsync(bits, st);
-    if (hist) cudaFreeAsync(hist, st);
-    if (ws) cudaFreeAsync(ws, st);
-    if (out) cudaFreeAsync(out, st);
+    struct {
+        double actions[16];
+        int64_t bracket;
+        int32_t status[2];
+    } got = {};
+    static_assert(sizeof(got) == 18 * 8, "the results' layout on the device");
+    if (rc == CS_OK) rc = from_cuda(cudaMemcpyAsync(&got, out, sizeof(got), cudaMemcpyDeviceToHost, st));
+    if (mem) cudaFreeAsync(mem, st);
     if (cudaStreamSynchronize(st) != cudaSuccess && rc == CS_OK) rc = CS_ECUDA;
+    if (rc == CS_OK) {
+        for (int e = 0; e < n_eps; ++e) actions_host[e] = got.actions[e];
+        if (bracket_host) *bracket_host = got.bracket;
+    }
     // Freed blocks stay in the pool for the next call, except after a call
     // that took more than a quarter of the device: those go back at once, so
     // one very large evaluation does not hold its memory for the process.
-    const size_t took = cs_coords_bytes(kind, n) + bits_bytes + size_t(hl) * 8 + ws_bytes;
-    if (took > device_total_memory() / 4) {
+    if (total > device_total_memory() / 4) {
         cudaMemPool_t pool;
         if (cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess) cudaMemPoolTrimTo(pool, 0);
     }
-    if (rc == CS_OK && status_sprinkle != 0) rc = status_sprinkle;
-    if (rc == CS_OK && status != 0) rc = status;
+    if (rc == CS_OK && got.status[0] != 0) rc = got.status[0];
+    if (rc == CS_OK && got.status[1] != 0) rc = got.status[1];
     return rc;
 }
 
