@@ -13,6 +13,10 @@ that copy lands.  Admission is bounded by the bitset memory of the active
 requests (n^2/8 bytes each), by their tensor-core operand memory, and by a
 slot count.
 
+With path AUTO a product order (a random 2D order, a 1+1 diamond or square) is
+counted whole from its coordinates behind its sprinkle, without operands or
+ticks: that takes less than the bookkeeping of its slices would.
+
 Counts are integer additions, so a request's histogram and actions are
 identical whether it runs alone or in the mix (tests/test_gpu_serve.py).
 
@@ -46,6 +50,7 @@ class Request:
     t_done: float = math.nan
     bitset_bytes: int = 0
     operand_bytes: int = 0
+    by_coords: bool = False      # counted from its coordinates
     # device / host buffers
     buf: object = None
     operands: object = None
@@ -99,12 +104,14 @@ class Server:
         self.torch = torch
         self.device = device
         self.eps = tuple(eps)
+        self.by_coords = False
         if path == cs.PATH_AUTO:
             # the FP4 pair path wherever the device has tcgen05: the large
             # requests dominate the work, and there it runs 2.2x the FP8 rate
             # (GB300, 200 req/s mix: p50 2.3 vs 6.8 ms, p99 31 vs 79 ms).
             # Asked at 2^16, the largest request size, whose operands fit.
             path = cs.PATH_MMA4 if cs.resolved_path(1 << 16) in (cs.PATH_MMA, cs.PATH_MMA4) else cs.PATH_POPC
+            self.by_coords = True  # and product orders from their coordinates, in one piece
         self.count_path = path
         self.bitset_budget = bitset_budget
         self.operand_budget = operand_budget
@@ -124,10 +131,25 @@ class Server:
         self.slot_events = [None] * ticks_in_flight
 
     # -- per request ------------------------------------------------------
+    def _admit_coords(self, r):
+        """A product order: sprinkled and counted whole on the preparation stream (0.1 to 1.3 ms up to
+        2^16 elements, less than its share of one tick), no causal matrix and no items left to grant."""
+        torch, st = self.torch, self.prep_stream
+        with torch.cuda.stream(st):
+            cs.sprinkle(r.kind, r.n, r.seed, r.buf.coords, r.buf.workspace, st)
+            cs.coords_abundance(r.kind, r.n, r.buf.coords, r.buf.hist, r.buf.workspace, st)
+        self._finish(r, st)
+
     def _admit(self, r, now):
         torch = self.torch
         r.state, r.t_admit = "prep", now
         r.buf = cs.allocate(r.kind, r.n, device=self.device, path=cs.PATH_POPC)
+        if r.by_coords:
+            need = cs.coords_abundance_workspace(r.kind, r.n)
+            if r.buf.workspace.numel() < need:
+                r.buf.workspace = torch.empty(need, dtype=torch.uint8, device=self.device)
+            self._admit_coords(r)
+            return
         r.total_items = cs.count_items(r.n, self.count_path)
         with torch.cuda.stream(self.prep_stream):
             st = self.prep_stream
@@ -142,10 +164,11 @@ class Server:
             r.prep_event = torch.cuda.Event()
             r.prep_event.record(st)
 
-    def _finish(self, r):
-        """Queue actions and the copies home behind the request's last slice."""
+    def _finish(self, r, st=None):
+        """Queue actions and the copies home behind the request's last slice (or, on the preparation
+        stream, its whole count)."""
         torch = self.torch
-        st = self.count_stream
+        st = st or self.count_stream
         with torch.cuda.stream(st):
             cs.action_device(r.buf.dim, r.n, r.buf.hist, list(self.eps), r.buf.actions, r.buf.bracket,
                              r.buf.workspace, st)
@@ -185,7 +208,8 @@ class Server:
         reqs = [Request(i, k, n, sd, t) for i, (t, k, n, sd) in enumerate(requests)]
         for r in reqs:
             r.bitset_bytes = cs.bitset_bytes(r.n)
-            r.operand_bytes = cs.operands_bytes(r.n, self.count_path) if self.tensor else 0
+            r.by_coords = self.by_coords and cs.coords_abundance_workspace(r.kind, r.n) > 0
+            r.operand_bytes = cs.operands_bytes(r.n, self.count_path) if self.tensor and not r.by_coords else 0
         queue = collections.deque(sorted(reqs, key=lambda r: (r.t_arrival, r.rid)))
         active = []
         used_b = used_o = 0

@@ -130,3 +130,20 @@ def test_batch_counts_product_orders_from_coordinates(cs, oracle, others):
     g.replay()
     torch.cuda.synchronize()
     assert torch.equal(b.hist, ref)
+
+
+def test_server_counts_orders_whole_among_sliced_requests(cs):
+    """AUTO server: product orders and other kinds together; each as alone."""
+    import torch
+    from paper_1805_04463_gb300 import serve
+    reqs = [(0.0, (0, 2, 1, 3, 5, 4)[r % 6], 1030 + 517 * r, 60 + r) for r in range(14)]
+    srv = serve.Server(tick_macs=2e9)
+    for _ in range(2):
+        stats, res = srv.run(reqs, realtime=False)
+        assert stats["requests"] == len(reqs)
+        for rid, (_, kind, n, seed) in enumerate(reqs):
+            buf = cs.allocate(kind, n, path=3)
+            cs.run(buf, seed, eps=serve.EPS)
+            torch.cuda.synchronize()
+            assert (res[rid][0] == buf.hist.cpu().numpy()).all(), rid
+            assert np.allclose(res[rid][1], buf.actions.cpu().numpy()[:4], rtol=1e-12, atol=1e-12)
