@@ -123,19 +123,21 @@ __global__ void __launch_bounds__(kThreads) k_keys(int64_t n, uint64_t seed, con
 // L2 in 16-byte words) and scans its own, so the blocks need not wait on one
 // another.  One block that walked all 65536 buckets, each thread its own run
 // of 64, took 103-110 us whatever n was (16-byte sectors of 64 separate
-// lines per thread and store); this takes about 3.
-__global__ void __launch_bounds__(256) k_bucket_scan(SprinkleScratch s, int64_t n) {
+// lines per thread and store); this takes about 5.
+constexpr int kScanThreads = 1024;  // the last blocks' sums in two rounds of loads
+__global__ void __launch_bounds__(kScanThreads) k_bucket_scan(SprinkleScratch s, int64_t n) {
     const uint32_t* count = s.count[blockIdx.y];
     uint32_t* start = s.start[blockIdx.y];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const uint4* c4 = reinterpret_cast<const uint4*>(count);
     uint32_t before = 0;
 #pragma unroll 8
-    for (int g = t; g < int(blockIdx.x) * (kScanBuckets / 4); g += 256) {
+    for (int g = t; g < int(blockIdx.x) * (kScanBuckets / 4); g += kScanThreads) {
         const uint4 v = c4[g];
         before += v.x + v.y + v.z + v.w;
     }
-    const uint4 own = c4[blockIdx.x * (kScanBuckets / 4) + t];
+    const bool mine = t < kScanBuckets / 4;  // threads with own buckets, four each
+    const uint4 own = mine ? c4[blockIdx.x * (kScanBuckets / 4) + t] : make_uint4(0u, 0u, 0u, 0u);
     const uint32_t sum = own.x + own.y + own.z + own.w;
     uint32_t incl = sum;
 #pragma unroll
@@ -144,16 +146,15 @@ __global__ void __launch_bounds__(256) k_bucket_scan(SprinkleScratch s, int64_t 
         if (lane >= o) incl += y;
         before += __shfl_xor_sync(0xffffffffu, before, o);
     }
-    __shared__ uint32_t wsum[8], wbefore[8];
+    __shared__ uint32_t wsum[kScanThreads / 32], wbefore[kScanThreads / 32];
     if (lane == 31) wsum[warp] = incl;
     if (lane == 0) wbefore[warp] = before;
     __syncthreads();
-    uint32_t at = incl - sum;
-#pragma unroll
-    for (int w = 0; w < 8; ++w) at += wbefore[w] + (w < warp ? wsum[w] : 0u);
+    if (!mine) return;
+    uint32_t at = incl - sum + __reduce_add_sync(0xffffffffu, wbefore[lane] + (lane < warp ? wsum[lane] : 0u));
     reinterpret_cast<uint4*>(start)[blockIdx.x * (kScanBuckets / 4) + t] =
         make_uint4(at, at + own.x, at + own.x + own.y, at + own.x + own.y + own.z);
-    if (t == 255 && blockIdx.x == gridDim.x - 1) start[gridDim.x * kScanBuckets] = uint32_t(n);
+    if (t == kScanBuckets / 4 - 1 && blockIdx.x == gridDim.x - 1) start[gridDim.x * kScanBuckets] = uint32_t(n);
 }
 
 __global__ void __launch_bounds__(kThreads) k_bucket_fill(int64_t n, SprinkleScratch s, int bits) {
@@ -315,7 +316,7 @@ cudaError_t sprinkle_kind(int64_t n, uint64_t seed, const uint64_t* thr, int32_t
     if (err != cudaSuccess) return err;
     const unsigned g = unsigned(grid_for(n));
     k_keys<KIND><<<g, kThreads, 0, st>>>(n, seed, thr, s, L.bits, hdr);
-    k_bucket_scan<<<dim3(unsigned(buckets / kScanBuckets), kStreams), 256, 0, st>>>(s, n);
+    k_bucket_scan<<<dim3(unsigned(buckets / kScanBuckets), kStreams), kScanThreads, 0, st>>>(s, n);
     k_bucket_fill<<<dim3(g, kStreams), kThreads, 0, st>>>(n, s, L.bits);
     k_rank_scatter<<<g, kThreads, 0, st>>>(n, kind_dim(KIND), kOrder, s, L.bits, coords);
     return cudaGetLastError();
