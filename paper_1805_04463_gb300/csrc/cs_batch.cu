@@ -111,20 +111,20 @@ __global__ void __launch_bounds__(256) k_batch_keys(const BatchSet* __restrict__
 }
 
 // One CTA per set: exact rank of each element (ties by index), then the
-// time-sorted coordinates.  Shared memory: keys 8P, bucket cursors 4P,
-// bucket slots 4P, ranks 4P (and the u ranks 4P of a 2D order): 24P bytes.
+// time-sorted coordinates.  Shared memory: keys 8n, bucket cursors 4P,
+// bucket slots 4n, ranks 4n (and the u ranks 4n of a 2D order), P <= max(n, 1024).
 __global__ void __launch_bounds__(kRankThreads) k_batch_rank(const BatchSet* __restrict__ sets) {
     extern __shared__ uint8_t smem_raw[];
     const BatchSet& b = sets[blockIdx.x];
     const int n = int(b.n);
-    int lgP = 10;  // at least kRankThreads buckets (the scan's runs)
-    while ((1 << lgP) < n) ++lgP;
+    int lgP = 10;  // at least kRankThreads buckets (the scan's runs), one to two elements each
+    while ((2 << lgP) <= n) ++lgP;
     const int P = 1 << lgP;
     uint64_t* sk = reinterpret_cast<uint64_t*>(smem_raw);
-    uint32_t* cnt = reinterpret_cast<uint32_t*>(sk + P);
+    uint32_t* cnt = reinterpret_cast<uint32_t*>(sk + n);
     uint32_t* slot = cnt + P;
-    uint32_t* rank = slot + P;
-    uint32_t* ru = rank + P;
+    uint32_t* rank = slot + n;
+    uint32_t* ru = rank + n;
     int32_t* op = const_cast<int32_t*>(b.order.p);
     int32_t* oq = const_cast<int32_t*>(b.order.q);
     if (by_order(b) && b.kind != CS_2D_ORDER) {  // the count needs the ranks of u and v, not the time order
@@ -439,7 +439,7 @@ struct cs_batch {
     int64_t ord_blocks = 0, ord_tasks = 0;
     int64_t ord_nmax = 0;      // the largest of them
     unsigned geoms = 0;  // bit G: some set relates with geometry G
-    int max_pow2 = 1;
+    int64_t n_largest = 1;
     const uint64_t* ds_thr = nullptr;  // de Sitter thresholds, when a set needs them
     dd* coef = nullptr;                 // smeared-sum coefficient tables
     int64_t* kends = nullptr;           // per (set, eps): smeared-sum cutoff [set * kMaxEps + e]
@@ -589,7 +589,7 @@ int cs_batch_create(const cs_set_desc* sets, int n_sets, int path, void* workspa
     int64_t elem = 0, rblk = 0, mblk = 0, hoff = 0, tiles = 0;
     int64_t ord_blocks = 0, ord_tasks = 0, ord_nmax = 0;
     std::vector<int32_t> otab, osets;
-    int max_pow2 = 1;
+    int64_t n_largest = 1;
     for (int s = 0; s < n_sets; ++s) {
         BatchSet& b = bs[s];
         b.kind = sets[s].kind;
@@ -632,7 +632,7 @@ int cs_batch_create(const cs_set_desc* sets, int n_sets, int path, void* workspa
         mblk += b.mir_side * b.mir_side;
         b.hist_off = hoff;
         hoff += cs_hist_len(b.n);
-        while (max_pow2 < b.n) max_pow2 <<= 1;
+        n_largest = b.n > n_largest ? b.n : n_largest;
     }
     // Count tables in decreasing set size (the largest sets' tiles go first).
     std::vector<int> order(static_cast<size_t>(n_sets));
@@ -734,7 +734,7 @@ int cs_batch_create(const cs_set_desc* sets, int n_sets, int path, void* workspa
     h->ttab = reinterpret_cast<int32_t*>(ws + L.ttab);
     h->etab = reinterpret_cast<int32_t*>(ws + L.etab);
     h->total_hist = hoff;
-    h->max_pow2 = max_pow2;
+    h->n_largest = n_largest;
     h->ds_thr = ds_thr;
     h->coef = reinterpret_cast<dd*>(ws + L.coef);
     h->kends = reinterpret_cast<int64_t*>(ws + L.kends);
@@ -804,7 +804,9 @@ int cs_batch_launch(const cs_batch* b, const double* eps_host, int n_eps, int64_
     if (g > int64_t(sms) * 16) g = int64_t(sms) * 16;
     k_batch_keys<<<unsigned(g), 256, 0, st>>>(b->sets_dev, b->nsets, b->total_elems, b->ds_thr, b->hdr);
 
-    const size_t rank_smem = size_t(b->max_pow2 > kRankThreads ? b->max_pow2 : kRankThreads) * 24;
+    // sized by the largest set itself: rounded up to a power of two, a batch
+    // whose sets scatter around 4096 left room for one CTA per SM instead of two
+    const size_t rank_smem = size_t(b->n_largest) * 20 + size_t(b->n_largest > kRankThreads ? b->n_largest : kRankThreads) * 4;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return CS_ECUDA;
     if (dev >= 0 && dev < 64 && !g_rank_attr[dev]) {

@@ -83,17 +83,17 @@ __device__ __forceinline__ void order_keys_smem(const int32_t* __restrict__ val,
 }
 
 // p and q of a set of at most 8192 elements by one CTA of kRankThreads
-// threads: u NULL: the labels are in u order.  smem: 24 << lgP bytes
-// (keys, bucket counts, slots, ranks, u ranks), 2^lgP >= max(n, kRankThreads).
+// threads; by_u: the labels are in u order.  smem: 20 n bytes (keys, slots,
+// ranks, u ranks) and 4 << lgP (bucket counts), 2^lgP >= kRankThreads.
 __device__ __forceinline__ void order_ranks_smem(const int32_t* __restrict__ u, const int32_t* __restrict__ v, bool by_u,
                                                  int n, int lgP, uint8_t* smem, int32_t* __restrict__ p,
                                                  int32_t* __restrict__ q) {
     const int P = 1 << lgP;
     uint64_t* sk = reinterpret_cast<uint64_t*>(smem);
-    uint32_t* cnt = reinterpret_cast<uint32_t*>(sk + P);
+    uint32_t* cnt = reinterpret_cast<uint32_t*>(sk + n);
     uint32_t* slot = cnt + P;
-    uint32_t* rank = slot + P;
-    uint32_t* ru = rank + P;
+    uint32_t* rank = slot + n;
+    uint32_t* ru = rank + n;
     if (!by_u) {
         order_keys_smem(u, v, n, sk);
         rank_keys_smem(n, lgP, sk, cnt, slot, ru);

@@ -32,7 +32,7 @@ def _order(v):
 
 # one band, its edges, one tile of the ranks and its edges, several words of the table's step
 @pytest.mark.parametrize("kind", [0, 1, 5])
-@pytest.mark.parametrize("n", [2, 3, 31, 32, 33, 64, 65, 255, 257, 1023, 1024, 1025, 2049, 4133, 8193, 9001])
+@pytest.mark.parametrize("n", [2, 3, 31, 32, 33, 64, 65, 255, 257, 1023, 1024, 1025, 2049, 3071, 3072, 3073, 4133, 8193, 9001])
 def test_sprinkled(cs, oracle, kind, n):
     c = oracle.sprinkle(kind, n, 0x0D0 + n)
     want = oracle.interval_abundance(oracle.causal_matrix(kind, c))
@@ -105,7 +105,7 @@ def test_batch_counts_product_orders_from_coordinates(cs, oracle, others):
     """AUTO batches at the edges of bands, chunks and table steps, with and without sets that need
     their causal matrix; replayed as a graph too."""
     import torch
-    sets = [(k, n, 900 + 7 * n + k) for k in (0, 1, 5) for n in (2, 3, 63, 64, 65, 128, 129, 1000, 2049)]
+    sets = [(k, n, 900 + 7 * n + k) for k in (0, 1, 5) for n in (2, 3, 63, 64, 65, 128, 129, 1000, 2049, 3073)]
     sets += [(1, 8192, 31), (0, 8191, 32), (5, 4097, 33)]
     if others:
         sets = [(2, 700, 1), (4, 333, 2)] + sets + [(3, 1025, 3), (0, 1, 4), (6, 100, 5)]
