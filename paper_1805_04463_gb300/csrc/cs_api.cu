@@ -37,16 +37,16 @@ inline cudaError_t clear_status(void* ws, cudaStream_t st) {
 }  // namespace
 
 // CS_PATH_AUTO table: entry e applies from size n_min[e] up to the next
-// entry.  The default follows GB300 measurements of random 2D orders: the
-// FP8 tensor path beats POPC from n = 1024 (0.032 vs 0.042 ms), the FP4 pair
-// path beats FP8 from n = 4096 (0.038 vs 0.044 ms; 12.1 vs 27.3 ms at
-// 65536, 89.5 vs 224 ms at 131072); the autotuner replaces it with
-// thresholds measured on the running device.
+// entry.  The default follows GB300 measurements of 3+1 diamonds and de Sitter
+// slabs (us, POPC / FP8 / FP4 pairs): n = 300 37 / 17 / 20, 700 42 / 19 / 21,
+// 1500 62 / 22 / 24, 2048 63 / 26 / 24, 3000 129 / 29 / 26, 4096 225 / 37 / 29;
+// 2D orders at 65536 27300 (FP8) / 12100 (FP4).  The autotuner replaces it
+// with thresholds measured on the running device.
 constexpr int kMaxAuto = 16;
 std::mutex g_auto_mu;
-int64_t g_auto_n[kMaxAuto] = {0, 1024, 4096};
-int g_auto_p[kMaxAuto] = {CS_PATH_POPC, CS_PATH_MMA, CS_PATH_MMA4};
-int g_auto_count = 3;
+int64_t g_auto_n[kMaxAuto] = {0, 2048};
+int g_auto_p[kMaxAuto] = {CS_PATH_MMA, CS_PATH_MMA4};
+int g_auto_count = 2;
 
 // Tile choices.  Raster side per size bucket of the single-set tensor
 // counts (default 8 everywhere: a GB300 sweep of 4..16 found 8 best or
