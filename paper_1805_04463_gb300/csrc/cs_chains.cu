@@ -24,6 +24,7 @@
 // checks of the number of elements left (rounds after the last one find
 // nothing to do).
 #include "cs_kernels.cuh"
+#include "cs_relate.cuh"
 
 namespace cs {
 
@@ -291,7 +292,8 @@ __device__ bool grid_barrier(ChainState* st, unsigned int r) {
 //
 // Two barriers a round of 1216 small blocks, and every element's row scanned
 // from its label down each round, took 20 us a round at n = 32768 (7.2 ms
-// for the 362 of a 2D order).
+// for the 355 of a 2D order); this takes 5.9 us.
+constexpr int kWide = 8;
 template <int kSlots>
 __global__ void __launch_bounds__(kPersistThreads) k_chain_persist(const uint64_t* __restrict__ bits,
                                                                    int64_t row_words, int64_t lo, int64_t hi,
@@ -337,19 +339,26 @@ __global__ void __launch_bounds__(kPersistThreads) k_chain_persist(const uint64_
                 int64_t w1 = __shfl_sync(0xffffffffu, w[t], f) - 1;  // the next word to look at
                 int64_t at = -1;
                 uint64_t found = 0ull;
-                while (w1 >= wlo) {
-                    // lane l: words w1 - l and w1 - 32 - l
-                    const int64_t wa = w1 - lane, wc = wa - 32;
-                    const uint64_t xa = wa >= wlo ? __ldg(row + wa) : 0ull, xc = wc >= wlo ? __ldg(row + wc) : 0ull;
-                    const uint32_t ma = __ballot_sync(0xffffffffu, wa >= wlo && (xa & S[wa]) != 0ull);
-                    const uint32_t mc = __ballot_sync(0xffffffffu, wc >= wlo && (xc & S[wc]) != 0ull);
-                    if (ma | mc) {  // the nearest one
-                        const int q = __ffs(int(ma ? ma : mc)) - 1;
-                        at = w1 - q - (ma ? 0 : 32);
-                        found = __shfl_sync(0xffffffffu, ma ? xa : xc, q);
-                        break;
+                // 64 words at first, where the next one usually is, then 256 at a
+                // time: a round waits for its longest search
+                for (int width = 2; w1 >= wlo; w1 -= 32 * width, width = kWide) {
+                    uint64_t y[kWide];  // lane l: words w1 - l - 32 c
+#pragma unroll
+                    for (int c = 0; c < kWide; ++c) {
+                        const int64_t wc = w1 - lane - 32 * c;
+                        y[c] = c < width && wc >= wlo ? __ldg(row + wc) : 0ull;
                     }
-                    w1 -= 64;
+#pragma unroll
+                    for (int c = 0; c < kWide; ++c) {
+                        const int64_t wc = w1 - lane - 32 * c;
+                        const uint32_t m = __ballot_sync(0xffffffffu, wc >= wlo && (y[c] & S[wc < 0 ? 0 : wc]) != 0ull);
+                        if (m && at < 0) {  // the nearest one
+                            const int q = __ffs(int(m)) - 1;
+                            at = w1 - q - 32 * c;
+                            found = __shfl_sync(0xffffffffu, y[c], q);
+                        }
+                    }
+                    if (at >= 0) break;
                 }
                 if (lane == f) {
                     w[t] = int(at);
@@ -383,8 +392,8 @@ __global__ void __launch_bounds__(kPersistThreads) k_chain_persist(const uint64_
 // one 64-bit atomicMin, barrier; then every block for itself reads row k and
 // takes J(k) and k out of X, lists the candidates R that this removed (A loses
 // exactly these: the members are unrelated to every candidate), and lowers
-// its overlaps by the number of R's elements related to j, the warps of a
-// group taking R's rows in turn (a row's word serves 32 candidates).  The
+// its overlaps by the number of R's elements related to j, 32 rows by 32
+// candidates at a time (bit transposes), the warps of a group in turn.  The
 // overlaps are counted in full once, at the start.  Three barriers a round
 // and one thread per candidate walking R took 37 us a round at n = 32768.
 constexpr int kListCap = 4096;  // elements of R listed at a time
@@ -419,6 +428,7 @@ __global__ void __launch_bounds__(kPersistThreads) k_anti_persist(const uint64_t
         if (lane == 0) over[c] = o;
     }
     __syncthreads();
+    const Tr32 tc = tr32_consts(lane);
     // warps per group (a group per warp, in turn, when there are more groups)
     const int share = ng > 0 && ng < kPersistWarps ? kPersistWarps / ng : 1;
     int64_t taken = 0;
@@ -478,11 +488,14 @@ __global__ void __launch_bounds__(kPersistThreads) k_anti_persist(const uint64_t
             const int nr = listed < valid ? listed : valid;
             for (int g = warp / share; g < ng; g += kPersistWarps / share) {
                 if (warp / share >= kPersistWarps / share) break;  // the warps left over
+                // 32 rows at a time: lane l reads its row's word of the group,
+                // the transpose gives lane l the 32 rows' bits of column l
                 const uint32_t* col = reinterpret_cast<const uint32_t*>(bits) + (g0 + g);
                 int d = 0;
-#pragma unroll 8
-                for (int t = warp % share; t < nr; t += share) {
-                    d += int((__ldg(col + int64_t(list[t]) * row_words * 2) >> lane) & 1u);
+#pragma unroll 2
+                for (int t = 32 * (warp % share); t < nr; t += 32 * share) {
+                    const uint32_t v = t + lane < nr ? __ldg(col + int64_t(list[t + lane]) * row_words * 2) : 0u;
+                    d += __popc(transpose32(v, tc));
                 }
                 if (d) atomicSub(&over[32 * g + lane], d);
             }
