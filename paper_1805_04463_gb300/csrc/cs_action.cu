@@ -17,6 +17,11 @@ namespace cs {
 
 namespace {
 
+// Programmatic dependent launch: let the next kernel of the stream launch;
+// wait for the whole end of the kernel before (at once without one).
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_primary() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Blocks of the smeared sum of cutoff kend with T threads each: one term per
 // thread until kActBlocks blocks are full.
 __host__ __device__ inline int act_blocks(int64_t kend, int T) {
@@ -24,17 +29,20 @@ __host__ __device__ inline int act_blocks(int64_t kend, int T) {
     return int(b < kActBlocks ? b : kActBlocks);
 }
 
-// Partial smeared sums, grid (blocks of the longest cutoff, eps).  A term is
-// about 150 dependent FP64 operations (the power, the polynomial, two
-// products), and GB300 issues about two FP64 lanes per SM
-// and cycle: what bounds this is how few SMs the terms sit on.  So a block
-// is one warp while the cutoffs are below 4096 terms (wider beyond),
-// the eps values run side by side, and the sum is a shuffle tree.  256
+// Partial smeared sums, grid (blocks of the longest cutoff, eps).  GB300
+// issues about two FP64 lanes per SM and cycle, and a term is a chain of
+// FP64 operations: what bounds this is the chain's length and how few SMs
+// the terms sit on.  So a block is one warp while the cutoffs are below 4096
+// terms (wider beyond), the eps values run side by side, what does not
+// depend on k comes from the host, and the sum is a shuffle tree.  256
 // threads per block walking the eps values one after another took 102 us
-// for n = 1024 .. 16384 and three smeared eps; this takes 12 (19 while every
-// thread squared its own powers).
+// for n = 1024 .. 16384 and three smeared eps, squared powers per thread 19,
+// powers from the host in one chain and the polynomial formed per term 16.8;
+// this takes 10.8 (a whole pass over a 2D order of 1024, with the final
+// kernel's launch hidden behind it: 72 -> 63.5 us).
 struct ActPowers {
     EpsPowers e[kMaxEps];
+    SmearCoef c[kMaxEps];
 };
 __global__ void __launch_bounds__(kActThreads) k_action_partial(int dim, const int64_t* __restrict__ hist,
                                                                 EpsArgs eps, const __grid_constant__ ActPowers powers,
@@ -43,15 +51,13 @@ __global__ void __launch_bounds__(kActThreads) k_action_partial(int dim, const i
     const int e = blockIdx.y, T = blockDim.x, tid = threadIdx.x;
     const int64_t kend = eps.kend[e];  // 0 for a local action
     const int nb = act_blocks(kend, T);
+    launch_dependents();  // k_action_final's launch, beside this one
     if (int(blockIdx.x) >= nb) return;
-    const double ep = eps.v[e];
-    const dd q = dd_two_sum(1.0, -ep);
     dd sum = dd_from(0.0);
     for (int64_t k = int64_t(blockIdx.x) * T + tid; k < kend; k += int64_t(nb) * T) {
         const int64_t hk = hist[k];
         if (hk == 0) continue;
-        const dd f = dd_mul(power_of(powers.e[e], smear_qexp(dim, k)), smear_poly(dim, k, q, ep));
-        sum = dd_accumulate(sum, hk, f);
+        sum = dd_accumulate(sum, hk, smear_term(dim, powers.c[e], powers.e[e], k));
     }
     sum = warp_sum_dd(sum);
     if (T > 32) {  // uniform
@@ -63,6 +69,8 @@ __global__ void __launch_bounds__(kActThreads) k_action_partial(int dim, const i
 }
 
 // One warp per eps: its partial sums, the action; warp 0 writes the bracket.
+// After k_action_partial it is launched while that one runs, and waits here
+// for its end (hist was complete before k_action_partial began).
 __global__ void __launch_bounds__(32 * kMaxEps) k_action_final(int dim, int64_t n, const int64_t* __restrict__ hist,
                                                                int64_t len, EpsArgs eps, int T,
                                                                const dd* __restrict__ partial,
@@ -72,8 +80,9 @@ __global__ void __launch_bounds__(32 * kMaxEps) k_action_final(int dim, int64_t 
     int64_t h4[4] = {0, 0, 0, 0};
     for (int k = 0; k < 4 && k < len; ++k) h4[k] = hist[k];
     const int64_t b = bracket_of(dim, n, h4);
-    if (threadIdx.x == 0 && bracket) *bracket = b;
     const double ep = eps.v[e];
+    wait_for_primary();
+    if (threadIdx.x == 0 && bracket) *bracket = b;
     dd s;
     if (is_local(ep)) {
         s = local_action(eps.factor[e], b);
@@ -166,12 +175,28 @@ cudaError_t launch_action_device(int dim, int64_t n, const int64_t* hist, int64_
     if (kmax > 0) {
         ActPowers powers;
         for (int e = 0; e < kMaxEps; ++e)
-            if (e < n_eps && !is_local(a.v[e])) powers.e[e] = eps_powers(a.v[e]);
+            if (e < n_eps && !is_local(a.v[e])) {
+                powers.e[e] = eps_powers(a.v[e]);
+                powers.c[e] = smear_coef(dim, a.v[e]);
+            }
         k_action_partial<<<dim3(unsigned(act_blocks(kmax, T)), unsigned(n_eps)), T, 0, st>>>(dim, hist, a, powers,
                                                                                           partial);
     }
-    k_action_final<<<1, 32 * n_eps, 0, st>>>(dim, n, hist, len, a, T, partial, out, bracket);
-    return cudaGetLastError();
+    if (kmax == 0) {
+        k_action_final<<<1, 32 * n_eps, 0, st>>>(dim, n, hist, len, a, T, partial, out, bracket);
+        return cudaGetLastError();
+    }
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(1);
+    cfg.blockDim = dim3(unsigned(32 * n_eps));
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    const dd* sums = partial;
+    return cudaLaunchKernelEx(&cfg, k_action_final, dim, n, hist, len, a, T, sums, out, bracket);
 }
 
 }  // namespace cs

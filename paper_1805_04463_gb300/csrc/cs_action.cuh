@@ -26,11 +26,68 @@ inline EpsPowers eps_powers(double eps) {
     for (int b = 1; b < kPowBits; ++b) t.p[b] = dd_mul(t.p[b - 1], t.p[b - 1]);
     return t;
 }
+// Two chains side by side, the five low bits of k (which differ between the
+// lanes) and the bits above them (which do not): one product of all the bits
+// made the chain twice as long.
 __device__ __forceinline__ dd power_of(const EpsPowers& t, int64_t k) {
-    dd r = dd_from(1.0);
-    if (k >> kPowBits) r = dd_pow(dd_mul(t.p[kPowBits - 1], t.p[kPowBits - 1]), k >> kPowBits);  // a longer histogram
-    for (uint32_t m = uint32_t(k) & ((1u << kPowBits) - 1u); m; m &= m - 1u) r = dd_mul(r, t.p[__ffs(int(m)) - 1]);
+    const uint32_t m = uint32_t(k) & ((1u << kPowBits) - 1u);
+    uint32_t lo = m & 31u, hi = m & ~31u;
+    dd r = dd_from(1.0), s = dd_from(1.0);
+    if (lo) r = t.p[__ffs(int(lo)) - 1];
+    if (hi) s = t.p[__ffs(int(hi)) - 1];
+    lo &= lo - 1u;
+    hi &= hi - 1u;
+    while (lo | hi) {
+        r = dd_mul(r, lo ? t.p[__ffs(int(lo)) - 1] : dd_from(1.0));
+        s = dd_mul(s, hi ? t.p[__ffs(int(hi)) - 1] : dd_from(1.0));
+        lo &= lo - 1u;
+        hi &= hi - 1u;
+    }
+    r = dd_mul(r, s);
+    if (k >> kPowBits) r = dd_mul(r, dd_pow(dd_mul(t.p[kPowBits - 1], t.p[kPowBits - 1]), k >> kPowBits));  // a longer histogram
     return r;
+}
+
+// The polynomial factor of f_d (smear_poly) as a - b k + c t - d C(k, 3),
+// t = k (k - 1) / 2, its coefficients and the values f_d(k), k < deg, found
+// on the host: they hold no k, and were most of a term's FP64 operations.
+// Rounded once to double-double, they move a sum by less than 1e-30 of its
+// largest term (terms: the same error as with the products formed per k).
+struct SmearCoef {
+    dd a, b, c, d, f[3];
+};
+inline SmearCoef smear_coef(int dim, double eps) {
+    const dd q = dd_two_sum(1.0, -eps), e = dd_from(eps), q2 = dd_mul(q, q), e2 = dd_mul(e, e);
+    SmearCoef r;
+    r.d = dd_from(0.0);
+    if (dim == 2) {
+        r.a = q2, r.b = dd_mul(dd_mul_d(e, 2.0), q), r.c = e2;
+    } else if (dim == 3) {
+        r.a = q2, r.b = dd_mul(dd_mul_d(e, 3.375), q), r.c = dd_mul_d(e2, 2.25);
+    } else {
+        r.a = dd_mul(q2, q), r.b = dd_mul(dd_mul_d(e, 9.0), q2), r.c = dd_mul(dd_mul_d(e2, 16.0), q);
+        r.d = dd_mul_d(dd_mul(e2, e), 8.0);
+    }
+    for (int k = 0; k < 3; ++k) r.f[k] = smear_poly(dim, k, q, eps);
+    return r;
+}
+__host__ __device__ __forceinline__ dd smear_poly_at(int dim, const SmearCoef& m, int64_t k) {
+    const int64_t t = k * (k - 1) / 2;  // below 2^43 for k < 2^22: exact in a double
+    const dd bk = dd_mul_d(m.b, static_cast<double>(k)), ct = dd_mul_d(m.c, static_cast<double>(t));
+    dd r = dd_add(dd_sub(m.a, bk), ct);
+    if (dim == 4) {
+        const int64_t w = k - 2;
+        const dd c3 = w % 3 == 0 ? dd_two_prod(static_cast<double>(t), static_cast<double>(w / 3))
+                                 : dd_two_prod(static_cast<double>(t / 3), static_cast<double>(w));  // C(k, 3), exactly
+        r = dd_sub(r, dd_mul(m.d, c3));
+    }
+    return r;
+}
+// f_d(k).
+__device__ __forceinline__ dd smear_term(int dim, const SmearCoef& m, const EpsPowers& t, int64_t k) {
+    const int64_t deg = smear_deg(dim);
+    if (k < deg) return m.f[k];
+    return dd_mul(power_of(t, k - deg), smear_poly_at(dim, m, k));
 }
 
 // sum + c * f for a count c < 2^53 (exact as a double): the product to double-double,

@@ -325,6 +325,7 @@ struct CoefArgs {
 // costly to repeat in every thread of the action kernel.
 struct BatchPowers {
     EpsPowers e[kMaxEps];
+    SmearCoef c[kDimSlots][kMaxEps];
 };
 __global__ void __launch_bounds__(32) k_batch_coef(dd* __restrict__ coef, CoefArgs c, EpsArgs eps,
                                                     const __grid_constant__ BatchPowers powers,
@@ -347,10 +348,8 @@ __global__ void __launch_bounds__(32) k_batch_coef(dd* __restrict__ coef, CoefAr
         while (c.seg[g + 1] <= t) ++g;  // at most 48 segments
         const int slot = g / kMaxEps, e = g % kMaxEps, dim = slot + 2;
         const int64_t k = t - c.seg[g];
-        const double ep = eps.v[e];
-        const dd q = dd_two_sum(1.0, -ep);
         coef[c.base[slot] + e * c.stride[slot] + k] =
-            dd_mul(power_of(powers.e[e], smear_qexp(dim, k)), smear_poly(dim, k, q, ep));
+            smear_term(dim, powers.c[slot][e], powers.e[e], k);
     }
 }
 
@@ -896,7 +895,10 @@ int cs_batch_launch(const cs_batch* b, const double* eps_host, int n_eps, int64_
             if (g > int64_t(sms) * 16) g = int64_t(sms) * 16;
             BatchPowers powers;
             for (int e = 0; e < kMaxEps; ++e)
-                if (e < n_eps && !is_local(a.v[e])) powers.e[e] = eps_powers(a.v[e]);
+                if (e < n_eps && !is_local(a.v[e])) {
+                    powers.e[e] = eps_powers(a.v[e]);
+                    for (int d = 0; d < kDimSlots; ++d) powers.c[d][e] = smear_coef(d + 2, a.v[e]);
+                }
             k_batch_coef<<<unsigned(g), 32, 0, st>>>(b->coef, c, a, powers, b->sets_dev, b->nsets, b->kends);
         }
         k_batch_action<<<unsigned(b->nsets * (a.n > 0 ? a.n : 1)), kActThreads, 0, st>>>(

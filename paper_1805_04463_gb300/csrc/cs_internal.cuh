@@ -540,10 +540,4 @@ __host__ __device__ inline dd smear_poly(int dim, int64_t k, dd q, double eps) {
 // Degree of the polynomial factor of f_d (the power of 1/(1-eps) pulled out).
 __host__ __device__ __forceinline__ int64_t smear_deg(int dim) { return dim == 4 ? 3 : 2; }
 
-// Exponent of q multiplying smear_poly for index k.
-__host__ __device__ __forceinline__ int64_t smear_qexp(int dim, int64_t k) {
-    const int64_t deg = smear_deg(dim);
-    return k >= deg ? k - deg : 0;
-}
-
 }  // namespace cs
