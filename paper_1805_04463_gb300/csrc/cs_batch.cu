@@ -8,8 +8,10 @@
 //   k_batch_rank    one CTA per set: exact ranks of the keys by a bucket
 //                   count in shared memory give the time order; scatter
 //                   coordinates;
+//   k_batch_ctab    the column tables of the light-cone sets' bitsets;
 //   k_batch_relate  every relate chunk (32 words of a 64-row tile, from its
-//                   diagonal word) of every bitset, one launch per geometry;
+//                   diagonal word) of every bitset, one launch per geometry
+//                   (light cone: k_batch_relate_cone, from the tables);
 //   k_batch_mirror  the lower triangle of every bitset, the transpose of the
 //                   upper one (the past rows);
 //   order table, order count   on CS_PATH_AUTO, for the product orders (2D
@@ -19,7 +21,8 @@
 //   count           the multi-set POPC kernel, or expand + multi-set tcgen05
 //                   kernel: one persistent grid over the tiles of all sets,
 //                   largest sets first (longest-processing-time order);
-//   k_batch_action  one CTA per set: bracket and smeared sums.
+//   k_batch_coef    the smearing coefficients and cutoffs;
+//   k_batch_action  one CTA per (set, eps): bracket and smeared sums.
 // Ensembles of Poisson-sized sprinklings are the thesis's experimental unit
 // (Section "Simulations and Scaling Evaluations": ten graphs per size; the
 // appendix's sprinklings draw N from a Poisson distribution).
@@ -73,21 +76,40 @@ __host__ __device__ __forceinline__ bool by_order(const BatchSet& b) { return b.
 constexpr int kBatchOrderM = 2;
 constexpr int kBatchOrderThreads = 512;
 
-__device__ __forceinline__ int find_set_elem(const BatchSet* sets, int nsets, int64_t idx) {
-    int lo = 0, hi = nsets - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (sets[mid].elem_begin <= idx) lo = mid; else hi = mid - 1;
+// The set of element idx, by the whole warp (idx uniform): 32 probes at a
+// time, where a search by halves is ten dependent loads for a thousand sets.
+__device__ __forceinline__ int find_set_warp(const BatchSet* sets, int nsets, int64_t idx) {
+    const int lane = threadIdx.x & 31;
+    int lo = 0, count = nsets;  // sets[lo].elem_begin <= idx, the next one's after lo + count is not
+    while (count > 1) {
+        const int step = (count + 31) / 32, i = lane * step;
+        const uint32_t m = __ballot_sync(0xffffffffu, i < count && sets[lo + (i < count ? i : 0)].elem_begin <= idx);
+        const int j = (31 - __clz(m)) * step;
+        lo += j;
+        count = count - j < step ? count - j : step;
     }
     return lo;
 }
 
 __global__ void __launch_bounds__(256) k_batch_keys(const BatchSet* __restrict__ sets, int nsets, int64_t total,
                                                     const uint64_t* __restrict__ ds_thr, WsHeader* hdr) {
-    for (int64_t idx = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; idx < total;
-         idx += int64_t(gridDim.x) * blockDim.x) {
-        const BatchSet& b = sets[find_set_elem(sets, nsets, idx)];
+    const int lane = threadIdx.x & 31;
+    for (int64_t at = blockIdx.x * int64_t(blockDim.x) + (threadIdx.x & ~31); at < total;
+         at += int64_t(gridDim.x) * blockDim.x) {  // whole warps
+        const int64_t idx = at + lane;
+        int set = find_set_warp(sets, nsets, at);
+        while (set + 1 < nsets && sets[set + 1].elem_begin <= idx) ++set;
+        const BatchSet& b = sets[set];
         const int64_t e = idx - b.elem_begin;
+        int32_t c[4];
+        uint64_t key;
+        const bool in = idx < total;
+        const uint32_t in3 = __ballot_sync(0xffffffffu, in && b.kind == CS_3D_DIAMOND);
+        const uint32_t in4 = __ballot_sync(0xffffffffu, in && b.kind == CS_4D_DIAMOND);
+        bool ok = false;
+        if (in3) ok |= draw_diamond<3>(in3, stream_key(b.seed, kStreamDiamond3), e, c, key);
+        if (in4) ok |= draw_diamond<4>(in4, stream_key(b.seed, kStreamDiamond4), e, c, key);
+        if (!in) continue;
         if (b.kind == CS_2D_ORDER) {
             draw_2d_order(stream_key(b.seed, kStreamOrderU), stream_key(b.seed, kStreamOrderV), e, b.key0[e],
                           b.key1[e]);
@@ -100,10 +122,7 @@ __global__ void __launch_bounds__(256) k_batch_keys(const BatchSet* __restrict__
         } else if (b.kind == CS_2D_DS_SLAB) {
             b.key0[e] = draw_ds_slab(stream_key(b.seed, kStreamDeSitter), e, ds_thr, b.raw[e], b.raw[b.n + e]);
         } else {
-            int32_t c[4];
-            const bool ok = b.kind == CS_3D_DIAMOND
-                                ? draw_3d_diamond(stream_key(b.seed, kStreamDiamond3), e, c, b.key0[e])
-                                : draw_4d_diamond(stream_key(b.seed, kStreamDiamond4), e, c, b.key0[e]);
+            b.key0[e] = key;
             if (!ok) set_status(hdr, CS_ERANGE);
             for (int k = 0; k < b.dim; ++k) b.raw[k * b.n + e] = c[k];
         }
@@ -281,7 +300,7 @@ __global__ void __launch_bounds__(kRelThreads) k_batch_relate(const BatchSet* __
     relate_block<G>(b.coords, b.n, b.bits, b.row_words, rb, w0, sm, zero_from);
 }
 
-// The light-cone kinds, from the column tables k_batch_rank built (one
+// The light-cone kinds, from the column tables of k_batch_ctab (one
 // look-up per word instead of 64 cone tests).
 __global__ void __launch_bounds__(kRelThreads, 4) k_batch_relate_cone(const BatchSet* __restrict__ sets,
                                                                    const int32_t* __restrict__ rblock_set,

@@ -73,11 +73,18 @@ struct SprinkleScratch {
     uint32_t* start[2];    // first slot of a bucket; start[buckets] = n
 };
 
-// Draw element e of a set: its sort key (two for a 2D order) and, for the
-// other kinds, its coordinates.  false: no rejection attempt was accepted.
+// Draw element e < n of a set: its sort key (two for a 2D order) and, for the
+// other kinds, its coordinates.  All lanes of a warp (e = n or more: nothing
+// is drawn).  false: no rejection attempt was accepted.
 template <int KIND>
-__device__ __forceinline__ bool draw_element(uint64_t seed, int64_t e, const uint64_t* __restrict__ thr,
+__device__ __forceinline__ bool draw_element(uint64_t seed, int64_t n, int64_t e, const uint64_t* __restrict__ thr,
                                              int32_t (&c)[4], uint64_t (&key)[2]) {
+    if constexpr (KIND == CS_3D_DIAMOND || KIND == CS_4D_DIAMOND) {
+        constexpr int D = KIND == CS_3D_DIAMOND ? 3 : 4;
+        const uint32_t todo = __ballot_sync(0xffffffffu, e < n);
+        return draw_diamond<D>(todo, stream_key(seed, D == 3 ? kStreamDiamond3 : kStreamDiamond4), e, c, key[0]) || e >= n;
+    }
+    if (e >= n) return true;
     if constexpr (KIND == CS_2D_ORDER)
         draw_2d_order(stream_key(seed, kStreamOrderU), stream_key(seed, kStreamOrderV), e, key[0], key[1]);
     else if constexpr (KIND == CS_2D_DIAMOND)
@@ -88,10 +95,6 @@ __device__ __forceinline__ bool draw_element(uint64_t seed, int64_t e, const uin
         key[0] = draw_2d_cylinder(stream_key(seed, kStreamCylinder), e, c[0], c[1]);
     else if constexpr (KIND == CS_2D_DS_SLAB)
         key[0] = draw_ds_slab(stream_key(seed, kStreamDeSitter), e, thr, c[0], c[1]);
-    else if constexpr (KIND == CS_3D_DIAMOND)
-        return draw_3d_diamond(stream_key(seed, kStreamDiamond3), e, c, key[0]);
-    else
-        return draw_4d_diamond(stream_key(seed, kStreamDiamond4), e, c, key[0]);
     return true;
 }
 
@@ -102,10 +105,12 @@ constexpr int kind_dim(int kind) { return kind == CS_4D_DIAMOND ? 4 : kind == CS
 template <int KIND>
 __global__ void __launch_bounds__(kThreads) k_keys(int64_t n, uint64_t seed, const uint64_t* __restrict__ thr,
                                                    SprinkleScratch s, int bits, WsHeader* hdr) {
-    for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < n; e += int64_t(gridDim.x) * blockDim.x) {
+    const int64_t first = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+    for (int64_t e = first; e - (threadIdx.x & 31) < n; e += int64_t(gridDim.x) * blockDim.x) {  // whole warps
         int32_t c[4];
         uint64_t key[2];
-        if (!draw_element<KIND>(seed, e, thr, c, key)) set_status(hdr, CS_ERANGE);
+        if (!draw_element<KIND>(seed, n, e, thr, c, key)) set_status(hdr, CS_ERANGE);
+        if (e >= n) continue;
 #pragma unroll
         for (int q = 0; q < (KIND == CS_2D_ORDER ? 2 : 1); ++q) {
             s.key[q][e] = key[q];
@@ -213,9 +218,8 @@ __global__ void __launch_bounds__(kRankThreads) k_sprinkle_small(int n, int lgP,
 #pragma unroll
     for (int q = 0; q < kPer; ++q) {
         const int e = int(threadIdx.x) + q * kRankThreads;
-        if (e >= n) continue;
-        if (!draw_element<KIND>(seed, e, thr, c[q], key[q])) set_status(hdr, CS_ERANGE);
-        sk[e] = key[q][0];
+        if (!draw_element<KIND>(seed, n, e, thr, c[q], key[q])) set_status(hdr, CS_ERANGE);
+        if (e < n) sk[e] = key[q][0];
     }
     rank_keys_smem(n, lgP, sk, cnt, slot, rank);
     if constexpr (KIND == CS_2D_ORDER) {

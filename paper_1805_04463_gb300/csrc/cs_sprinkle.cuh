@@ -33,43 +33,78 @@ __device__ __forceinline__ uint64_t draw_2d_diamond(uint64_t s, int64_t e, int32
     return uint64_t(uu + vv) << 32;
 }
 
+// Lane of the k-th (from 0) set bit of m, k < popc(m).
+__device__ __forceinline__ int nth_lane(uint32_t m, int k) {
+    int at = 0;
+#pragma unroll
+    for (int w = 16; w > 0; w >>= 1) {
+        const int c = __popc((m >> at) & ((1u << w) - 1u));
+        if (k >= c) {
+            k -= c;
+            at += w;
+        }
+    }
+    return at;
+}
+
 // D-dimensional diamond of height 1 (D = 3: 2+1, D = 4: 3+1): rejection
 // sampling in the box t in [0, 2^20), spatial coordinates in [-2^19, 2^19),
 // accepting |x|^2 < min(t, 2^20-t)^2; attempt a uses slots D*a .. D*a+D-1.
 // Sort key t in the top 20 bits.  Returns false if no attempt was accepted.
+//
+// All 32 lanes of the warp call it; those of `todo` draw an element (seed s,
+// number e) each.  An attempt is accepted with probability pi/24 (3+1) or
+// pi/12, so lane by lane a warp went on until its unluckiest one, about 29
+// (13) rounds; here the lanes of accepted elements take later attempts of
+// the others, 2^lg side by side, and the first accepted one of an element is
+// its draw: about 11 (7) rounds, the same coordinates.
 template <int D>
-__device__ __forceinline__ bool draw_diamond(uint64_t s, int64_t e, int32_t (&c)[4], uint64_t& key) {
+__device__ __forceinline__ bool draw_diamond(uint32_t todo, uint64_t s, int64_t e, int32_t (&c)[4], uint64_t& key) {
+    constexpr uint32_t kAll = 0xffffffffu;
     const int64_t half = kGrid / 2;
-    for (int a = 0; a < kMaxAttempts; ++a) {
-        int64_t q[D];
-#pragma unroll
-        for (int k = 0; k < D; ++k) q[k] = int64_t(draw_from(s, uint64_t(e), uint32_t(D * a + k)) >> (64 - kGridBits));
+    const int lane = threadIdx.x & 31;
+    uint32_t left = todo;  // uniform
+    bool ok = false;
+    if ((todo >> lane) & 1u) {
+        c[0] = c[1] = c[2] = c[3] = 0;
+        key = 0;
+    }
+    for (int a = 0; left && a < kMaxAttempts;) {
+        const int u = __popc(left), lg = __clz(u - 1) - 27;  // the largest 2^lg <= 32 / u
+        const bool live = (lane >> lg) < u;
+        const int owner = live ? nth_lane(left, lane >> lg) : lane;
+        const uint64_t se = __shfl_sync(kAll, s, owner);
+        const int64_t ee = __shfl_sync(kAll, e, owner);
+        const int at = a + (lane & ((1 << lg) - 1));
+        int32_t q[D];
         int64_t r2 = 0;
 #pragma unroll
-        for (int k = 1; k < D; ++k) {
-            q[k] -= half;
-            r2 += q[k] * q[k];
-        }
-        const int64_t t = q[0];
-        const int64_t h = t < kGrid - t ? t : kGrid - t;
-        if (r2 < h * h) {
+        for (int k = 0; k < D; ++k)
+            q[k] = int32_t(int64_t(draw_from(se, uint64_t(ee), uint32_t(D * at + k)) >> (64 - kGridBits)));
 #pragma unroll
-            for (int k = 0; k < 4; ++k) c[k] = k < D ? int32_t(q[k < D ? k : 0]) : 0;
-            key = uint64_t(t) << (64 - kGridBits);
-            return true;
+        for (int k = 1; k < D; ++k) {
+            q[k] -= int32_t(half);
+            r2 += int64_t(q[k]) * q[k];
         }
+        const int64_t h = q[0] < kGrid - q[0] ? q[0] : kGrid - q[0];
+        const uint32_t accepted = __ballot_sync(kAll, live && at < kMaxAttempts && r2 < h * h);
+        // an element's attempts: lanes [r 2^lg, (r + 1) 2^lg) for its place r in left
+        const bool mine = (left >> lane) & 1u;
+        const int r = __popc(left & ((1u << lane) - 1u));
+        const uint32_t group = mine ? (kAll >> (32 - (1 << lg))) << (r << lg) : 0u;
+        const uint32_t hit = accepted & group;
+        const int src = hit ? __ffs(int(hit)) - 1 : lane;
+#pragma unroll
+        for (int k = 0; k < D; ++k) {
+            const int32_t v = __shfl_sync(kAll, q[k], src);
+            if (hit) c[k] = v;
+        }
+        if (hit) ok = true;
+        left = __ballot_sync(kAll, mine && !hit);
+        a += 1 << lg;
     }
-    c[0] = c[1] = c[2] = c[3] = 0;
-    key = 0;
-    return false;
-}
-
-__device__ __forceinline__ bool draw_4d_diamond(uint64_t s, int64_t e, int32_t (&c)[4], uint64_t& key) {
-    return draw_diamond<4>(s, e, c, key);
-}
-
-__device__ __forceinline__ bool draw_3d_diamond(uint64_t s, int64_t e, int32_t (&c)[4], uint64_t& key) {
-    return draw_diamond<3>(s, e, c, key);
+    if (ok) key = uint64_t(uint32_t(c[0])) << (64 - kGridBits);
+    return ok;
 }
 
 // 1+1 de Sitter slab (spherical foliation, Eq. ds_metric): theta uniform on
