@@ -23,11 +23,28 @@ namespace {
 // de Sitter slab n = 50021 632 / 253 us, 1+1 diamond n = 30011 79 / 79 us, 2D
 // order n = 131072 789 / 802 us.  What bounds it now is the integer pipe (the
 // circle 83%, the light cone 70%), in 3+1 the FMA pipe (53%) with it (44%).
-template <int G>
+template <int G, int kWords>
 __global__ void __launch_bounds__(kRelThreads) k_relate(const int32_t* __restrict__ coords, int64_t n,
                                                         uint64_t* __restrict__ bits, int64_t row_words) {
     __shared__ __align__(16) uint8_t sm[relate_stage_bytes(G)];
-    relate_block<G>(coords, n, bits, row_words, blockIdx.x, int64_t(blockIdx.y) * kRelWordsPerBlock, sm);
+    relate_block<G, kWords>(coords, n, bits, row_words, blockIdx.x,
+                            int64_t(blockIdx.y) * (kWords * (kRelThreads / 32)), sm);
+}
+
+// Chunks of 32 words; of 8, one per warp, where those would be fewer than two
+// per SM (n up to 6144): a chunk is then
+// latency, four words in turn.  With the mirror, 32 / 8 words, back to back: 1+1
+// diamond n = 2048 12.1 / 9.0 us, 3+1 n = 1024 10.2 / 7.4, n = 4099 12.9 / 10.7,
+// 2D order 2048 13.7 / 11.9, 4099 13.9 / 14.2 (its own words' exact tests are the
+// longest chain).
+template <int G>
+void launch_upper(const int32_t* coords, int64_t n, uint64_t* bits, int64_t row_words, cudaStream_t st) {
+    const unsigned rows = unsigned((n + kRelRowsPerBlock - 1) / kRelRowsPerBlock);
+    const int64_t chunks = (row_words + kRelWordsPerBlock - 1) / kRelWordsPerBlock;
+    if (int64_t(rows) * chunks < 2 * int64_t(device_sm_count()))
+        k_relate<G, 1><<<dim3(rows, unsigned((row_words + 7) / 8)), kRelThreads, 0, st>>>(coords, n, bits, row_words);
+    else
+        k_relate<G, kRelWarpWords><<<dim3(rows, unsigned(chunks)), kRelThreads, 0, st>>>(coords, n, bits, row_words);
 }
 
 __global__ void __launch_bounds__(kRelThreads, 4) k_mirror(uint64_t* __restrict__ bits, int64_t n, int64_t row_words) {
@@ -39,18 +56,16 @@ __global__ void __launch_bounds__(kRelThreads, 4) k_mirror(uint64_t* __restrict_
 
 cudaError_t launch_relate(int kind, int64_t n, const int32_t* coords, uint64_t* bits, int64_t row_words,
                           cudaStream_t st) {
-    dim3 grid(unsigned((n + kRelRowsPerBlock - 1) / kRelRowsPerBlock),
-              unsigned((row_words + kRelWordsPerBlock - 1) / kRelWordsPerBlock));
     if (kind == CS_4D_DIAMOND)
-        k_relate<kGeom4><<<grid, kRelThreads, 0, st>>>(coords, n, bits, row_words);
+        launch_upper<kGeom4>(coords, n, bits, row_words, st);
     else if (kind == CS_3D_DIAMOND)
-        k_relate<kGeom3><<<grid, kRelThreads, 0, st>>>(coords, n, bits, row_words);
+        launch_upper<kGeom3>(coords, n, bits, row_words, st);
     else if (kind == CS_2D_DS_SLAB || kind == CS_2D_CYLINDER)
-        k_relate<kGeomDeSitter><<<grid, kRelThreads, 0, st>>>(coords, n, bits, row_words);
+        launch_upper<kGeomDeSitter>(coords, n, bits, row_words, st);
     else if (kind == CS_2D_ORDER)
-        k_relate<kGeomOrder><<<grid, kRelThreads, 0, st>>>(coords, n, bits, row_words);
+        launch_upper<kGeomOrder>(coords, n, bits, row_words, st);
     else
-        k_relate<kGeomLightCone><<<grid, kRelThreads, 0, st>>>(coords, n, bits, row_words);
+        launch_upper<kGeomLightCone>(coords, n, bits, row_words, st);
     const int64_t st8 = ((n + 63) / 64 + kMirTiles - 1) / kMirTiles;  // super-tiles per side
     if (st8 > 0) k_mirror<<<dim3(unsigned(st8), unsigned(st8)), kRelThreads, 0, st>>>(bits, n, row_words);
     return cudaGetLastError();

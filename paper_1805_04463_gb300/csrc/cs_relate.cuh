@@ -279,13 +279,16 @@ __device__ __forceinline__ void relate_word(const uint8_t* __restrict__ smem, in
 //     with a value near the cone is found exactly.
 // The integer tests' own word of the row tile (it holds the diagonal and both
 // cones) is found exactly; the filter is symmetric and takes it too.
-template <int G>
+// kWords: words per warp (4), or 1 for a set whose chunks leave SMs idle; the
+// block then covers 8 words (w0 a multiple of 8).
+template <int G, int kWords = kRelWarpWords>
 __device__ __forceinline__ void relate_block(const int32_t* __restrict__ coords, int64_t n,
                                              uint64_t* __restrict__ bits, int64_t row_words, int64_t rb, int64_t w0,
                                              uint8_t* smem, int64_t zero_from = -1) {
     constexpr int D = geom_dim(G);
     constexpr bool kFilter = G == kGeom3 || G == kGeom4;
-    if (w0 + kRelWordsPerBlock <= rb) return;  // wholly below the diagonal
+    constexpr int kBlockWords = kWords * (kRelThreads / 32);
+    if (w0 + kBlockWords <= rb) return;  // wholly below the diagonal
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t V = (n + 63) >> 6;  // valid words
     const int64_t c0 = w0 * 64, r0 = rb * kRelRowsPerBlock;
@@ -300,7 +303,7 @@ __device__ __forceinline__ void relate_block(const int32_t* __restrict__ coords,
         ulonglong2* q0 = reinterpret_cast<ulonglong2*>(smem);      // (t, t), (x, x)
         ulonglong2* q1 = q0 + kRelColsPerBlock / 2;                // (y, y), (z, z); 2+1: (y, y), (A, A)
         uint64_t* q2 = reinterpret_cast<uint64_t*>(q1 + kRelColsPerBlock / 2);  // 3+1: (A, A)
-        for (int p = first + threadIdx.x; p < kRelColsPerBlock / 2; p += kRelThreads) {
+        for (int p = first + threadIdx.x; p < 32 * kBlockWords; p += kRelThreads) {
             int32_t c[2][D];
 #pragma unroll
             for (int k = 0; k < 2; ++k)
@@ -329,7 +332,7 @@ __device__ __forceinline__ void relate_block(const int32_t* __restrict__ coords,
         }
         fast = !__syncthreads_or(out);
     } else {
-        for (int p = first + threadIdx.x; p < kRelColsPerBlock / 2; p += kRelThreads) {
+        for (int p = first + threadIdx.x; p < 32 * kBlockWords; p += kRelThreads) {
             int32_t c[2][2];
 #pragma unroll
             for (int k = 0; k < 2; ++k)
@@ -373,21 +376,21 @@ __device__ __forceinline__ void relate_block(const int32_t* __restrict__ coords,
             row[r].nv = ~c[1];
         }
     }
-    const int64_t wb = w0 + kRelWarpWords * warp;  // this warp's first word
-    if (wb + kRelWarpWords > rb && wb < row_words) {  // warp-uniform: some word at or after the row tile
+    const int64_t wb = w0 + kWords * warp;  // this warp's first word
+    if (wb + kWords > rb && wb < row_words) {  // warp-uniform: some word at or after the row tile
         // [word][row]; the words shift down as they are found, so that the loop
         // is one copy of the tests (unrolled, the instruction cache missed)
-        uint64_t word[kRelWarpWords][2] = {};
+        uint64_t word[kWords][2] = {};
 #pragma unroll 1
-        for (int k = 0; k < kRelWarpWords; ++k) {
+        for (int k = 0; k < kWords; ++k) {
             const int64_t W = wb + k;
 #pragma unroll
             for (int r = 0; r < 2; ++r) {
 #pragma unroll
-                for (int x = 0; x + 1 < kRelWarpWords; ++x) word[x][r] = word[x + 1][r];
-                word[kRelWarpWords - 1][r] = 0ull;
+                for (int x = 0; x + 1 < kWords; ++x) word[x][r] = word[x + 1][r];
+                word[kWords - 1][r] = 0ull;
             }
-            uint64_t (&found)[2] = word[kRelWarpWords - 1];
+            uint64_t (&found)[2] = word[kWords - 1];
             if (W < rb || W >= V) continue;  // warp-uniform
             // rows to find exactly: the own word of the integer tests, coordinates beyond the
             // filter's range, and below the rows whose tests could not decide
@@ -436,19 +439,19 @@ __device__ __forceinline__ void relate_block(const int32_t* __restrict__ coords,
             }
         }
         // a row's four words as one 32-byte store; words before the row tile are mirror_block's
-        const bool whole = wb >= rb && (reinterpret_cast<uintptr_t>(bits) & 31) == 0;  // warp-uniform
+        const bool whole = kWords == kRelWarpWords && wb >= rb && (reinterpret_cast<uintptr_t>(bits) & 31) == 0;  // warp-uniform
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
             const int64_t i = r0 + lane + 32 * r;
             if (i >= n) continue;
             uint64_t* dst = bits + i * row_words + wb;
             if (whole) {
-                asm volatile("st.global.v4.b64 [%0], {%1, %2, %3, %4};" ::"l"(dst), "l"(word[0][r]), "l"(word[1][r]),
-                             "l"(word[2][r]), "l"(word[3][r])
+                asm volatile("st.global.v4.b64 [%0], {%1, %2, %3, %4};" ::"l"(dst), "l"(word[0][r]),
+                             "l"(word[1 % kWords][r]), "l"(word[2 % kWords][r]), "l"(word[3 % kWords][r])
                              : "memory");
             } else {
 #pragma unroll
-                for (int k = 0; k < kRelWarpWords; ++k)
+                for (int k = 0; k < kWords; ++k)
                     if (wb + k >= rb) dst[k] = word[k][r];
             }
         }
