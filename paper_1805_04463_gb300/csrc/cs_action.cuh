@@ -136,18 +136,16 @@ __host__ __device__ inline int64_t bracket_of(int dim, int64_t n, const int64_t*
 }
 
 // The 2+1 constant (pi/(3 sqrt 2))^(2/3) / Gamma(5/3) of Eqs. s3d_local and
-// b3d_local, from the math library in double (a constant factor; its
-// rounding is ~1e-16 relative).
-__host__ __device__ inline double c3_const() {
-    const double v = cbrt(3.14159265358979323846 / (3.0 * sqrt(2.0)));
-    return v * v / tgamma(5.0 / 3.0);
-}
+// b3d_local, 0.90665872967043620699..., in double (a constant factor, 7e-17
+// from the exact one; the C libraries' cube root and gamma function gave
+// values up to two units in the last place off, and not the same ones).
+inline double c3_const() { return 0.9066587296704361; }
 
 __host__ __device__ inline bool is_local(double eps) { return eps <= 0.0 || eps == 1.0; }
 
 // Factors of the actions that depend on eps (and the dimension) alone, found
-// on the host: on the device the 2+1 and 3+1 ones are a cube root, a gamma
-// function and two double-double divisions, FP64 work in one thread.
+// on the host: on the device the 2+1 and 3+1 ones are a cube root and two
+// double-double divisions, FP64 work in one thread.
 //   local:   2 * bracket (1+1), c3 * bracket / 8 (2+1), 4/sqrt(6) * bracket (3+1)
 //   smeared, from sum = sum_k N_k f(k, eps):
 //     1+1: 2 eps [N - 2 eps sum];  2+1: c3 eps^(2/3) [N - eps sum];
@@ -160,10 +158,7 @@ inline dd local_factor(int dim) {
 
 inline dd smeared_factor(int dim, double eps) {
     if (dim == 2) return dd_mul_d(dd_from(eps), 2.0);
-    if (dim == 3) {
-        const double r = cbrt(eps);
-        return dd_from(c3_const() * (r * r));
-    }
+    if (dim == 3) return dd_two_prod(c3_const(), pow(eps, 2.0 / 3.0));  // the power within a unit in the last place
     return dd_mul_d(dd_sqrt(dd_div(dd_from(eps), dd_from(6.0))), 4.0);
 }
 
