@@ -9,8 +9,10 @@ Prints one JSON line (rank 0).  value = related pairs counted per second
 (Gpairs/s) over the whole job; e2e = the same metric through the host-buffer
 entry point cs_evaluate (coordinates copied from pinned host memory, the
 histogram and actions copied back, every step); roofline = the count
-kernel's achieved rate against the POPC (or tensor) peak; cpu_baseline = the
-CPU oracle on a bounded sample of the same workload.
+kernel's achieved rate against its peak (--path auto counts a product order
+from its coordinates, bound by shared-memory adds; roofline_tensor is then
+the contraction of the same matrix, timed apart); cpu_baseline = the CPU
+oracle on a bounded sample of the same workload.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--workload NAME] [--path auto|popc|mma|mma4]
   python bench.py --impl reference ...   # the CPU oracle as the reference arm
@@ -40,8 +42,10 @@ WORKLOADS = {
 }
 EPS = (0.0, 0.05, 0.1, 0.2)
 PATHS = {"auto": 0, "popc": 1, "mma": 2, "mma4": 3}
-PATH_NAMES = {1: "popc", 2: "mma", 3: "mma4"}
+COORDS = 4  # counted from the coordinates (cs_coords_abundance), AUTO's choice for product orders
+PATH_NAMES = {1: "popc", 2: "mma", 3: "mma4", COORDS: "coords"}
 POPC_PER_SM_PER_CLK = 16  # 32-bit population count, per SM per clock
+ADD_CLK_PER_WARP = 2.3    # full-warp shared-memory add, conflict-free, measured clocks per SM
 
 
 def _peaks():
@@ -61,7 +65,10 @@ def _dist():
 
 
 class ClockSampler:
-    """nvidia-smi clock/throttle samples during the timed region."""
+    """nvidia-smi clock/throttle samples during the timed region: the sampler is up
+    (its first line written) before the region begins, and samples often enough
+    for a region of tens of milliseconds; lines written before it count only if
+    none was written in it."""
 
     Q = ("index,clocks.sm,clocks.max.sm,power.draw,clocks_event_reasons.active,"
          "clocks_event_reasons.hw_slowdown,clocks_event_reasons.hw_thermal_slowdown,"
@@ -71,6 +78,7 @@ class ClockSampler:
         self.gpu = gpu_index
         self.proc = None
         self.path = None
+        self.before = 0  # bytes written before the region
 
     def __enter__(self):
         fd, self.path = tempfile.mkstemp(prefix="clocks_", suffix=".csv")
@@ -78,9 +86,14 @@ class ClockSampler:
         try:
             self.proc = subprocess.Popen(
                 ["nvidia-smi", "-i", str(self.gpu), "--query-gpu=" + self.Q, "--format=csv,noheader,nounits",
-                 "-lms", "200"], stdout=open(self.path, "w"), stderr=subprocess.DEVNULL)
+                 "-lms", "10"], stdout=open(self.path, "w"), stderr=subprocess.DEVNULL)
         except OSError:
             self.proc = None
+            return self
+        limit = time.perf_counter() + 3.0
+        while not os.path.getsize(self.path) and self.proc.poll() is None and time.perf_counter() < limit:
+            time.sleep(0.01)
+        self.before = os.path.getsize(self.path)
         return self
 
     def __exit__(self, *a):
@@ -95,7 +108,9 @@ class ClockSampler:
         sm, mx, reasons = [], [], set()
         names = ["hw_slowdown", "hw_thermal_slowdown", "sw_thermal_slowdown", "sw_power_cap"]
         try:
-            for line in open(self.path):
+            text = open(self.path).read()
+            inside = text[self.before:]
+            for line in (inside if inside.count(",") >= 8 else text).splitlines():
                 f = [x.strip() for x in line.split(",")]
                 if len(f) < 9:
                     continue
@@ -130,6 +145,15 @@ def roofline_for(resolved, n, count_s, peaks, src, sm_count):
     cap (the clocks record of the run shows it), not a seconds-long loop.  The
     fraction of the sustained-derived peak is reported beside it."""
     terms = n * (n - 1) * (n - 2) / 6.0
+    if resolved == COORDS:
+        adds = n * (n - 1) / 2.0  # one histogram add per pair i < j (unrelated ones to a spare bin)
+        peak = sm_count * 32 / ADD_CLK_PER_WARP * peaks.get("sm_max_mhz", 2070.0) * 1e6 / 1e12
+        achieved = adds / count_s / 1e12
+        return {"bound": "smem", "kernel": "k_count_order (+ ranks and table)", "achieved": achieved, "peak": peak,
+                "unit": "T adds/s", "frac": achieved / peak, "traffic": None, "algorithmic_adds": adds,
+                "contraction_macs": terms,
+                "peak_source": f"{sm_count} SMs x 32 lanes / {ADD_CLK_PER_WARP} clk (measured conflict-free add) x "
+                               f"{peaks.get('sm_max_mhz')} MHz (sm_max_mhz, {src})"}
     if resolved in (2, 3):
         ratio, kind, kern = ((6.0, "FP4 kind::mxf4", "k_count_mma4 (+ k_expand_f4)") if resolved == 3 else
                              (2.0, "FP8 kind::f8f6f4", "k_count_mma (+ k_expand_f8)"))
@@ -151,19 +175,21 @@ def roofline_for(resolved, n, count_s, peaks, src, sm_count):
                            f"(sm_max_mhz, {src})"}
 
 
-TRAFFIC_RECORDS = {2: "k_count_mma__2d_order_131072__dram.md", 3: "k_count_mma4__2d_order_131072__dram.md"}
-MMA_SOURCES = [os.path.join(ROOT, "paper_1805_04463_gb300", "csrc", f)
-               for f in ("cs_count_mma.cu", "cs_internal.cuh", "cs_kernels.cuh")]
+TRAFFIC_RECORDS = {2: "k_count_mma__2d_order_131072__dram.md", 3: "k_count_mma4__2d_order_131072__dram.md",
+                   COORDS: "k_count_order__2d_order_131072.md"}
+MMA_SOURCES = ("cs_count_mma.cu", "cs_internal.cuh", "cs_kernels.cuh")
+TRAFFIC_SOURCES = {2: MMA_SOURCES, 3: MMA_SOURCES, COORDS: ("cs_order.cu", "cs_order.cuh", "cs_internal.cuh")}
 
 
 def recorded_traffic(resolved):
-    """DRAM bytes per full-size count launch (k_count_mma or k_count_mma4) from the
+    """DRAM bytes per full-size count launch (of the path's count kernel) from the
     committed ncu record, or None when the kernel sources changed since it was captured."""
     import hashlib
     try:
         path = os.path.join(ROOT, "profiles", TRAFFIC_RECORDS[resolved])
         rec = dict(line.split(":", 1) for line in open(path) if line.startswith(("traffic_", "kernel_")))
-        h = hashlib.sha256(b"".join(open(f, "rb").read() for f in MMA_SOURCES)).hexdigest()[:16]
+        files = (os.path.join(ROOT, "paper_1805_04463_gb300", "csrc", f) for f in TRAFFIC_SOURCES[resolved])
+        h = hashlib.sha256(b"".join(open(f, "rb").read() for f in files)).hexdigest()[:16]
     except (OSError, ValueError, KeyError):
         return None
     if rec.get("kernel_sources_sha256_16", "").strip() != h:
@@ -216,7 +242,7 @@ def ensemble_bench(cs, torch, path, steps=5, warmup=3, n2d=512, n4d=256):
         raise cs.CsError(b.status(), "ensemble")
     pairs = int(b.hist.sum().item())
     # one-at-a-time: the same sets through the single-set entry points
-    bufs = [cs.allocate(k, n, path=b.path) for k, n, _ in sets]
+    bufs = [cs.allocate(k, n, path=path) for k, n, _ in sets]
     def plain():
         for (k, n, sd), buf in zip(sets, bufs):
             cs.run(buf, sd, eps=EPS, stream=stream)
@@ -341,12 +367,13 @@ def batch_path(name):
     return PATHS[name]
 
 
-def launches_per_step(kind, path):
-    """Kernels of this library launched by one step: sprinkle (keys, 4 bucket-rank
-    kernels per key stream, scatter), relate (upper part, mirror), count
-    (operand expansion first on the tensor paths) and actions (partial, final)."""
-    sprinkle = 1 + (2 if kind == 0 else 1) * 4 + 1
-    count = 1 if path == 1 else 2
+def launches_per_step(n, path):
+    """Kernels of this library launched by one step: sprinkle (one small kernel, or keys,
+    bucket scan, fill, rank and scatter), relate (upper part, mirror), count (operand
+    expansion first on the tensor paths; from coordinates the ranks -- one kernel, or
+    sort, rank and scatter -- then table and count) and actions (partial, final)."""
+    sprinkle = 1 if n <= 2048 else 4
+    count = (3 if n <= 8192 else 5) if path == COORDS else 1 if path == 1 else 2
     return sprinkle + 2 + count + 2
 
 
@@ -473,6 +500,13 @@ def main():
     path = PATHS[args.path]
     buf = cs.allocate(kind, n, path=path)
     stream = torch.cuda.current_stream()
+    resolved = COORDS if buf.by_coords else cs.resolved_path(n, path)
+
+    def count():
+        if buf.by_coords:
+            cs.coords_abundance(kind, n, buf.coords, buf.hist, buf.workspace, stream)
+        else:
+            cs.interval_abundance(n, buf.bits, buf.hist, path, buf.workspace, stream)
 
     # count-kernel timing: events on the launching stream around each count call
     ev = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for _ in range(args.steps)]
@@ -482,7 +516,7 @@ def main():
         cs.causal_matrix(kind, n, buf.coords, buf.bits, stream)
         if i is not None:
             ev[i][0].record(stream)
-        cs.interval_abundance(n, buf.bits, buf.hist, path, buf.workspace, stream)
+        count()
         if i is not None:
             ev[i][1].record(stream)
         cs.action_device(cs.dim(kind), n, buf.hist, list(EPS), buf.actions, buf.bracket, buf.workspace, stream)
@@ -516,7 +550,7 @@ def main():
     se[1].record(stream)
     cs.causal_matrix(kind, n, buf.coords, buf.bits, stream)
     se[2].record(stream)
-    cs.interval_abundance(n, buf.bits, buf.hist, path, buf.workspace, stream)
+    count()
     se[3].record(stream)
     cs.action_device(cs.dim(kind), n, buf.hist, list(EPS), buf.actions, buf.bracket, buf.workspace, stream)
     se[4].record(stream)
@@ -555,24 +589,43 @@ def main():
 
     peaks, src = _peaks()
     clocks = clk.summary()
-    roofline = roofline_for(cs.resolved_path(n, path), n, statistics.mean(count_ms) / 1e3, peaks, src,
-                            torch.cuda.get_device_properties(local).multi_processor_count)
-    roofline["count_ms"] = statistics.mean(count_ms)
-    resolved = cs.resolved_path(n, path)
-    if roofline["bound"] == "tensor" and args.workload == "2d_order_131072":
-        tr = recorded_traffic(resolved)
-        roofline["traffic"] = tr
-        roofline["traffic_source"] = (f"profiles/{TRAFFIC_RECORDS[resolved]} (dram__bytes_read.sum + "
-                                      "dram__bytes_write.sum, one full-size launch)" if tr else
-                                      "no capture for the current kernel sources")
+    sms = torch.cuda.get_device_properties(local).multi_processor_count
+    matrix_path = cs.resolved_path(n, path)  # of the contraction
+
+    def roofline_of(which, ms):
+        r = roofline_for(which, n, ms / 1e3, peaks, src, sms)
+        r["count_ms"] = ms
+        if which in TRAFFIC_RECORDS and args.workload == "2d_order_131072":
+            tr = recorded_traffic(which)
+            r["traffic"] = tr
+            r["traffic_source"] = (f"profiles/{TRAFFIC_RECORDS[which]} (dram__bytes_read.sum + "
+                                   "dram__bytes_write.sum, one full-size launch)" if tr else
+                                   "no capture for the current kernel sources")
+        if which == COORDS:
+            return r
+        # context beside the contract's peak: the path's innermost operation timed
+        # alone on every SM (cs_peak_probe), and the count's fraction of it
+        probe = cs.peak_probe(which, PROBE_REPS[which]) / 1e12
+        r["probe"] = {"value": probe, "unit": r["unit"], "frac": r["achieved"] / probe, "what": PROBE_WHAT[which]}
+        r["frac_probe"] = r["achieved"] / probe
+        return r
+
+    roofline = roofline_of(resolved, statistics.mean(count_ms))
+    roofline_tensor = None
+    if buf.by_coords:
+        # the contraction of the same matrix, outside the timed region
+        check, tev = torch.empty_like(buf.hist), [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+        for e in tev:
+            e.record(stream)  # the second pass is timed
+            cs.interval_abundance(n, buf.bits, check, matrix_path, buf.workspace, stream)
+        tend = torch.cuda.Event(enable_timing=True)
+        tend.record(stream)
+        torch.cuda.synchronize()
+        if not torch.equal(check, buf.hist):
+            raise RuntimeError("the contraction disagrees with the count from coordinates")
+        roofline_tensor = roofline_of(matrix_path, tev[1].elapsed_time(tend))
     if args.compare_paths:
         roofline["paths_ms"] = compare_paths(cs, torch, buf, n, stream)
-    # context beside the contract's peak: the path's innermost operation timed
-    # alone on every SM (cs_peak_probe), and the count's fraction of it
-    probe = cs.peak_probe(resolved, PROBE_REPS[resolved]) / 1e12
-    roofline["probe"] = {"value": probe, "unit": roofline["unit"], "frac": roofline["achieved"] / probe,
-                         "what": PROBE_WHAT[resolved]}
-    roofline["frac_probe"] = roofline["achieved"] / probe
     # the clock the count ran at: the time in SM cycles makes runs at
     # different clocks comparable
     roofline["sm_mhz_median"] = clocks.get("sm_mhz")
@@ -583,10 +636,11 @@ def main():
         "steps": args.steps, "warmup": args.warmup, "ms_per_step": elapsed_ms / args.steps,
         "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
         # the count's arithmetic: 0/1 E4M3 (FP8 path) or E2M1 (FP4 path) products summed
-        # in FP32 on the tensor paths, AND + popcount on 64-bit words on the POPC path
-        "dtype": {1: "u64", 2: "fp8e4m3", 3: "fp4e2m1"}[cs.resolved_path(n, path)], "data": "synthetic",
+        # in FP32 on the tensor paths, AND + popcount on 64-bit words on the POPC path, 32-bit
+        # integer ranks and prefix counts from the coordinates
+        "dtype": {1: "u64", 2: "fp8e4m3", 3: "fp4e2m1", COORDS: "int32"}[resolved], "data": "synthetic",
         "config": {"workload": args.workload, "kind": cs.KIND_NAMES[kind], "n": n, "seed": seed0,
-                   "path": args.path, "resolved_path": PATH_NAMES[cs.resolved_path(n, path)],
+                   "path": args.path, "resolved_path": PATH_NAMES[resolved],
                    "eps": list(EPS),
                    "l2": "inputs larger than L2" if cs.bitset_bytes(n) > 129e6 else "inputs smaller than L2",
                    "parallelism": f"replicas{args.gpus}"},
@@ -594,8 +648,8 @@ def main():
         "pairs_per_step": pairs, "actions": actions,
         "e2e": {"value": e2e_value, "unit": "Gpairs/s", "h2d_bytes_per_step": int(cp.nbytes),
                 "d2h_bytes_per_step": int(hist_pinned.nbytes + 8 * len(EPS) + 8), "steps": e2e_steps},
-        "gpu_launches": launches_per_step(kind, cs.resolved_path(n, path)) * args.steps,
-        "roofline": roofline,
+        "gpu_launches": launches_per_step(n, resolved) * args.steps,
+        "roofline": roofline, "roofline_tensor": roofline_tensor,
         "clocks": clocks,
         "stages_ms": stages_ms,
         "tuning": tuning if tuning is not None else {"paths": cs.get_auto_paths(), "tiles": cs.get_auto_tiles(),
