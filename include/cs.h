@@ -277,7 +277,7 @@ int cs_interval_abundance(int64_t n, const uint64_t *bits_dev, int64_t row_words
  * The same abundances from the coordinates of a set whose relation is the
  * product order of two of them (CS_2D_ORDER, CS_2D_DIAMOND, CS_2D_SQUARE): with
  * elements numbered by u, |A_ab| is a difference of four counts
- * #{c < x : v_c < y}, looked up in a table of n^2 / 128 bytes, O(n^2) for the
+ * #{c < x : v_c < y}, looked up in a table of n^2 / 256 bytes, O(n^2) for the
  * whole set.  coords_dev as for cs_causal_matrix (any order of labels for the
  * diamond and the square).  hist_dev is zeroed and then filled by the
  * callee, with the same values as cs_interval_abundance on the set's causal
@@ -375,7 +375,8 @@ int cs_action_device(int dim, int64_t n, const int64_t *hist_dev, int64_t len,
 /*
  * One whole evaluation from host buffers, for callers that keep their data
  * on the host: copies coords_host (cs_coords_bytes) to the device, builds the
- * causal matrix, counts intervals on `path`, evaluates the actions for n_eps
+ * causal matrix, counts intervals on `path` (CS_PATH_AUTO counts a product
+ * order from its coordinates instead, see cs_coords_abundance), evaluates the actions for n_eps
  * values of eps, and copies hist_host (cs_hist_len(n) int64), actions_host
  * (n_eps doubles) and *bracket_host back.  If coords_host is NULL the set is
  * sprinkled on the device from (kind, n, seed) instead.  Device memory comes
@@ -436,7 +437,9 @@ int cs_batch_create(const cs_set_desc *sets, int n_sets, int path, void *workspa
 /*
  * Evaluate every set of the plan: sprinkle, causal matrix, interval
  * abundances and actions, for all sets at once (one persistent count kernel
- * over the tiles of all sets, largest sets first).  Enqueues memsets and
+ * over the tiles of all sets, largest sets first; a plan made with
+ * CS_PATH_AUTO counts its product orders from their coordinates, without a
+ * causal matrix, see cs_coords_abundance).  Enqueues memsets and
  * kernels only, so the call can be captured into a CUDA graph and replayed.
  * hist_dev: cs_batch_hist_len int64 (zeroed by the callee); actions_dev:
  * n_sets x n_eps doubles, set-major (may be NULL when n_eps = 0);
@@ -462,7 +465,8 @@ int cs_batch_launch(const cs_batch *b, const double *eps_host, int n_eps, int64_
  */
 int cs_batch_poll(const cs_batch *b);
 
-/* The count path a plan runs (CS_PATH_POPC, CS_PATH_MMA or CS_PATH_MMA4;
+/* The count path a plan runs for the sets it counts from a causal matrix
+ * (CS_PATH_POPC, CS_PATH_MMA or CS_PATH_MMA4;
  * CS_PATH_AUTO plans the batch path of cs_set_batch_tuning, by default
  * CS_PATH_MMA4 where the device has tcgen05), -1 for NULL. */
 int cs_batch_path(const cs_batch *b);

@@ -32,3 +32,29 @@ def test_smeared_actions(oracle, dim, n):
         want, bracket = oracle.action(dim, n, h.astype(np.int64), ep)
         assert int(br[0]) == bracket
         assert abs(got[e] - want) <= 1e-12 * max(1.0, abs(want)), (ep, got[e], want)
+
+
+def test_captured_action(oracle):
+    """The dependent launch inside a CUDA graph, between other kernels, replayed back to back."""
+    import torch
+    from paper_1805_04463_gb300 import build
+    build.build()
+    import paper_1805_04463_gb300 as cs
+    buf = cs.allocate(0, 700)
+    g, st = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    with torch.cuda.stream(st):
+        cs.run(buf, 5, eps=EPS, stream=st)
+        st.synchronize()
+        with torch.cuda.graph(g, stream=st):
+            cs.run(buf, 4, eps=EPS, stream=st)
+            cs.run(buf, 5, eps=EPS, stream=st)
+    buf.actions.zero_()
+    for _ in range(5):
+        g.replay()
+    torch.cuda.synchronize()
+    h = oracle.interval_abundance(oracle.causal_matrix(0, oracle.sprinkle(0, 700, 5)))
+    assert (buf.hist.cpu().numpy() == h).all()
+    for e, ep in enumerate(EPS):
+        want, bracket = oracle.action(2, 700, h, ep)
+        assert int(buf.bracket[0]) == bracket
+        assert abs(float(buf.actions[e]) - want) <= 1e-12 * max(1.0, abs(want)), ep
