@@ -12,15 +12,11 @@
 
 #include "cs_action.cuh"
 #include "cs_kernels.cuh"
+#include "cs_launch.cuh"
 
 namespace cs {
 
 namespace {
-
-// Programmatic dependent launch: let the next kernel of the stream launch;
-// wait for the whole end of the kernel before (at once without one).
-__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void wait_for_primary() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Blocks of the smeared sum of cutoff kend with T threads each: one term per
 // thread until kActBlocks blocks are full.
@@ -186,17 +182,8 @@ cudaError_t launch_action_device(int dim, int64_t n, const int64_t* hist, int64_
         k_action_final<<<1, 32 * n_eps, 0, st>>>(dim, n, hist, len, a, T, partial, out, bracket);
         return cudaGetLastError();
     }
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(1);
-    cfg.blockDim = dim3(unsigned(32 * n_eps));
-    cfg.stream = st;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    const dd* sums = partial;
-    return cudaLaunchKernelEx(&cfg, k_action_final, dim, n, hist, len, a, T, sums, out, bracket);
+    return launch_after(k_action_final, dim3(1), unsigned(32 * n_eps), 0, st, dim, n, hist, len, a, T, partial, out,
+                        bracket);
 }
 
 }  // namespace cs

@@ -10,6 +10,7 @@
 #include <atomic>
 
 #include "cs_kernels.cuh"
+#include "cs_launch.cuh"
 #include "cs_order.cuh"
 
 namespace cs {
@@ -130,6 +131,7 @@ __device__ __forceinline__ void order_ranks_small(const int32_t* __restrict__ co
     uint32_t* cnt = reinterpret_cast<uint32_t*>(sk + P);
     uint32_t* slot = cnt + P;
     uint32_t* rank = slot + P;
+    launch_dependents();
     for (int k = blockIdx.x * kRankThreads + threadIdx.x; k < len; k += ctas * kRankThreads) hist[k] = 0ull;
     const bool v = kByU || blockIdx.x == 1;
     order_keys_smem(v ? coords + n : coords, v ? coords : coords + n, n, sk);
@@ -164,7 +166,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kRankThreads)
     order_ranks_small<false>(coords, n, lgP, rank_u, rank_v, p, q, hist, len);
 }
 
-__global__ void __launch_bounds__(kOrdBuildThreads) k_order_table(OrderSet s) { order_build_rows(s, blockIdx.x); }
+__global__ void __launch_bounds__(kOrdBuildThreads) k_order_table(OrderSet s) {
+    launch_dependents();
+    wait_for_primary();
+    order_build_rows(s, blockIdx.x);
+}
 
 constexpr int kCountWarps = 32;
 constexpr int kCountThreads = 32 * kCountWarps;
@@ -181,6 +187,7 @@ __global__ void __launch_bounds__(kCountThreads, 1) k_count_order(OrderSet s, in
     int2* stage = reinterpret_cast<int2*>(smem_ord) + 32 * (threadIdx.x >> 5);
     uint32_t* shist = reinterpret_cast<uint32_t*>(smem_ord + kCountStage);
     for (int k = threadIdx.x; k < bins; k += kCountThreads) shist[k] = 0u;
+    wait_for_primary();
     __syncthreads();
     const uint32_t hist_s = smem_u32(shist);
     const int64_t warps = int64_t(gridDim.x) * kCountWarps;
@@ -298,7 +305,10 @@ cudaError_t launch_count_order(int kind, int64_t n, const int32_t* coords, int64
         k_order_scatter<<<unsigned(blocks < 2432 ? blocks : 2432), 256, 0, st>>>(n, by_u ? nullptr : rank,
                                                                               by_u ? rank : rank + n, p, q);
     }
-    k_order_table<<<unsigned(order_build_blocks(n)), kOrdBuildThreads, 0, st>>>(s);
+    if ((err = cudaGetLastError()) != cudaSuccess ||
+        (err = launch_after(k_order_table, dim3(unsigned(order_build_blocks(n))), kOrdBuildThreads, 0, st, s)) !=
+            cudaSuccess)
+        return err;
 
     // Column chunks of 64 m: long enough to amortise a task's start (two
     // dependent gathers), short enough that the warps get several tasks each.
@@ -313,8 +323,7 @@ cudaError_t launch_count_order(int kind, int64_t n, const int32_t* coords, int64
     int64_t grid = (tasks + 7) / 8;
     if (grid > sms) grid = sms;
     unsigned long long* h = reinterpret_cast<unsigned long long*>(hist);
-    k_count_order<<<unsigned(grid), kCountThreads, smem, st>>>(s, tasks, m, bins, h);
-    return cudaGetLastError();
+    return launch_after(k_count_order, dim3(unsigned(grid)), kCountThreads, size_t(smem), st, s, tasks, m, bins, h);
 }
 
 }  // namespace cs

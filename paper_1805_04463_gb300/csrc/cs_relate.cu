@@ -12,6 +12,7 @@
 // transposes of the tiles above (the relation is symmetric), which halves
 // the tests.
 #include "cs_kernels.cuh"
+#include "cs_launch.cuh"
 #include "cs_relate.cuh"
 
 namespace cs {
@@ -27,6 +28,7 @@ template <int G, int kWords>
 __global__ void __launch_bounds__(kRelThreads) k_relate(const int32_t* __restrict__ coords, int64_t n,
                                                         uint64_t* __restrict__ bits, int64_t row_words) {
     __shared__ __align__(16) uint8_t sm[relate_stage_bytes(G)];
+    launch_dependents();
     relate_block<G, kWords>(coords, n, bits, row_words, blockIdx.x,
                             int64_t(blockIdx.y) * (kWords * (kRelThreads / 32)), sm);
 }
@@ -49,6 +51,7 @@ void launch_upper(const int32_t* coords, int64_t n, uint64_t* bits, int64_t row_
 
 __global__ void __launch_bounds__(kRelThreads, 4) k_mirror(uint64_t* __restrict__ bits, int64_t n, int64_t row_words) {
     __shared__ uint64_t sm[kMirRows][kMirTiles + 1];
+    wait_for_primary();
     mirror_block(bits, n, row_words, blockIdx.x, blockIdx.y, sm);
 }
 
@@ -67,8 +70,9 @@ cudaError_t launch_relate(int kind, int64_t n, const int32_t* coords, uint64_t* 
     else
         launch_upper<kGeomLightCone>(coords, n, bits, row_words, st);
     const int64_t st8 = ((n + 63) / 64 + kMirTiles - 1) / kMirTiles;  // super-tiles per side
-    if (st8 > 0) k_mirror<<<dim3(unsigned(st8), unsigned(st8)), kRelThreads, 0, st>>>(bits, n, row_words);
-    return cudaGetLastError();
+    const cudaError_t err = cudaGetLastError();
+    if (err != cudaSuccess || st8 <= 0) return err;
+    return launch_after(k_mirror, dim3(unsigned(st8), unsigned(st8)), kRelThreads, 0, st, bits, n, row_words);
 }
 
 }  // namespace cs

@@ -18,6 +18,7 @@
 #include <vector>
 
 #include "cs_kernels.cuh"
+#include "cs_launch.cuh"
 #include "cs_sprinkle.cuh"
 
 namespace cs {
@@ -105,6 +106,7 @@ constexpr int kind_dim(int kind) { return kind == CS_4D_DIAMOND ? 4 : kind == CS
 template <int KIND>
 __global__ void __launch_bounds__(kThreads) k_keys(int64_t n, uint64_t seed, const uint64_t* __restrict__ thr,
                                                    SprinkleScratch s, int bits, WsHeader* hdr) {
+    launch_dependents();
     const int64_t first = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
     for (int64_t e = first; e - (threadIdx.x & 31) < n; e += int64_t(gridDim.x) * blockDim.x) {  // whole warps
         int32_t c[4];
@@ -131,6 +133,8 @@ __global__ void __launch_bounds__(kThreads) k_keys(int64_t n, uint64_t seed, con
 // lines per thread and store); this takes about 5.
 constexpr int kScanThreads = 1024;  // the last blocks' sums in two rounds of loads
 __global__ void __launch_bounds__(kScanThreads) k_bucket_scan(SprinkleScratch s, int64_t n) {
+    launch_dependents();
+    wait_for_primary();
     const uint32_t* count = s.count[blockIdx.y];
     uint32_t* start = s.start[blockIdx.y];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -163,6 +167,8 @@ __global__ void __launch_bounds__(kScanThreads) k_bucket_scan(SprinkleScratch s,
 }
 
 __global__ void __launch_bounds__(kThreads) k_bucket_fill(int64_t n, SprinkleScratch s, int bits) {
+    launch_dependents();
+    wait_for_primary();
     const int q = blockIdx.y;
     for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < n; e += int64_t(gridDim.x) * blockDim.x)
         s.slot[q][s.start[q][s.key[q][e] >> (64 - bits)] + s.arrival[q][e]] = uint32_t(e);
@@ -186,6 +192,7 @@ __device__ __forceinline__ uint32_t rank_of(const uint64_t* __restrict__ key, co
 // Ranks and, with them, the time-sorted coordinates.
 __global__ void __launch_bounds__(kThreads) k_rank_scatter(int64_t n, int dim, bool order2d, SprinkleScratch s, int bits,
                                                            int32_t* __restrict__ coords) {
+    wait_for_primary();
     for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < n; e += int64_t(gridDim.x) * blockDim.x) {
         const uint32_t r = rank_of(s.key[0], s.start[0], s.slot[0], bits, e);
         if (order2d) {
@@ -320,10 +327,12 @@ cudaError_t sprinkle_kind(int64_t n, uint64_t seed, const uint64_t* thr, int32_t
     if (err != cudaSuccess) return err;
     const unsigned g = unsigned(grid_for(n));
     k_keys<KIND><<<g, kThreads, 0, st>>>(n, seed, thr, s, L.bits, hdr);
-    k_bucket_scan<<<dim3(unsigned(buckets / kScanBuckets), kStreams), kScanThreads, 0, st>>>(s, n);
-    k_bucket_fill<<<dim3(g, kStreams), kThreads, 0, st>>>(n, s, L.bits);
-    k_rank_scatter<<<g, kThreads, 0, st>>>(n, kind_dim(KIND), kOrder, s, L.bits, coords);
-    return cudaGetLastError();
+    if ((err = cudaGetLastError()) != cudaSuccess ||
+        (err = launch_after(k_bucket_scan, dim3(unsigned(buckets / kScanBuckets), kStreams), kScanThreads, 0, st, s,
+                            n)) != cudaSuccess ||
+        (err = launch_after(k_bucket_fill, dim3(g, kStreams), kThreads, 0, st, n, s, L.bits)) != cudaSuccess)
+        return err;
+    return launch_after(k_rank_scatter, dim3(g), kThreads, 0, st, n, kind_dim(KIND), kOrder, s, L.bits, coords);
 }
 
 }  // namespace
