@@ -67,11 +67,9 @@ __global__ void __launch_bounds__(kActThreads) k_action_partial(int dim, const i
 // One warp per eps: its partial sums, the action; warp 0 writes the bracket.
 // After k_action_partial it is launched while that one runs, and waits here
 // for its end (hist was complete before k_action_partial began).
-__global__ void __launch_bounds__(32 * kMaxEps) k_action_final(int dim, int64_t n, const int64_t* __restrict__ hist,
-                                                               int64_t len, EpsArgs eps, int T,
-                                                               const dd* __restrict__ partial,
-                                                               double* __restrict__ out,
-                                                               int64_t* __restrict__ bracket) {
+__global__ void __launch_bounds__(32 * kMaxEps) k_action_final(int dim, int64_t n, const int64_t* hist,
+                                                               int64_t len, EpsArgs eps, int T, const dd* partial,
+                                                               double* out, int64_t* bracket) {
     const int e = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int64_t h4[4] = {0, 0, 0, 0};
     for (int k = 0; k < 4 && k < len; ++k) h4[k] = hist[k];

@@ -206,8 +206,7 @@ __global__ void __launch_bounds__(kOrdBuildThreads) k_batch_order_table(const Ba
 // histogram to the set's and clears it.  order_sets: the sets in task order.
 __global__ void __launch_bounds__(kBatchOrderThreads, 2) k_batch_order_count(const BatchSet* __restrict__ sets,
                                                                           const int32_t* __restrict__ order_sets,
-                                                                          int n_order, int64_t tasks,
-                                                                          int64_t* __restrict__ hist_base) {
+                                                                          int n_order, int64_t tasks, int64_t* hist_base) {
     wait_for_primary();
     constexpr int kWarps = kBatchOrderThreads / 32;
     extern __shared__ __align__(16) uint8_t smem_ord[];
@@ -354,10 +353,10 @@ struct BatchPowers {
     EpsPowers e[kMaxEps];
     SmearCoef c[kDimSlots][kMaxEps];
 };
-__global__ void __launch_bounds__(32) k_batch_coef(dd* __restrict__ coef, CoefArgs c, EpsArgs eps,
+__global__ void __launch_bounds__(32) k_batch_coef(dd* coef, CoefArgs c, EpsArgs eps,
                                                     const __grid_constant__ BatchPowers powers,
                                                     const BatchSet* __restrict__ sets, int nsets,
-                                                    int64_t* __restrict__ kends) {
+                                                    int64_t* kends) {
     launch_dependents();
     wait_for_primary();
     const int64_t total = c.seg[kDimSlots * kMaxEps];
@@ -388,11 +387,9 @@ __global__ void __launch_bounds__(32) k_batch_coef(dd* __restrict__ coef, CoefAr
 // left the FP64 pipe waiting on the sums' dependency chains (0.29 ms for 768
 // sets and three smeared eps).
 __global__ void __launch_bounds__(kActThreads) k_batch_action(const BatchSet* __restrict__ sets,
-                                                              const int64_t* __restrict__ hist_base, EpsArgs eps,
-                                                              const dd* __restrict__ coef, CoefArgs c,
-                                                              const int64_t* __restrict__ kends,
-                                                              double* __restrict__ actions,
-                                                              int64_t* __restrict__ brackets) {
+                                                              const int64_t* hist_base, EpsArgs eps,
+                                                              const dd* coef, CoefArgs c, const int64_t* kends,
+                                                              double* actions, int64_t* brackets) {
     wait_for_primary();
     __shared__ dd red[kActThreads];
     const int per = eps.n > 0 ? eps.n : 1;  // no eps: one CTA per set for the bracket

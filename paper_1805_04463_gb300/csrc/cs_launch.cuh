@@ -11,6 +11,14 @@ namespace cs {
 // for the whole end of the kernel before, ahead of its first access to global
 // memory that any earlier work of the stream touches.  Every kernel of a
 // chain waits, so the end of one is the end of all before it.
+//
+// After the wait it reads what the chain's earlier kernels wrote by plain loads or
+// __ldcg: not by __ldg, and not through __restrict__ kernel parameters.  It
+// lives from before those writes on, and the read-only path is defined only for
+// data that nothing writes while the kernel lives; through a __restrict__
+// parameter the compiler may take that path, or move a load above the wait,
+// whose memory clobber does not bind it.  Tables that the host had written before
+// the chain's first launch are free of the rule.
 __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_for_primary() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

@@ -182,7 +182,7 @@ constexpr int kCountBins = 55296;
 
 // One CTA per SM, its warps striding over the tasks.
 __global__ void __launch_bounds__(kCountThreads, 1) k_count_order(OrderSet s, int64_t tasks, int m, int bins,
-                                                                  unsigned long long* __restrict__ hist) {
+                                                                  unsigned long long* hist) {
     extern __shared__ __align__(16) uint8_t smem_ord[];
     int2* stage = reinterpret_cast<int2*>(smem_ord) + 32 * (threadIdx.x >> 5);
     uint32_t* shist = reinterpret_cast<uint32_t*>(smem_ord + kCountStage);

@@ -46,8 +46,8 @@ __host__ __device__ inline int order_build_blocks(int64_t n) {
 }
 
 // D(64 X, y), 0 <= y < n.
-__device__ __forceinline__ int order_lookup(const uint2* __restrict__ D, int W, int X, int y) {
-    const uint2 e = __ldg(D + size_t(X) * W + (y >> 5));
+__device__ __forceinline__ int order_lookup(const uint2* D, int W, int X, int y) {
+    const uint2 e = D[size_t(X) * W + (y >> 5)];
     return int(e.y) + __popc(e.x & ((1u << (y & 31)) - 1u));
 }
 
@@ -58,12 +58,12 @@ __device__ __forceinline__ int order_lookup(const uint2* __restrict__ D, int W, 
 // range: ranks 0..n-1 and 31-bit light-cone coordinates alike).  Values in
 // [0, 2^31).  All kRankThreads threads; sk[i] is written by thread
 // i % kRankThreads.
-__device__ __forceinline__ void order_keys_smem(const int32_t* __restrict__ val, const int32_t* __restrict__ sec, int n,
+__device__ __forceinline__ void order_keys_smem(const int32_t* val, const int32_t* sec, int n,
                                                 uint64_t* sk) {
     __shared__ int lo_w[kRankThreads / 32], hi_w[kRankThreads / 32];
     int lo = INT32_MAX, hi = INT32_MIN;
     for (int i = threadIdx.x; i < n; i += kRankThreads) {
-        const int v = __ldg(val + i);
+        const int v = val[i];
         lo = min(lo, v);
         hi = max(hi, v);
     }
@@ -78,8 +78,8 @@ __device__ __forceinline__ void order_keys_smem(const int32_t* __restrict__ val,
     hi = __reduce_max_sync(0xffffffffu, hi_w[threadIdx.x & 31]);
     const int nb = 32 - __clz(max(uint32_t(hi) - uint32_t(lo), 1u));
     for (int i = threadIdx.x; i < n; i += kRankThreads)
-        sk[i] = (uint64_t(uint32_t(__ldg(val + i)) - uint32_t(lo)) << (64 - nb)) |
-                (uint64_t((0x7FFFFFFFu - uint32_t(__ldg(sec + i))) & 0x7FFFFFFFu) << (33 - nb));
+        sk[i] = (uint64_t(uint32_t(val[i]) - uint32_t(lo)) << (64 - nb)) |
+                (uint64_t((0x7FFFFFFFu - uint32_t(sec[i])) & 0x7FFFFFFFu) << (33 - nb));
 }
 
 // p and q of a set of at most 8192 elements by one CTA of kRankThreads
@@ -118,7 +118,7 @@ __device__ __forceinline__ void order_build_rows(const OrderSet& s, int g) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int X0 = g * kOrdRowsPerBlock, X = X0 + warp;
     const int a0 = kOrdBand * X + lane;  // this thread's elements: a0 and a0 + 32
-    const int p0 = a0 < s.n ? __ldg(s.p + a0) : INT32_MAX, p1 = a0 + 32 < s.n ? __ldg(s.p + a0 + 32) : INT32_MAX;
+    const int p0 = a0 < s.n ? s.p[a0] : INT32_MAX, p1 = a0 + 32 < s.n ? s.p[a0 + 32] : INT32_MAX;
     const bool row = X < order_bands(s.n);  // warp-uniform
     uint32_t carry = 0;  // elements before the step's words, in row X
     for (int w0 = 0; w0 < s.W; w0 += kOrdBuildWords) {
@@ -130,7 +130,7 @@ __device__ __forceinline__ void order_build_rows(const OrderSet& s, int g) {
 #pragma unroll
             for (int k = 0; k < 16; ++k) {
                 const int y = 32 * (w0 + wb + k * kOrdRowsPerBlock) + lane;
-                qy[k] = __ldg(s.q + min(y, s.n - 1));
+                qy[k] = s.q[min(y, s.n - 1)];
                 if (y >= s.n) qy[k] = INT32_MAX;
             }
 #pragma unroll
@@ -278,7 +278,7 @@ __device__ __forceinline__ void order_column_own(OrderRows& r, int pb, int xb, u
 
 // A column whose counts may lie at or past the bins: those add to hist_g.
 __device__ __forceinline__ void order_column_wide(OrderRows& r, int pb, int xb, int row, int own, uint32_t hist_s,
-                                                  uint32_t spare, unsigned long long* __restrict__ hist_g) {
+                                                  uint32_t spare, unsigned long long* hist_g) {
     const bool p = r.p0 < pb, q = r.p1 < pb;
     const uint32_t c = __popc(__ballot_sync(0xffffffffu, p) & r.le) + __popc(__ballot_sync(0xffffffffu, q) & r.lt);
     const uint32_t t = r.y0 + uint32_t(xb) - 4u * c, u = r.y1 + uint32_t(xb) - 4u * c;
@@ -302,7 +302,7 @@ __device__ __forceinline__ void order_column_wide(OrderRows& r, int pb, int xb, 
 // hist_s: shared address of the bins [0, bins) and a spare one; counts at or
 // past bins go to hist_g.  stage: 32 int2 of the warp.
 __device__ __forceinline__ void order_task(const OrderSet& s, int A, int C, int chunk, uint32_t hist_s, int bins,
-                                           unsigned long long* __restrict__ hist_g, int2* stage) {
+                                           unsigned long long* hist_g, int2* stage) {
     const int lane = threadIdx.x & 31, n = s.n, W = s.W;
     const int a0 = kOrdBand * A;
     const int c0 = C * chunk, cend = min(c0 + chunk, n);
@@ -318,12 +318,12 @@ __device__ __forceinline__ void order_task(const OrderSet& s, int A, int C, int 
     r.p0 = r.p1 = INT32_MAX;
     r.y0 = r.y1 = hist_s;
     if (a < n) {
-        r.p0 = __ldg(s.p + a);
-        r.y0 += 4u * uint32_t(__ldg(s.R + a) - order_lookup(s.D, W, b0 / kOrdBand, r.p0));
+        r.p0 = s.p[a];
+        r.y0 += 4u * uint32_t(s.R[a] - order_lookup(s.D, W, b0 / kOrdBand, r.p0));
     }
     if (a + 1 < n) {
-        r.p1 = __ldg(s.p + a + 1);
-        r.y1 += 4u * uint32_t(__ldg(s.R + a + 1) - order_lookup(s.D, W, b0 / kOrdBand, r.p1)) - 4u;
+        r.p1 = s.p[a + 1];
+        r.y1 += 4u * uint32_t(s.R[a + 1] - order_lookup(s.D, W, b0 / kOrdBand, r.p1)) - 4u;
     }
     // A count is below b - a, and at most y + x: in a task where it can pass the
     // bins only the columns where y + x does, for the largest y, take the
@@ -334,8 +334,8 @@ __device__ __forceinline__ void order_task(const OrderSet& s, int A, int C, int 
     auto column_of = [&](int b) {
         int2 v = make_int2(-1, 0);
         if (b < cend) {
-            v.x = __ldg(s.p + b);
-            v.y = 4 * (__ldg(s.R + b) - order_lookup(s.D, W, A, v.x));
+            v.x = s.p[b];
+            v.y = 4 * (s.R[b] - order_lookup(s.D, W, A, v.x));
         }
         return v;
     };

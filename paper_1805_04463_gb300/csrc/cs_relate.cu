@@ -49,7 +49,7 @@ void launch_upper(const int32_t* coords, int64_t n, uint64_t* bits, int64_t row_
         k_relate<G, kRelWarpWords><<<dim3(rows, unsigned(chunks)), kRelThreads, 0, st>>>(coords, n, bits, row_words);
 }
 
-__global__ void __launch_bounds__(kRelThreads, 4) k_mirror(uint64_t* __restrict__ bits, int64_t n, int64_t row_words) {
+__global__ void __launch_bounds__(kRelThreads, 4) k_mirror(uint64_t* bits, int64_t n, int64_t row_words) {
     __shared__ uint64_t sm[kMirRows][kMirTiles + 1];
     wait_for_primary();
     mirror_block(bits, n, row_words, blockIdx.x, blockIdx.y, sm);

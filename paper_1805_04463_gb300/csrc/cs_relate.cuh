@@ -69,13 +69,13 @@ struct ExactWord {
         for (int k = 0; k < 2; ++k) {
             in[k] = j0 + 32 * k < n;
 #pragma unroll
-            for (int d = 0; d < D; ++d) b[k][d] = in[k] ? __ldg(coords + d * n + j0 + 32 * k) : 0;
+            for (int d = 0; d < D; ++d) b[k][d] = in[k] ? coords[d * n + j0 + 32 * k] : 0;
         }
     }
     __device__ __forceinline__ uint64_t row(const int32_t* __restrict__ coords, int64_t n, int64_t i) const {
         int32_t a[D];
 #pragma unroll
-        for (int d = 0; d < D; ++d) a[d] = __ldg(coords + d * n + i);
+        for (int d = 0; d < D; ++d) a[d] = coords[d * n + i];
         const uint32_t lo = __ballot_sync(0xffffffffu, in[0] && rel_related<G>(a, b[0], i, j0));
         const uint32_t hi = __ballot_sync(0xffffffffu, in[1] && rel_related<G>(a, b[1], i, j0 + 32));
         return (uint64_t(hi) << 32) | lo;
@@ -310,7 +310,7 @@ __device__ __forceinline__ void relate_block(const int32_t* __restrict__ coords,
 #pragma unroll
                 for (int d = 0; d < D; ++d) {
                     const int64_t j = c0 + 2 * p + k;
-                    c[k][d] = j < n ? __ldg(coords + d * n + j) : 0;
+                    c[k][d] = j < n ? coords[d * n + j] : 0;
                     out |= c[k][d] < -kFilterRange || c[k][d] > kFilterRange;
                 }
             auto pair = [&](int d) { return f2_pack(float(c[0][d]), float(c[1][d])); };
@@ -326,7 +326,7 @@ __device__ __forceinline__ void relate_block(const int32_t* __restrict__ coords,
         if (threadIdx.x < 64 && r0 + threadIdx.x < n) {
 #pragma unroll
             for (int d = 0; d < D; ++d) {
-                const int32_t x = __ldg(coords + d * n + r0 + threadIdx.x);
+                const int32_t x = coords[d * n + r0 + threadIdx.x];
                 out |= x < -kFilterRange || x > kFilterRange;
             }
         }
@@ -339,7 +339,7 @@ __device__ __forceinline__ void relate_block(const int32_t* __restrict__ coords,
 #pragma unroll
                 for (int d = (G == kGeomOrder ? 1 : 0); d < 2; ++d) {
                     const int64_t j = c0 + 2 * p + k;
-                    c[k][d] = j < n ? __ldg(coords + d * n + j) : 0;
+                    c[k][d] = j < n ? coords[d * n + j] : 0;
                 }
             if constexpr (G == kGeomOrder)
                 reinterpret_cast<int2*>(smem)[p] = make_int2(c[0][1], c[1][1]);
@@ -359,7 +359,7 @@ __device__ __forceinline__ void relate_block(const int32_t* __restrict__ coords,
         const int64_t i = r0 + lane + 32 * r;
         int32_t c[D];
 #pragma unroll
-        for (int d = 0; d < D; ++d) c[d] = i < n ? __ldg(coords + d * n + i) : 0;
+        for (int d = 0; d < D; ++d) c[d] = i < n ? coords[d * n + i] : 0;
         if constexpr (kFilter) {
 #pragma unroll
             for (int d = 0; d < D; ++d) {
@@ -410,7 +410,7 @@ __device__ __forceinline__ void relate_block(const int32_t* __restrict__ coords,
                     if constexpr (G == kGeomLightCone || G == kGeomOrder) x = ~x;  // sign set: not in the future cone
                     found[r] = x & valid;
                     if constexpr (kFilter) exact[r] = band[r] <= kBandBits;
-                    if constexpr (G == kGeomDeSitter) exact[r] = row[r].nu == __ldg(coords + 64 * W);
+                    if constexpr (G == kGeomDeSitter) exact[r] = row[r].nu == coords[64 * W];
                 }
             }
             const uint32_t todo0 = __ballot_sync(0xffffffffu, exact[0] && r0 + lane < n);
@@ -707,7 +707,7 @@ __device__ __forceinline__ void transpose64(uint64_t& x, uint64_t& y, const Tr32
 
 // Super-tile (A8, B8): output rows [512 A8, 512 A8 + 512), output words
 // [8 B8, 8 B8 + 8).  sm: 512 x 9 words of shared memory.  All 256 threads.
-__device__ __forceinline__ void mirror_block(uint64_t* __restrict__ bits, int64_t n, int64_t row_words, int64_t A8,
+__device__ __forceinline__ void mirror_block(uint64_t* bits, int64_t n, int64_t row_words, int64_t A8,
                                              int64_t B8, uint64_t (*sm)[kMirTiles + 1]) {
     const int64_t tiles = (n + 63) >> 6;  // row tiles = valid words
     const int64_t A0 = A8 * kMirTiles, B0 = B8 * kMirTiles;
@@ -726,7 +726,7 @@ __device__ __forceinline__ void mirror_block(uint64_t* __restrict__ bits, int64_
     for (int s = 0; s < kPerThread; ++s) {
         const int t = threadIdx.x + s * kRelThreads;
         const int64_t row = 64 * B0 + t / (kMirTiles / 2), word = A0 + 2 * (t % (kMirTiles / 2));
-        v[s] = (row < n && word < tiles) ? __ldg(reinterpret_cast<const ulonglong2*>(bits + row * row_words + word))
+        v[s] = (row < n && word < tiles) ? __ldcg(reinterpret_cast<const ulonglong2*>(bits + row * row_words + word))
                                          : make_ulonglong2(0ull, 0ull);
     }
 #pragma unroll

@@ -175,8 +175,8 @@ __global__ void __launch_bounds__(kThreads) k_bucket_fill(int64_t n, SprinkleScr
 }
 
 // Rank of element e's key, ties by index.
-__device__ __forceinline__ uint32_t rank_of(const uint64_t* __restrict__ key, const uint32_t* __restrict__ start,
-                                            const uint32_t* __restrict__ slot, int bits, int64_t e) {
+__device__ __forceinline__ uint32_t rank_of(const uint64_t* key, const uint32_t* start, const uint32_t* slot, int bits,
+                                            int64_t e) {
     const uint64_t ke = key[e];
     const uint32_t b = uint32_t(ke >> (64 - bits));
     const uint32_t begin = start[b], end = start[b + 1];
@@ -191,7 +191,7 @@ __device__ __forceinline__ uint32_t rank_of(const uint64_t* __restrict__ key, co
 
 // Ranks and, with them, the time-sorted coordinates.
 __global__ void __launch_bounds__(kThreads) k_rank_scatter(int64_t n, int dim, bool order2d, SprinkleScratch s, int bits,
-                                                           int32_t* __restrict__ coords) {
+                                                           int32_t* coords) {
     wait_for_primary();
     for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < n; e += int64_t(gridDim.x) * blockDim.x) {
         const uint32_t r = rank_of(s.key[0], s.start[0], s.slot[0], bits, e);
