@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(kActThreads) k_action_partial(int dim, const i
     for (int64_t k = int64_t(blockIdx.x) * T + tid; k < kend; k += int64_t(nb) * T) {
         const int64_t hk = hist[k];
         if (hk == 0) continue;
-        sum = dd_accumulate(sum, hk, smear_term(dim, powers.c[e], powers.e[e], k));
+        sum = dd_add(sum, dd_times_i64(smear_term(dim, powers.c[e], powers.e[e], k), hk));
     }
     sum = warp_sum_dd(sum);
     if (T > 32) {  // uniform

@@ -48,59 +48,53 @@ __device__ __forceinline__ dd power_of(const EpsPowers& t, int64_t k) {
     return r;
 }
 
-// The polynomial factor of f_d (smear_poly) as a - b k + c t - d C(k, 3),
-// t = k (k - 1) / 2, its coefficients and the values f_d(k), k < deg, found
-// on the host: they hold no k, and were most of a term's FP64 operations.
-// Rounded once to double-double, they move a sum by less than 1e-30 of its
-// largest term (terms: the same error as with the products formed per k).
+// f times a whole number, c as exactly as it stands: one double below 2^53 (every
+// count of a set), both halves of the int64 from there on (a caller's histogram).
+__host__ __device__ __forceinline__ dd dd_times_i64(dd f, int64_t c) {
+    if (c < (int64_t(1) << 53) && c > -(int64_t(1) << 53)) return dd_mul_d(f, static_cast<double>(c));
+    return dd_mul(dd_from_i64(c), f);
+}
+
+// What smear_poly holds without k, and the values f_d(k), k < deg, found on
+// the host: products of q and eps were half of a term's FP64 operations.  What
+// is left per k are smear_poly's own products, to the last bit.  (With
+// coefficients a - b k + c t - d C(k, 3) rounded on the host a term took up to ten operations
+// less, but their roundings are the same in every term: the sum's error was
+// 8e-31 of its largest term instead of 3e-31.)
 struct SmearCoef {
-    dd a, b, c, d, f[3];
+    dd a, q, e2, d, f[3];  // q^deg; q (3+1: q^2) and q; eps^2; 8 eps^3
+    dd q1;
+    double e;
 };
 inline SmearCoef smear_coef(int dim, double eps) {
-    const dd q = dd_two_sum(1.0, -eps), e = dd_from(eps), q2 = dd_mul(q, q), e2 = dd_mul(e, e);
+    const dd q = dd_two_sum(1.0, -eps), e = dd_from(eps), q2 = dd_mul(q, q);
     SmearCoef r;
-    r.d = dd_from(0.0);
-    if (dim == 2) {
-        r.a = q2, r.b = dd_mul(dd_mul_d(e, 2.0), q), r.c = e2;
-    } else if (dim == 3) {
-        r.a = q2, r.b = dd_mul(dd_mul_d(e, 3.375), q), r.c = dd_mul_d(e2, 2.25);
-    } else {
-        r.a = dd_mul(q2, q), r.b = dd_mul(dd_mul_d(e, 9.0), q2), r.c = dd_mul(dd_mul_d(e2, 16.0), q);
-        r.d = dd_mul_d(dd_mul(e2, e), 8.0);
-    }
+    r.e = eps;
+    r.q1 = q;
+    r.q = dim == 4 ? q2 : q;
+    r.a = dim == 4 ? dd_mul(q2, q) : q2;
+    r.e2 = dd_mul(e, e);
+    r.d = dd_mul_d(dd_mul(r.e2, e), 8.0);
     for (int k = 0; k < 3; ++k) r.f[k] = smear_poly(dim, k, q, eps);
     return r;
 }
 __host__ __device__ __forceinline__ dd smear_poly_at(int dim, const SmearCoef& m, int64_t k) {
-    const int64_t t = k * (k - 1) / 2;  // below 2^43 for k < 2^22: exact in a double
-    const dd bk = dd_mul_d(m.b, static_cast<double>(k)), ct = dd_mul_d(m.c, static_cast<double>(t));
-    dd r = dd_add(dd_sub(m.a, bk), ct);
-    if (dim == 4) {
-        const int64_t w = k - 2;
-        const dd c3 = w % 3 == 0 ? dd_two_prod(static_cast<double>(t), static_cast<double>(w / 3))
-                                 : dd_two_prod(static_cast<double>(t / 3), static_cast<double>(w));  // C(k, 3), exactly
-        r = dd_sub(r, dd_mul(m.d, c3));
-    }
-    return r;
+    const int64_t t = k * (k - 1) / 2;
+    const double x = static_cast<double>(k);
+    const dd b = dd_mul(dd_two_prod(m.e, (dim == 2 ? 2.0 : dim == 3 ? 3.375 : 9.0) * x), m.q);
+    if (dim == 2) return dd_add(dd_sub(m.a, b), dd_times_i64(m.e2, t));
+    if (dim == 3) return dd_add(dd_sub(m.a, b), dd_mul_d(m.e2, 2.25 * static_cast<double>(t)));
+    const int64_t w = k - 2;
+    const dd c3 = w % 3 == 0 ? dd_two_prod(static_cast<double>(t), static_cast<double>(w / 3))
+                             : dd_two_prod(static_cast<double>(t / 3), static_cast<double>(w));  // C(k, 3), exactly
+    const dd c = dd_mul(dd_times_i64(m.e2, 16 * t), m.q1);
+    return dd_sub(dd_add(dd_sub(m.a, b), c), dd_mul(m.d, c3));
 }
 // f_d(k).
 __device__ __forceinline__ dd smear_term(int dim, const SmearCoef& m, const EpsPowers& t, int64_t k) {
     const int64_t deg = smear_deg(dim);
     if (k < deg) return m.f[k];
     return dd_mul(power_of(t, k - deg), smear_poly_at(dim, m, k));
-}
-
-// sum + c * f for a count c < 2^53 (exact as a double): the product to double-double,
-// its high part added with its rounding error kept, the low parts in plain
-// FP64.  The low sums stay below 2^-53 of the high ones, so what is lost is
-// below 2^-105 of the largest partial sum per term, at 15 FP64 operations
-// where the full double-double product and sum take 34.
-__device__ __forceinline__ dd dd_accumulate(dd sum, int64_t c, dd f) {
-    const double x = static_cast<double>(c);
-    const double p = x * f.hi;
-    const double e = fma(x, f.lo, fma(x, f.hi, -p));
-    const dd s = dd_two_sum(sum.hi, p);
-    return {s.hi, sum.lo + (s.lo + e)};
 }
 
 struct EpsArgs {

@@ -417,7 +417,7 @@ __global__ void __launch_bounds__(kActThreads) k_batch_action(const BatchSet* __
     dd sum = dd_from(0.0);
     for (int64_t k = tid; k < kend; k += kActThreads) {
         const int64_t hk = hist[k];
-        if (hk != 0) sum = dd_accumulate(sum, hk, f[k]);
+        if (hk != 0) sum = dd_add(sum, dd_times_i64(f[k], hk));
     }
     red[tid] = sum;
     __syncthreads();
