@@ -180,6 +180,15 @@ constexpr int kCountStage = kCountWarps * 32 * int(sizeof(int2));
 // pairs of a 2^17 order lie past 55296 bins), so wide sets spill little.
 constexpr int kCountBins = 55296;
 
+// Bands per column chunk, at most, and the tasks a warp takes between two
+// flushes of the bins: a CTA's adds in between stay below 2^32 however few CTAs
+// share the pairs, and so does every bin.  (One flush at the end holds up to n = 2^20 on 152 SMs, not on
+// 128.)  Up to n = 2^18 a warp's whole share is less than this on 152 SMs.
+constexpr int kCountMaxM = 16;
+constexpr int64_t kFlushTasks = 256;
+static_assert(kFlushTasks * kCountWarps * kOrdBand * (kOrdBand * kCountMaxM) < (int64_t(1) << 32),
+              "a bin holds every pair between two flushes");
+
 // One CTA per SM, its warps striding over the tasks.
 __global__ void __launch_bounds__(kCountThreads, 1) k_count_order(OrderSet s, int64_t tasks, int m, int bins,
                                                                   unsigned long long* hist) {
@@ -191,15 +200,23 @@ __global__ void __launch_bounds__(kCountThreads, 1) k_count_order(OrderSet s, in
     __syncthreads();
     const uint32_t hist_s = smem_u32(shist);
     const int64_t warps = int64_t(gridDim.x) * kCountWarps;
-    for (int64_t t = int64_t(threadIdx.x >> 5) * gridDim.x + blockIdx.x; t < tasks; t += warps) {
-        int A, C;
-        order_decode(t, m, A, C);
-        order_task(s, A, C, kOrdBand * m, hist_s, bins, hist, stage);
-    }
-    __syncthreads();
-    for (int k = threadIdx.x; k < bins; k += kCountThreads) {
-        const uint32_t c = shist[k];
-        if (c) atomicAdd(hist + k, (unsigned long long)c);
+    int64_t t = int64_t(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    for (int64_t end = kFlushTasks * warps;; end += kFlushTasks * warps) {
+        for (const int64_t stop = end < tasks ? end : tasks; t < stop; t += warps) {
+            int A, C;
+            order_decode(t, m, A, C);
+            order_task(s, A, C, kOrdBand * m, hist_s, bins, hist, stage);
+        }
+        __syncthreads();
+        for (int k = threadIdx.x; k < bins; k += kCountThreads) {
+            const uint32_t c = shist[k];
+            if (c) {
+                atomicAdd(hist + k, (unsigned long long)c);
+                shist[k] = 0u;
+            }
+        }
+        if (end >= tasks) return;
+        __syncthreads();
     }
 }
 
@@ -244,8 +261,7 @@ std::atomic<bool> g_order_attr[64];  // per device: the large-shared-memory attr
 
 bool order_kind(int kind) { return kind == CS_2D_ORDER || kind == CS_2D_DIAMOND || kind == CS_2D_SQUARE; }
 
-// The count's 32-bit shared bins hold every pair of a CTA's share (n^2 / 2 over
-// the SMs) up to n = 2^20.
+// Up to the largest set that the count is checked at (its table takes 4.3 GB there).
 bool order_count_fits(int kind, int64_t n) { return order_kind(kind) && n >= 2 && n <= (int64_t(1) << 20); }
 
 size_t order_workspace_bytes(int64_t n) { return order_layout(n).total; }
@@ -313,7 +329,7 @@ cudaError_t launch_count_order(int kind, int64_t n, const int32_t* coords, int64
     // Column chunks of 64 m: long enough to amortise a task's start (two
     // dependent gathers), short enough that the warps get several tasks each.
     const int sms = device_sm_count();
-    int m = 16;
+    int m = kCountMaxM;
     while (m > 1 && order_tasks(n, m) < int64_t(sms) * kCountWarps * 12) m >>= 1;
     const int64_t tasks = order_tasks(n, m);
     const int bins = int(len < kCountBins ? len : kCountBins);
