@@ -1,9 +1,9 @@
 // cs_order.cu -- the single-set interval count of product orders
 // (cs_order.cuh): ranks of the two coordinates, the table D, the pair count.
 //
-// Ranks.  Up to 8192 elements one CTA ranks them by buckets in shared memory.
-// Beyond, the callers' coordinates may be distributed anyhow, so the ranks
-// come from sorted tiles: every tile of 4096 elements is sorted in shared
+// Ranks.  Callers' coordinates may be distributed anyhow.  Up to 8192 elements
+// one CTA ranks them by buckets in shared memory, or, where a bucket holds many of
+// them, sorts them there.  Beyond, the ranks come from sorted tiles: every tile of 4096 elements is sorted in shared
 // memory, and an element's rank is the sum over the tiles of its lower (or
 // upper) bound -- n / 4096 binary searches of twelve steps, under 1% of the
 // n^2 / 2 pairs counted after it and the same for every distribution.
@@ -136,9 +136,9 @@ __device__ __forceinline__ void order_ranks_small(const int32_t* __restrict__ co
     const bool v = kByU || blockIdx.x == 1;
     order_keys_smem(v ? coords + n : coords, v ? coords : coords + n, n, sk);
     if (v)
-        rank_keys_smem<true>(n, lgP, sk, cnt, slot, rank);
+        rank_keys_smem<true, true>(n, lgP, sk, cnt, slot, rank);
     else
-        rank_keys_smem<false>(n, lgP, sk, cnt, slot, rank);
+        rank_keys_smem<false, true>(n, lgP, sk, cnt, slot, rank);
     if (kByU) {
         for (int e = threadIdx.x; e < n; e += kRankThreads) {
             const int r = int(rank[e]);
