@@ -24,11 +24,15 @@ namespace {
 // de Sitter slab n = 50021 632 / 253 us, 1+1 diamond n = 30011 79 / 79 us, 2D
 // order n = 131072 789 / 802 us.  What bounds it now is the integer pipe (the
 // circle 83%, the light cone 70%), in 3+1 the FMA pipe (53%) with it (44%).
+//
+// The mirror is launched behind it without an early trigger: its blocks
+// come when the last ones here end.  Triggered at the start they crowded onto the few SMs that
+// still had room, four to an SM: with the mirror, early / so, slab n = 4099 19.3 / 13.3 us,
+// 3+1 n = 7000 29.5 / 25.4, n >= 12000 alike (an ordinary launch: 16.9, 29.2).
 template <int G, int kWords>
 __global__ void __launch_bounds__(kRelThreads) k_relate(const int32_t* __restrict__ coords, int64_t n,
                                                         uint64_t* __restrict__ bits, int64_t row_words) {
     __shared__ __align__(16) uint8_t sm[relate_stage_bytes(G)];
-    launch_dependents();
     relate_block<G, kWords>(coords, n, bits, row_words, blockIdx.x,
                             int64_t(blockIdx.y) * (kWords * (kRelThreads / 32)), sm);
 }
