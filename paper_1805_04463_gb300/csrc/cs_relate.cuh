@@ -14,18 +14,16 @@ constexpr int kRelWarpWords = kRelWordsPerBlock / (kRelThreads / 32);  // words 
 static_assert(kRelWarpWords == 4, "a warp's words of a row are one sector");
 
 // Geometries of the relation test; the number of coordinates is geom_dim(G).
-// kGeomOrder: a random 2D order labelled by u (u increases with the label).
-constexpr int kGeomLightCone = 2, kGeom3 = 3, kGeom4 = 4, kGeomDeSitter = 5, kGeomOrder = 6;
+constexpr int kGeomLightCone = 2, kGeom3 = 3, kGeom4 = 4, kGeomDeSitter = 5;
 constexpr int geom_dim(int g) { return g == kGeom3 || g == kGeom4 ? g : 2; }
 
-// Symmetric timelike test between elements i and j (coordinates a, b): du * dv > 0 (1+1,
+// Symmetric timelike test between two elements (coordinates a, b): du * dv > 0 (1+1,
 // light-cone coordinates), dt^2 - |dx|^2 > 0 (2+1, 3+1) exact in int64, or,
 // on a circle (the de Sitter slab's conformal grid, Eq. ds_metric, and the
 // 1+1 cylinder), the angular separation below the (conformal-)time
 // separation.
 template <int G>
-__device__ __forceinline__ bool rel_related(const int32_t (&a)[geom_dim(G)], const int32_t (&b)[geom_dim(G)],
-                                            int64_t i, int64_t j) {
+__device__ __forceinline__ bool rel_related(const int32_t (&a)[geom_dim(G)], const int32_t (&b)[geom_dim(G)]) {
     if constexpr (G == kGeomDeSitter) {
         // |eta| < 2^30 (slab: < 2^29, cylinder: < 2^31 / pi), so de fits
         // int32; theta differences wrap modulo 2^32, one full turn.
@@ -38,8 +36,6 @@ __device__ __forceinline__ bool rel_related(const int32_t (&a)[geom_dim(G)], con
         const int32_t du = b[0] - a[0];
         const int32_t dv = b[1] - a[1];
         return (du ^ dv) >= 0 && du != 0 && dv != 0;
-    } else if constexpr (G == kGeomOrder) {
-        return j > i ? b[1] > a[1] : (j < i && b[1] < a[1]);
     } else {
         // |coordinates| < 2^29: differences fit int32 and each square is one
         // widening multiply-add into the int64 sum (< 2^62, exact)
@@ -76,8 +72,8 @@ struct ExactWord {
         int32_t a[D];
 #pragma unroll
         for (int d = 0; d < D; ++d) a[d] = coords[d * n + i];
-        const uint32_t lo = __ballot_sync(0xffffffffu, in[0] && rel_related<G>(a, b[0], i, j0));
-        const uint32_t hi = __ballot_sync(0xffffffffu, in[1] && rel_related<G>(a, b[1], i, j0 + 32));
+        const uint32_t lo = __ballot_sync(0xffffffffu, in[0] && rel_related<G>(a, b[0]));
+        const uint32_t hi = __ballot_sync(0xffffffffu, in[1] && rel_related<G>(a, b[1]));
         return (uint64_t(hi) << 32) | lo;
     }
 };
@@ -140,13 +136,10 @@ __device__ __forceinline__ int32_t circle_gap(int32_t d, int32_t ei, int32_t ej)
     return int32_t(a + uint32_t(ei) - uint32_t(ej));
 }
 
-// Staged bytes per column: u and v (light cone, circle), v alone (2D order),
-// the coordinates and A (filtered 2+1, 3+1).
+// Staged bytes per column: u and v (light cone, circle), the coordinates and
+// A (filtered 2+1, 3+1).
 __host__ __device__ constexpr int relate_stage_bytes(int g) {
-    return kRelColsPerBlock * (g == kGeomOrder                              ? 4
-                               : g == kGeomLightCone || g == kGeomDeSitter ? 8
-                               : g == kGeom3                               ? 16
-                                                                           : 20) +
+    return kRelColsPerBlock * (g == kGeomLightCone || g == kGeomDeSitter ? 8 : g == kGeom3 ? 16 : 20) +
            16;  // and a runtime 1 (the multiplier)
 }
 
@@ -213,20 +206,6 @@ __device__ __forceinline__ void relate_word(const uint8_t* __restrict__ smem, in
                     }
                 }
             }
-        } else if constexpr (G == kGeomOrder) {
-            const int4* q = reinterpret_cast<const int4*>(smem) + pbase / 2;  // four columns
-#pragma unroll
-            for (int p = 8 * h + 7; p >= 8 * h; --p) {
-                const int4 v = q[p];
-#pragma unroll
-                for (int r = 0; r < 2; ++r) {
-                    uint32_t& a = r == 0 ? s0 : s1;
-                    a = push_sign(uint32_t(cone_mad(v.w, one, row[r].nv)), a);
-                    a = push_sign(uint32_t(cone_mad(v.z, one, row[r].nv)), a);
-                    a = push_sign(uint32_t(cone_mad(v.y, one, row[r].nv)), a);
-                    a = push_sign(uint32_t(cone_mad(v.x, one, row[r].nv)), a);
-                }
-            }
         } else {
             const int4* q = reinterpret_cast<const int4*>(smem) + pbase;  // two columns
 #pragma unroll
@@ -270,7 +249,6 @@ __device__ __forceinline__ void relate_word(const uint8_t* __restrict__ smem, in
 //   light cone: x_j - x_i - 1 < 0 for u or v (coordinates in [0, 2^31): no
 //     overflow), one integer multiply-add each (x_j * 1 + ~x_i, the multiplier a runtime 1
 //     that keeps it on the FMA pipe; compares and ORs held the integer pipe);
-//   2D order: the same for v alone;
 //   circle: |dtheta| - deta < 0, dtheta modulo 2^32 in [-2^31, 2^31) and
 //     0 <= deta < 2^31: exact in 32 bits but where deta = 0 and |dtheta| = 2^31,
 //     so a word whose first column has the row's eta is found exactly;
@@ -337,14 +315,11 @@ __device__ __forceinline__ void relate_block(const int32_t* __restrict__ coords,
 #pragma unroll
             for (int k = 0; k < 2; ++k)
 #pragma unroll
-                for (int d = (G == kGeomOrder ? 1 : 0); d < 2; ++d) {
+                for (int d = 0; d < 2; ++d) {
                     const int64_t j = c0 + 2 * p + k;
                     c[k][d] = j < n ? coords[d * n + j] : 0;
                 }
-            if constexpr (G == kGeomOrder)
-                reinterpret_cast<int2*>(smem)[p] = make_int2(c[0][1], c[1][1]);
-            else
-                reinterpret_cast<int4*>(smem)[p] = make_int4(c[0][0], c[0][1], c[1][0], c[1][1]);
+            reinterpret_cast<int4*>(smem)[p] = make_int4(c[0][0], c[0][1], c[1][0], c[1][1]);
         }
         if (threadIdx.x == 0) *one_s = 1;
         __syncthreads();
@@ -407,7 +382,7 @@ __device__ __forceinline__ void relate_block(const int32_t* __restrict__ coords,
 #pragma unroll
                 for (int r = 0; r < 2; ++r) {
                     uint64_t x = (uint64_t(acc[r][1]) << 32) | acc[r][0];
-                    if constexpr (G == kGeomLightCone || G == kGeomOrder) x = ~x;  // sign set: not in the future cone
+                    if constexpr (G == kGeomLightCone) x = ~x;  // sign set: not in the future cone
                     found[r] = x & valid;
                     if constexpr (kFilter) exact[r] = band[r] <= kBandBits;
                     if constexpr (G == kGeomDeSitter) exact[r] = row[r].nu == coords[64 * W];
@@ -459,6 +434,127 @@ __device__ __forceinline__ void relate_block(const int32_t* __restrict__ coords,
     if (zero_from >= 0 && zero_from < row_words)
         for (int64_t i = r0 + warp; i < r0 + 64 && i < n; i += kRelThreads / 32)
             for (int64_t w = zero_from + lane; w < row_words; w += 32) bits[i * row_words + w] = 0ull;
+}
+
+// ------------------------------------------- light-cone kinds, a lane per word
+//
+// Labels are in time order, so in a word wholly after the row tile only the
+// future cone can hold (u_j > u_i and v_j > v_i); for a random 2D order labelled
+// by u the u test is implied by j > i and only v is compared (kUseU = false).
+// Each lane owns one word (64 columns) of the block's 32 and tests its columns one by one, for
+// four rows at a time, with no ballots: one or two multiply-adds per test as above, an OR with u,
+// and a funnel shift that appends the sign bit to the half-word's
+// accumulator (the complement of the relation bits).
+// The column coordinates are staged transposed, st[c][w] = column 64 w + c
+// (row pitch kConePitch: the lanes' reads of one offset c hit consecutive
+// banks); columns at or beyond n are staged as 0, which no cone test
+// passes.  The row tile's own word (lane rb - w0) takes the full symmetric test
+// by ballots in all eight warps; words before the row tile are left to mirror_block.
+constexpr int kConePitch = kRelWordsPerBlock + 1;  // staged words per column offset
+constexpr int kConeRows = 4;                       // rows a lane tests together
+constexpr int kConeOne = 2 * 64 * kConePitch;      // after the (u, v) staging: a runtime 1 (the multiplier)
+constexpr int kConeInts = kConeOne + 1;
+
+// The 64 rows from r0 of one block whose columns are staged in st; ws: the own word, < 0: none.
+template <bool kUseU>
+__device__ __forceinline__ void relate_rows_cone(const int32_t* __restrict__ coords, int64_t n,
+                                                 uint64_t* __restrict__ bits, int64_t row_words, int64_t w0,
+                                                 int64_t r0, int64_t r1, int ws, const int32_t* __restrict__ st) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    constexpr int kWarps = kRelThreads / 32;
+    const int2* st2 = reinterpret_cast<const int2*>(st);  // kUseU: (u, v) pairs
+    const int wbeg = ws > 0 ? ws : 0;
+    const int32_t one = st[kConeOne];
+    for (int64_t ib = r0 + int64_t(warp) * kConeRows; ib < r1; ib += int64_t(kWarps) * kConeRows) {
+        int32_t ru[kConeRows], rv[kConeRows], nu[kConeRows], nv[kConeRows];
+        uint32_t lo[kConeRows], hi[kConeRows];
+#pragma unroll
+        for (int r = 0; r < kConeRows; ++r) {
+            const int64_t i = ib + r;
+            ru[r] = i < r1 ? coords[i] : INT32_MAX;  // a missing row passes no test
+            rv[r] = i < r1 ? coords[n + i] : INT32_MAX;
+            nu[r] = ~ru[r];  // -x_i - 1
+            nv[r] = ~rv[r];
+            lo[r] = hi[r] = 0u;
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {  // the word's low and high halves
+            // highest column first: after 32 shifts column 32 h is bit 0
+#pragma unroll 8
+            for (int c = 32 * h + 31; c >= 32 * h; --c) {
+                int32_t xu = 0, xv;
+                if constexpr (kUseU) {
+                    const int2 x = st2[c * kConePitch + lane];
+                    xu = x.x;
+                    xv = x.y;
+                } else {
+                    xv = st[c * kConePitch + lane];
+                }
+#pragma unroll
+                for (int r = 0; r < kConeRows; ++r) {
+                    // sign bit set iff the column is not in the future cone
+                    const int32_t d = kUseU ? (cone_mad(xu, one, nu[r]) | cone_mad(xv, one, nv[r]))
+                                            : cone_mad(xv, one, nv[r]);
+                    if (h == 0)
+                        lo[r] = __funnelshift_l(uint32_t(d), lo[r], 1);
+                    else
+                        hi[r] = __funnelshift_l(uint32_t(d), hi[r], 1);
+                }
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < kConeRows; ++r) {
+            const int64_t i = ib + r;
+            if (i >= r1) break;  // warp-uniform
+            uint64_t word = ~((uint64_t(hi[r]) << 32) | lo[r]);
+            if (ws >= 0) {  // the row tile's own word: full test (warp-uniform)
+                bool b[2];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int k = lane + 32 * h;  // column offset in the word
+                    const int64_t j = (w0 + ws) * 64 + k;
+                    if constexpr (kUseU) {
+                        const int2 x = st2[k * kConePitch + ws];
+                        const int32_t du = x.x - ru[r], dv = x.y - rv[r];
+                        b[h] = j < n && (du ^ dv) >= 0 && du != 0 && dv != 0;
+                    } else {  // u increases with the label
+                        const int32_t xv = st[k * kConePitch + ws];
+                        b[h] = j < n && (j > i ? xv > rv[r] : (j < i && xv < rv[r]));
+                    }
+                }
+                const uint64_t d = (uint64_t(__ballot_sync(0xffffffffu, b[1])) << 32) | __ballot_sync(0xffffffffu, b[0]);
+                if (lane == ws) word = d;
+            }
+            if (lane >= wbeg && w0 + lane < row_words) bits[i * row_words + w0 + lane] = word;
+        }
+    }
+}
+
+// Rows [64 rb, 64 rb + 64) x words [w0, w0 + 32), w0 a multiple of 32.  order2d: only v is
+// staged and tested.  st: kConeInts ints, 16-byte aligned (no __restrict__: the threads
+// read one another's columns).  All 256 threads.
+__device__ __forceinline__ void relate_block_cone(const int32_t* __restrict__ coords, int64_t n,
+                                                  uint64_t* __restrict__ bits, int64_t row_words, int64_t rb,
+                                                  int64_t w0, int32_t* st, bool order2d) {
+    if (w0 + kRelWordsPerBlock <= rb) return;  // wholly below the diagonal
+    const int ws = rb < w0 ? -1 : int(rb - w0);
+    const int wbeg = ws > 0 ? ws : 0;
+    const int64_t c0 = w0 * 64, r0 = rb * kRelRowsPerBlock;
+    const int64_t r1 = r0 + kRelRowsPerBlock < n ? r0 + kRelRowsPerBlock : n;
+    for (int t = threadIdx.x + 64 * wbeg; t < kRelColsPerBlock; t += kRelThreads) {
+        const int64_t col = c0 + t;
+        const int at = (t & 63) * kConePitch + (t >> 6);
+        if (order2d)
+            st[at] = col < n ? coords[n + col] : 0;
+        else
+            reinterpret_cast<int2*>(st)[at] = col < n ? make_int2(coords[col], coords[n + col]) : make_int2(0, 0);
+    }
+    if (threadIdx.x == 0) st[kConeOne] = 1;
+    __syncthreads();
+    if (order2d)
+        relate_rows_cone<false>(coords, n, bits, row_words, w0, r0, r1, ws, st);
+    else
+        relate_rows_cone<true>(coords, n, bits, row_words, w0, r0, r1, ws, st);
 }
 
 // ------------------------------------------------ light-cone column tables

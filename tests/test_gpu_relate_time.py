@@ -1,6 +1,6 @@
 """Causal matrices of the 1+1 kinds take no longer than a 3+1 diamond's of the same size, whose
 test is five packed operations per two pairs: the slab at a size where the mirror's blocks could crowd onto the
-SMs that the upper part leaves first."""
+SMs that the upper part leaves first, the 2D order where the chunks are few."""
 import pytest
 
 pytestmark = pytest.mark.gpu
@@ -24,7 +24,7 @@ def _best(cs, kind, n):
     return min(times)
 
 
-@pytest.mark.parametrize("kind,n", [(4, 4099)])
+@pytest.mark.parametrize("kind,n", [(4, 4099), (0, 5000)])
 def test_against_3d_space(kind, n):
     from paper_1805_04463_gb300 import build
     build.build()
