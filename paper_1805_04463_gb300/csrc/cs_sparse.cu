@@ -176,13 +176,16 @@ __global__ void k_scan_add(int64_t* __restrict__ out, int64_t n, const int64_t* 
 //     where half of the bits are set);
 //   many: word after word (read by broadcast), lane l placing bits l and l + 32 by
 //     their rank within the word: consecutive places, one pass per store and
-//     the same cost whatever is set, about that of the first way at 640
-//     relations a step (with a limit of 320 the lists of a de Sitter slab,
-//     whose steps hold up to 650, took 341 us instead of 308).
+//     the same cost whatever is set.  From 1024 relations a step on, where no
+//     kind measured loses by it: with a limit of 640 the past lists of a cylinder of 45000 took
+//     354 us and of a 2D order 543, with 1024 341 and 539 (first way alone 337 and 569); a
+//     diamond's, a square's, a 3+1 one's are alike from 640 to 1280.
+// The choice needs the step's total, by one reduction beside the scan rather than
+// behind it (behind: lists of a slab of 45000 277.9 us, so 276.0, without the second way 274.5).
 // Future list of a 1+1 diamond, n = 30011: 398 -> 205 us (4.4 TB/s).
 constexpr int kColsWarps = 4;                      // warps per block
 constexpr int kColsRun = 32 * 64 + 4;              // the most columns one step emits, and an alignment shift
-constexpr int kManyColumns = 640;                  // columns of a step from which they are placed word after word
+constexpr int kManyColumns = 1024;                 // columns of a step from which they are placed word after word
 __global__ void __launch_bounds__(kColsWarps * 32) k_side_columns(const uint64_t* __restrict__ bits, int64_t n,
                                                                    int64_t row_words, bool future,
                                                                    const int64_t* __restrict__ offsets,
@@ -209,13 +212,13 @@ __global__ void __launch_bounds__(kColsWarps * 32) k_side_columns(const uint64_t
             uint64_t x = w < whi ? xn & side_mask(i, w, future) : 0ull;
             xn = w + 32 < whi ? __ldg(row + w + 32) : 0ull;
             const int c = __popcll(x);
+            const int total = int(__reduce_add_sync(0xffffffffu, unsigned(c)));
             int incl = c;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
                 const int t = __shfl_up_sync(0xffffffffu, incl, o);
                 if (lane >= o) incl += t;
             }
-            const int total = __shfl_sync(0xffffffffu, incl, 31);
             // element k of the run goes to cols[pos + k] and to run[s0 + k],
             // s0 = that position's 4-byte slot in its 16-byte group, so the
             // run's 16-byte groups are the output's
