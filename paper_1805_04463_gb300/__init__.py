@@ -363,19 +363,22 @@ def evaluate(kind, n, seed=0, coords_host=None, path=PATH_AUTO, eps=(), stream=N
 # ---------------------------------------------------- device buffer helper
 
 class Buffers:
-    """Device buffers for one causal set of `kind` and size n (torch tensors)."""
+    """Device buffers for one causal set of `kind` and size n (torch tensors).
 
-    def __init__(self, kind, n, device="cuda", path=PATH_AUTO):
+    matrix=False: without the causal matrix, for a product order that is counted from its coordinates only (bits is None)."""
+
+    def __init__(self, kind, n, device="cuda", path=PATH_AUTO, matrix=True):
         import torch
         self.kind, self.n, self.path = kind, n, path
         self.dim = dim(kind)
         self.rw = row_words(n)
         self.coords = torch.empty((self.dim, n), dtype=torch.int32, device=device)
-        self.bits = torch.empty((n, self.rw), dtype=torch.int64, device=device)
+        self.bits = torch.empty((n, self.rw), dtype=torch.int64, device=device) if matrix else None
         self.hist = torch.empty(hist_len(n), dtype=torch.int64, device=device)
         # AUTO counts a 1+1 product order from its coordinates
         self.by_coords = path == PATH_AUTO and coords_abundance_workspace(kind, n) > 0
-        ws = max(sprinkle_workspace_bytes(kind, n), interval_abundance_workspace(n, path), action_workspace_bytes(),
+        ws = max(sprinkle_workspace_bytes(kind, n), interval_abundance_workspace(n, path) if matrix else 0,
+                 action_workspace_bytes(),
                  coords_abundance_workspace(kind, n) if self.by_coords else 0)
         self.workspace = torch.empty(ws, dtype=torch.uint8, device=device)
         self.actions = torch.empty(16, dtype=torch.float64, device=device)

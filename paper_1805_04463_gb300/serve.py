@@ -14,8 +14,10 @@ requests (n^2/8 bytes each), by their tensor-core operand memory, and by a
 slot count.
 
 With path AUTO a product order (a random 2D order, a 1+1 diamond or square) is
-counted whole from its coordinates behind its sprinkle, without operands or
-ticks: that takes less than the bookkeeping of its slices would.
+counted whole from its coordinates behind its sprinkle, without a causal matrix,
+operands or ticks, on a stream of its own: that takes less than the bookkeeping of its
+slices would, and the preparation of other requests does not wait for it.  It is
+charged its workspace (n^2/256 bytes) instead of a bitset.
 
 Counts are integer additions, so a request's histogram and actions are
 identical whether it runs alone or in the mix (tests/test_gpu_serve.py).
@@ -122,6 +124,7 @@ class Server:
         self.ticks_in_flight = ticks_in_flight
         self.max_jobs = max_jobs
         self.prep_stream = torch.cuda.Stream(device=device)
+        self.order_stream = torch.cuda.Stream(device=device)
         self.count_stream = torch.cuda.Stream(device=device)
         tb = cs.lib().cs_count_jobs_table_bytes(max_jobs, self.count_path)
         wb = cs.lib().cs_count_jobs_workspace_bytes(max_jobs, self.count_path)
@@ -132,9 +135,11 @@ class Server:
 
     # -- per request ------------------------------------------------------
     def _admit_coords(self, r):
-        """A product order: sprinkled and counted whole on the preparation stream (0.1 to 1.3 ms up to
-        2^16 elements, less than its share of one tick), no causal matrix and no items left to grant."""
-        torch, st = self.torch, self.prep_stream
+        """A product order: sprinkled and counted whole on its own stream (0.1 to 1.3 ms up to
+        2^16 elements, less than its share of one tick, and more while a tick holds the SMs), no causal
+        matrix and no items left to grant."""
+        torch, st = self.torch, self.order_stream
+        r.buf = cs.Buffers(r.kind, r.n, device=self.device, matrix=False)
         with torch.cuda.stream(st):
             cs.sprinkle(r.kind, r.n, r.seed, r.buf.coords, r.buf.workspace, st)
             cs.coords_abundance(r.kind, r.n, r.buf.coords, r.buf.hist, r.buf.workspace, st)
@@ -143,13 +148,10 @@ class Server:
     def _admit(self, r, now):
         torch = self.torch
         r.state, r.t_admit = "prep", now
-        r.buf = cs.allocate(r.kind, r.n, device=self.device, path=cs.PATH_POPC)
         if r.by_coords:
-            need = cs.coords_abundance_workspace(r.kind, r.n)
-            if r.buf.workspace.numel() < need:
-                r.buf.workspace = torch.empty(need, dtype=torch.uint8, device=self.device)
             self._admit_coords(r)
             return
+        r.buf = cs.allocate(r.kind, r.n, device=self.device, path=cs.PATH_POPC)
         r.total_items = cs.count_items(r.n, self.count_path)
         with torch.cuda.stream(self.prep_stream):
             st = self.prep_stream
@@ -165,7 +167,7 @@ class Server:
             r.prep_event.record(st)
 
     def _finish(self, r, st=None):
-        """Queue actions and the copies home behind the request's last slice (or, on the preparation
+        """Queue actions and the copies home behind the request's last slice (or, on the product orders'
         stream, its whole count)."""
         torch = self.torch
         st = st or self.count_stream
@@ -207,8 +209,9 @@ class Server:
         torch = self.torch
         reqs = [Request(i, k, n, sd, t) for i, (t, k, n, sd) in enumerate(requests)]
         for r in reqs:
-            r.bitset_bytes = cs.bitset_bytes(r.n)
-            r.by_coords = self.by_coords and cs.coords_abundance_workspace(r.kind, r.n) > 0
+            table = cs.coords_abundance_workspace(r.kind, r.n) if self.by_coords else 0
+            r.by_coords = table > 0
+            r.bitset_bytes = table or cs.bitset_bytes(r.n)
             r.operand_bytes = cs.operands_bytes(r.n, self.count_path) if self.tensor and not r.by_coords else 0
         queue = collections.deque(sorted(reqs, key=lambda r: (r.t_arrival, r.rid)))
         active = []
