@@ -375,11 +375,14 @@ class Buffers:
         self.coords = torch.empty((self.dim, n), dtype=torch.int32, device=device)
         self.bits = torch.empty((n, self.rw), dtype=torch.int64, device=device) if matrix else None
         self.hist = torch.empty(hist_len(n), dtype=torch.int64, device=device)
-        # AUTO counts a 1+1 product order from its coordinates
-        self.by_coords = path == PATH_AUTO and coords_abundance_workspace(kind, n) > 0
+        # AUTO counts a 1+1 product order from its coordinates, where their table fits
+        # beside the bitset within the AUTO memory limit
+        table = coords_abundance_workspace(kind, n)
+        self.by_coords = (path == PATH_AUTO and table > 0 and
+                          (not matrix or bitset_bytes(n) + table <= get_auto_memory_limit()))
         ws = max(sprinkle_workspace_bytes(kind, n), interval_abundance_workspace(n, path) if matrix else 0,
                  action_workspace_bytes(),
-                 coords_abundance_workspace(kind, n) if self.by_coords else 0)
+                 table if self.by_coords else 0)
         self.workspace = torch.empty(ws, dtype=torch.uint8, device=device)
         self.actions = torch.empty(16, dtype=torch.float64, device=device)
         self.bracket = torch.empty(1, dtype=torch.int64, device=device)

@@ -1,0 +1,26 @@
+"""What Buffers plans on PATH_AUTO (no GPU: buffers on the meta device)."""
+import pytest
+
+
+@pytest.fixture
+def cs():
+    from paper_1805_04463_gb300 import build
+    build.build()
+    import paper_1805_04463_gb300 as m
+    yield m
+    m.set_auto_memory_limit(0)
+
+
+@pytest.mark.parametrize("kind", [0, 1, 5])
+def test_a_product_order_keeps_to_the_memory_limit(cs, kind):
+    """The count from coordinates takes n^2/256 bytes: only where they fit beside the bitset."""
+    n = 1 << 16
+    table = cs.coords_abundance_workspace(kind, n)
+    small = max(cs.sprinkle_workspace_bytes(kind, n), cs.action_workspace_bytes())
+    assert small < table
+    for limit, by_coords in ((cs.bitset_bytes(n) + table, True), (cs.bitset_bytes(n) + table - 1, False),
+                             (cs.bitset_bytes(n) + small, False)):
+        cs.set_auto_memory_limit(limit)
+        buf = cs.Buffers(kind, n, device="meta")
+        assert buf.by_coords == by_coords
+        assert buf.bits.numel() * 8 + buf.workspace.numel() <= limit
