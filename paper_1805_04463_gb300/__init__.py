@@ -397,7 +397,7 @@ def run(buf: Buffers, seed: int, eps=(0.0,), stream=None, sprinkle_=True):
     if sprinkle_:
         sprinkle(buf.kind, buf.n, seed, buf.coords, buf.workspace, stream)
     causal_matrix(buf.kind, buf.n, buf.coords, buf.bits, stream)
-    if buf.by_coords:
+    if buf.by_coords and buf.path == PATH_AUTO:  # the path may have been set since
         coords_abundance(buf.kind, buf.n, buf.coords, buf.hist, buf.workspace, stream)
     else:
         interval_abundance(buf.n, buf.bits, buf.hist, buf.path, buf.workspace, stream)

@@ -24,3 +24,20 @@ def test_a_product_order_keeps_to_the_memory_limit(cs, kind):
         buf = cs.Buffers(kind, n, device="meta")
         assert buf.by_coords == by_coords
         assert buf.bits.numel() * 8 + buf.workspace.numel() <= limit
+
+
+@pytest.mark.parametrize("path", [0, 1, 2, 3])
+def test_run_counts_on_the_path_the_buffers_name(cs, monkeypatch, path):
+    """A path set on the buffers after they were planned is the one that counts."""
+    cs.set_auto_memory_limit(1 << 34)
+    buf = cs.Buffers(0, 2000, device="meta")
+    assert buf.by_coords
+    calls = []
+    for name in ("sprinkle", "causal_matrix", "coords_abundance", "interval_abundance", "action_device"):
+        monkeypatch.setattr(cs, name, lambda *a, _n=name, **k: calls.append((_n, a)))
+    buf.path = path
+    cs.run(buf, 1)
+    assert [c for c, _ in calls] == ["sprinkle", "causal_matrix",
+                                     "interval_abundance" if path else "coords_abundance", "action_device"]
+    if path:
+        assert calls[2][1][3] == path
