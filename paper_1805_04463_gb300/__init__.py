@@ -377,9 +377,8 @@ class Buffers:
         self.hist = torch.empty(hist_len(n), dtype=torch.int64, device=device)
         # AUTO counts a 1+1 product order from its coordinates, where their table fits
         # beside the bitset within the AUTO memory limit
-        table = coords_abundance_workspace(kind, n)
-        self.by_coords = (path == PATH_AUTO and table > 0 and
-                          (not matrix or bitset_bytes(n) + table <= get_auto_memory_limit()))
+        table = coords_abundance_workspace(kind, n) if path == PATH_AUTO else 0
+        self.by_coords = table > 0 and (not matrix or bitset_bytes(n) + table <= get_auto_memory_limit())
         ws = max(sprinkle_workspace_bytes(kind, n), interval_abundance_workspace(n, path) if matrix else 0,
                  action_workspace_bytes(),
                  table if self.by_coords else 0)

@@ -546,6 +546,9 @@ Layout batch_layout(const cs_set_desc* sets, int n_sets, int path, bool auto_pat
     }
     L.coef = take(size_t(nmax[0] + nmax[1] + nmax[2]) * kMaxEps * sizeof(dd));  // coefficient tables
     L.kends = take(size_t(n_sets) * kMaxEps * 8);                                 // smeared-sum cutoffs
+    for (auto* v : {&L.coords, &L.bits, &L.key0, &L.key1, &L.raw, &L.ctab, &L.op0, &L.op1, &L.ord_p, &L.ord_q, &L.ord_r,
+                    &L.ord_d})
+        v->reserve(size_t(n_sets));
     for (int s = 0; s < n_sets; ++s) {
         const int64_t n = sets[s].n;
         const int dim = cs_dim(sets[s].kind);
@@ -660,6 +663,7 @@ int cs_batch_create(const cs_set_desc* sets, int n_sets, int path, void* workspa
         hoff += cs_hist_len(b.n);
         n_largest = b.n > n_largest ? b.n : n_largest;
     }
+    auto rblocks_end = [&](int s) { return s + 1 < n_sets ? bs[s + 1].rblock_begin : rblk; };
     // Count tables in decreasing set size (the largest sets' tiles go first).
     std::vector<int> order(static_cast<size_t>(n_sets));
     std::iota(order.begin(), order.end(), 0);
@@ -673,8 +677,7 @@ int cs_batch_create(const cs_set_desc* sets, int n_sets, int path, void* workspa
         std::fill(mtab.begin() + bs[s].mblock_begin, mtab.begin() + bs[s].mblock_begin + bs[s].mir_side * bs[s].mir_side,
                   int32_t(s));
     for (int s = 0; s < n_sets; ++s)
-        std::fill(rtab.begin() + bs[s].rblock_begin, rtab.begin() + bs[s].rblock_begin + chunks_before(bs[s].vwords, bs[s].vwords),
-                  int32_t(s));
+        std::fill(rtab.begin() + bs[s].rblock_begin, rtab.begin() + rblocks_end(s), int32_t(s));
     // the relate blocks grouped by geometry, so that each geometry's launch
     // covers only its own blocks (blocks of the other geometries returning at
     // once had cost their dispatch)
@@ -685,7 +688,7 @@ int cs_batch_create(const cs_set_desc* sets, int n_sets, int path, void* workspa
         geo_begin[g] = int64_t(rorder.size());
         for (int s = 0; s < n_sets; ++s)
             if (batch_geom(bs[s].kind) == g)
-                for (int64_t k = 0; k < chunks_before(bs[s].vwords, bs[s].vwords); ++k) rorder.push_back(int32_t(bs[s].rblock_begin + k));
+                for (int64_t k = bs[s].rblock_begin, end = rblocks_end(s); k < end; ++k) rorder.push_back(int32_t(k));
         geo_count[g] = int64_t(rorder.size()) - geo_begin[g];
     }
     std::vector<PopcSetEntry> pe;
