@@ -162,6 +162,17 @@ __global__ void k_scan_add(int64_t* __restrict__ out, int64_t n, const int64_t* 
         out[r] += totals[r / kScanBlock];
 }
 
+// v plus the value of the lane o below, where there is one (the shuffle's own predicate).
+__device__ __forceinline__ int add_from_below(int v, int o) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .s32 t;\n\t"
+        "shfl.sync.up.b32 t|p, %0, %1, 0, 0xffffffff;\n\t"
+        "@p add.s32 %0, %0, t;\n\t}"
+        : "+r"(v)
+        : "r"(o));
+    return v;
+}
+
 // Column indices of each row's relations on one side, in increasing order,
 // at cols[offsets[i] ..).  A row whose list would end past cols_capacity is
 // skipped and CS_ENOMEM recorded.  The warp walks its row 32 words at a
@@ -181,7 +192,8 @@ __global__ void k_scan_add(int64_t* __restrict__ out, int64_t n, const int64_t* 
 //     354 us and of a 2D order 543, with 1024 341 and 539 (first way alone 337 and 569); a
 //     diamond's, a square's, a 3+1 one's are alike from 640 to 1280.
 // The choice needs the step's total, by one reduction beside the scan rather than
-// behind it (behind: lists of a slab of 45000 277.9 us, so 276.0, without the second way 274.5).
+// behind it, and the scan adds by the shuffle's predicate: past list of a slab of 45000 with the
+// total behind the scan 281 us, beside it 279.6, so 278.4 (without the second way 276.8).
 // Future list of a 1+1 diamond, n = 30011: 398 -> 205 us (4.4 TB/s).
 constexpr int kColsWarps = 4;                      // warps per block
 constexpr int kColsRun = 32 * 64 + 4;              // the most columns one step emits, and an alignment shift
@@ -215,10 +227,7 @@ __global__ void __launch_bounds__(kColsWarps * 32) k_side_columns(const uint64_t
             const int total = int(__reduce_add_sync(0xffffffffu, unsigned(c)));
             int incl = c;
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int t = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += t;
-            }
+            for (int o = 1; o < 32; o <<= 1) incl = add_from_below(incl, o);
             // element k of the run goes to cols[pos + k] and to run[s0 + k],
             // s0 = that position's 4-byte slot in its 16-byte group, so the
             // run's 16-byte groups are the output's
