@@ -164,6 +164,8 @@ int cs_resolved_path(int64_t n, int path);
 /* The device memory, in bytes, that CS_PATH_AUTO may plan a set's bitset and
  * count workspace into (process-wide).  0 (the default) means 90% of the
  * current device's memory.  Set it lower when other work shares the GPU.
+ * A product order that cs_evaluate or cs_batch_* counts from its coordinates
+ * has no bitset; its table takes n^2 / 256 bytes, a thirty-second of one.
  * Returns CS_OK. */
 int cs_set_auto_memory_limit(size_t bytes);
 
@@ -175,7 +177,10 @@ size_t cs_get_auto_memory_limit(void);
  * (CS_PATH_POPC, CS_PATH_MMA or CS_PATH_MMA4) for n_min[e] <= n < n_min[e+1].
  * n_min must start at 0 and increase; at most 16 entries.  The default is
  * {0: MMA, 2048: MMA4}; the autotuner
- * (paper_1805_04463_gb300/tune.py) installs measured thresholds.
+ * (paper_1805_04463_gb300/tune.py) installs measured thresholds.  The table is
+ * for counts of a causal matrix: the product orders that cs_evaluate and
+ * cs_batch_* count from their coordinates on CS_PATH_AUTO (cs_coords_abundance)
+ * do not consult it; an explicit path does away with that route.
  * Errors: CS_EINVAL.
  */
 int cs_set_auto_paths(const int64_t *n_min, const int *paths, int count);
@@ -207,7 +212,10 @@ int cs_get_auto_tiles(int64_t *n_min, int *raster, int capacity);
  * tensor path on a device without tcgen05 also falls back to POPC);
  * max_run (1..64, default 16) is the longest run of consecutive work items
  * one CTA (pair) takes from the shared queue, so that a small set is counted
- * by few CTAs.  Results do not depend on either.  Errors: CS_EINVAL.
+ * by few CTAs.  Results do not depend on either.  A batch planned on
+ * CS_PATH_AUTO counts its product orders from their coordinates whatever `path` is
+ * (see cs_coords_abundance); a batch planned on an explicit path does not.
+ * Errors: CS_EINVAL.
  */
 int cs_set_batch_tuning(int path, int max_run);
 
@@ -356,9 +364,9 @@ size_t cs_action_workspace_bytes(void);
  * The same actions evaluated on the device, for n_eps values of eps at once
  * (eps_host is read at call time): out_dev[e] receives S for eps_host[e] and
  * *bracket_dev (may be NULL) the local bracket.  Asynchronous on `stream`;
- * hist_dev is the device histogram written by cs_interval_abundance.  The
- * smeared sums are split over 128 blocks whose double-double partial sums
- * go to the workspace.  Both action entry points stop each smeared sum at
+ * hist_dev is the device histogram written by cs_interval_abundance (any
+ * int64 counts, taken whole).  The smeared sums are split over up to 128 blocks
+ * per eps, whose double-double partial sums go to the workspace.  Both action entry points stop each smeared sum at
  * the first k past which the remaining terms provably move S by less than
  * 1e-15 (bounding the abundances' sum by n(n-1)/2 here, by the histogram's
  * own sum in cs_action).

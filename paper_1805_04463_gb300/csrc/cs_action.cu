@@ -33,9 +33,9 @@ __host__ __device__ inline int act_blocks(int64_t kend, int T) {
 // depend on k comes from the host, and the sum is a shuffle tree.  256
 // threads per block walking the eps values one after another took 102 us
 // for n = 1024 .. 16384 and three smeared eps, squared powers per thread 19,
-// powers from the host in one chain and the polynomial formed per term 16.8;
-// this takes 10.8 (a whole pass over a 2D order of 1024, with the final
-// kernel's launch hidden behind it: 72 -> 63.5 us).
+// powers from the host in one chain and the polynomial's products in eps all formed per
+// term 16.8; this takes 11.4 (3+1 n = 16384: 13.0; with the final
+// kernel's launch hidden behind it, a whole pass over a 2D order of 1024 lost 7 of 72 us).
 struct ActPowers {
     EpsPowers e[kMaxEps];
     SmearCoef c[kMaxEps];

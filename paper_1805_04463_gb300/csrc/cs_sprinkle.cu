@@ -205,7 +205,7 @@ __global__ void __launch_bounds__(kThreads) k_rank_scatter(int64_t n, int dim, b
 }
 
 // A whole small set in one CTA: draws, ranks in shared memory, coordinates
-// out; no scratch in the workspace.  Five launches of a handful of blocks
+// out; no scratch in the workspace.  Four launches of a handful of blocks
 // are all latency there.
 template <int KIND>
 __global__ void __launch_bounds__(kRankThreads) k_sprinkle_small(int n, int lgP, uint64_t seed,
