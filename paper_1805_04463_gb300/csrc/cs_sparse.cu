@@ -187,17 +187,17 @@ __device__ __forceinline__ int add_from_below(int v, int o) {
 //     where half of the bits are set);
 //   many: word after word (read by broadcast), lane l placing bits l and l + 32 by
 //     their rank within the word: consecutive places, one pass per store and
-//     the same cost whatever is set.  From 1024 relations a step on, where no
-//     kind measured loses by it: with a limit of 640 the past lists of a cylinder of 45000 took
-//     354 us and of a 2D order 543, with 1024 341 and 539 (first way alone 337 and 569); a
-//     diamond's, a square's, a 3+1 one's are alike from 640 to 1280.
-// The choice needs the step's total, by one reduction beside the scan rather than
-// behind it, and the scan adds by the shuffle's predicate: past list of a slab of 45000 with the
-// total behind the scan 281 us, beside it 279.6, so 278.4 (without the second way 276.8).
+//     the same cost whatever is set.  Where 16 of the 32 words hold 36 columns or more, so
+//     that no kind measured loses by it: from 640 relations a step the past lists of a cylinder of
+//     45000 took 354 us and of a 2D order 543, from 1024 on 341 and 539 (first way alone 337 and
+//     569); a diamond's, a square's, a 3+1 one's are alike from 640 to 1280.
+// The choice is one ballot beside the scan, which adds by the shuffle's predicate (by the
+// step's total: columns of a slab of 45000 218.1 us behind the scan, 217.0 by a reduction
+// beside it, so 216.1; without the second way 215.0).
 // Future list of a 1+1 diamond, n = 30011: 398 -> 205 us (4.4 TB/s).
 constexpr int kColsWarps = 4;                      // warps per block
 constexpr int kColsRun = 32 * 64 + 4;              // the most columns one step emits, and an alignment shift
-constexpr int kManyColumns = 1024;                 // columns of a step from which they are placed word after word
+constexpr int kFullWord = 36, kFullWords = 16;      // a step of that many words of that many columns is placed word after word
 __global__ void __launch_bounds__(kColsWarps * 32) k_side_columns(const uint64_t* __restrict__ bits, int64_t n,
                                                                    int64_t row_words, bool future,
                                                                    const int64_t* __restrict__ offsets,
@@ -224,16 +224,17 @@ __global__ void __launch_bounds__(kColsWarps * 32) k_side_columns(const uint64_t
             uint64_t x = w < whi ? xn & side_mask(i, w, future) : 0ull;
             xn = w + 32 < whi ? __ldg(row + w + 32) : 0ull;
             const int c = __popcll(x);
-            const int total = int(__reduce_add_sync(0xffffffffu, unsigned(c)));
+            const bool dense = __popc(__ballot_sync(0xffffffffu, c >= kFullWord)) >= kFullWords;
             int incl = c;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) incl = add_from_below(incl, o);
+            const int total = __shfl_sync(0xffffffffu, incl, 31);
             // element k of the run goes to cols[pos + k] and to run[s0 + k],
             // s0 = that position's 4-byte slot in its 16-byte group, so the
             // run's 16-byte groups are the output's
             const int s0 = int((reinterpret_cast<uintptr_t>(cols + pos) >> 2) & 3);
             int at = s0 + incl - c;
-            if (total >= kManyColumns) {  // warp-uniform
+            if (dense) {  // warp-uniform
                 words[warp][lane] =
                     make_int4(int(uint32_t(x)), int(uint32_t(x >> 32)), at, at + __popc(uint32_t(x)));
                 __syncwarp();
