@@ -379,6 +379,8 @@ class Buffers:
         # beside the bitset within the AUTO memory limit
         table = coords_abundance_workspace(kind, n) if path == PATH_AUTO else 0
         self.by_coords = table > 0 and (not matrix or bitset_bytes(n) + table <= get_auto_memory_limit())
+        if not matrix and not self.by_coords:
+            raise ValueError("matrix=False is for product orders on PATH_AUTO")
         ws = max(sprinkle_workspace_bytes(kind, n), interval_abundance_workspace(n, path) if matrix else 0,
                  action_workspace_bytes(),
                  table if self.by_coords else 0)

@@ -41,3 +41,12 @@ def test_run_counts_on_the_path_the_buffers_name(cs, monkeypatch, path):
                                      "interval_abundance" if path else "coords_abundance", "action_device"]
     if path:
         assert calls[2][1][3] == path
+
+
+def test_buffers_without_a_matrix_are_for_product_orders(cs):
+    cs.set_auto_memory_limit(1)  # no bitset, nothing to fit beside it
+    buf = cs.Buffers(1, 3000, device="meta", matrix=False)
+    assert buf.by_coords and buf.bits is None and buf.workspace.numel() < cs.bitset_bytes(3000)
+    for kind, path in ((2, 0), (4, 0), (1, 3)):
+        with pytest.raises(ValueError):
+            cs.Buffers(kind, 3000, device="meta", path=path, matrix=False)
